@@ -30,8 +30,12 @@
  *    computed in FP64 once per point.  Fletcher-Powell A, B, E are always
  *    double.
  *  - csize (the chunk size) must be one of 1, 2, 4, 8, 16, 32, or 0 for
- *    "choose for me" (the autotuned table entry for (function, n, precision)
- *    if one exists, else a default).  It need not divide n: the last chunk is
+ *    "choose for me".  A call that names neither a chunk size nor a method
+ *    (csize 0, no configuration or one of zeros) gets the structured
+ *    evaluation: the same hDual rules on the components the seeds make
+ *    nonzero, with the dense method's results for finite and non-finite
+ *    inputs (to rounding).  Naming a chunk size or a method runs the dense
+ *    chunked algorithm with it.  csize need not divide n: the last chunk is
  *    ragged and its positions beyond n are never seeded.
  *  - 1 <= n <= CHESSFAD_MAX_N.  batch == 0 is a valid no-op; batch < 0 is an
  *    error.  NaN and Inf inputs propagate; they are not trapped.  The
@@ -131,7 +135,8 @@ typedef struct {
  *   threads_per_point symmetric method: threads sharing one point's
  *                     (row, chunk) items, 8..256 power of two (below 32 a
  *                     warp serves several points)
- * Zero in any field means "default".  With csize 0, method 0 means the
+ * Zero in any field means "default"; zero in every field is the structured
+ * evaluation (see conventions).  Else, with csize 0, method 0 means the
  * default method (the tuned one, else chessfad_default_config's), not
  * necessarily the plain method, and the chunk size follows the method: the
  * tuned or default configuration's for that method, else the Sec. V optimum
@@ -207,11 +212,12 @@ CHESSFAD_API int chessfad_hvp_host(int fn, int n, long long batch, int csize, co
                                    const void *v_host, void *out_host, void *x_dev, void *v_dev, void *out_dev,
                                    const chessfad_fp_params *params, int prec, int slices, chessfad_stream_t stream);
 
-/* The configuration chessfad_hvp would use for csize = 0: the tuned entry if
- * present, else the default (n >= 4: the symmetric method at the Sec. V
+/* The default configuration of the dense chunked evaluation: the tuned entry
+ * if present, else (n >= 4: the symmetric method at the Sec. V
  * optimum csize = sqrt(n/2) rounded up to a power of two; n < 4: the plain
  * method).  A call with csize != 0 and no configuration uses the plain method
- * with that chunk size.  Host only; launches nothing. */
+ * with that chunk size; a call with csize 0 and no configuration needs none
+ * (the structured evaluation).  Host only; launches nothing. */
 CHESSFAD_API int chessfad_default_config(int fn, int n, long long batch, int prec, chessfad_config *cfg);
 
 /* The configuration chessfad_hvp_config (hvp != 0) or
@@ -228,8 +234,9 @@ CHESSFAD_API int chessfad_resolve_config(int fn, int n, long long batch, int pre
  * block_threads) and the symmetric method over (threads_per_point 8..256,
  * block_threads), discarding chunk sizes whose kernels spill registers.  The
  * seed-sparse and one-thread-per-point methods are never candidates.  The
- * winner is stored in the process-wide table used by
- * csize = 0 (chessfad_hvp) and returned in *best (may be NULL).
+ * winner, the fastest dense configuration, is stored in the process-wide
+ * table that configurations with csize 0 are completed from
+ * (chessfad_resolve_config) and returned in *best (may be NULL).
  * Synchronises `stream`.  Allocates no device memory. */
 CHESSFAD_API int chessfad_autotune_hvp(int fn, int n, long long batch, const void *x, const void *v, void *out,
                           const chessfad_fp_params *params, int prec, chessfad_stream_t stream,
@@ -238,8 +245,9 @@ CHESSFAD_API int chessfad_autotune_hvp(int fn, int n, long long batch, const voi
 /* Autotune the Hessian launch configuration for (fn, n, prec) as
  * chessfad_autotune_hvp does for the HVP (the same candidates, timed as
  * Hessian launches on a prefix of the caller's x and H, which is
- * overwritten).  The winner is stored in the process-wide Hessian table used
- * by chessfad_hessian with csize = 0 and returned in *best (may be NULL).
+ * overwritten).  The winner is stored in the process-wide Hessian table that
+ * configurations with csize 0 are completed from and returned in *best (may
+ * be NULL).
  * Synchronises `stream`; allocates no device memory. */
 CHESSFAD_API int chessfad_autotune_hessian(int fn, int n, long long batch, const void *x, void *H,
                                            const chessfad_fp_params *params, int prec, chessfad_stream_t stream,

@@ -13,6 +13,7 @@
 
 #include "../../include/chessfad.h"
 #include "dispatch.h"
+#include "structured.h"
 
 namespace chessfad {
 
@@ -294,6 +295,41 @@ static int launch(int fn, int n, long long batch, const chessfad_config &c, cons
     return e == cudaSuccess ? CHESSFAD_SUCCESS : CHESSFAD_ERR_CUDA;
 }
 
+// Whether the dense symmetric HVP of n variables at the default chunk size
+// adds its rows in FP64 accumulators (compensated FP32: the staged chunk
+// matrix of a point beyond the 200 KiB budget of launch()) instead of as a
+// Dot2; the structured evaluation returns the same for a v that is not finite.
+static bool dense_rows_in_fp64(int fn, int n, int prec)
+{
+    if (prec == CHESSFAD_FP64 || n < 128) return false;
+    const int mt = fn == CHESSFAD_FLETCHER_POWELL ? fp_tile_rows(n, prec) : 8;
+    return align_up(smem_layout<float>(fn, true, n, 1, mt).total, 16) + sym_hs_bytes<float>(n, sym_chunk(fn, n, prec)) >
+           200 * 1024;
+}
+
+// The library's own choice of evaluation, for calls that name neither a chunk
+// size nor a method: the structured evaluation.
+static int launch_structured(int fn, int n, long long batch, const void *x, const void *v, void *out,
+                             const chessfad_fp_params *params, int prec, cudaStream_t stream)
+{
+    StructArgs a{};
+    a.x = x;
+    a.v = v;
+    a.out = out;
+    if (fn == CHESSFAD_FLETCHER_POWELL) {
+        a.A = params->A;
+        a.B = params->B;
+        a.E = params->E;
+        a.ld = params->ld;
+    }
+    a.batch = batch;
+    a.n = n;
+    a.wide = dense_rows_in_fp64(fn, n, prec);
+    const cudaError_t e = structured_hvp(fn, prec == CHESSFAD_FP64, a, stream);
+    if (e == cudaErrorInvalidConfiguration) return CHESSFAD_ERR_BATCH;
+    return e == cudaSuccess ? CHESSFAD_SUCCESS : CHESSFAD_ERR_CUDA;
+}
+
 static cudaError_t kernel_attr(int fn, int prec, int csize, bool hvp, cudaFuncAttributes *fa)
 {
     if (fn < 0 || fn > 2) return cudaErrorInvalidValue;
@@ -308,6 +344,13 @@ static int run(int fn, int n, long long batch, const chessfad_config *cfg, int c
     if (st) return st;
     if (csize_hint != 0 && !valid_chunk(csize_hint)) return CHESSFAD_ERR_CHUNK;
     if (cfg && cfg->csize != 0 && !valid_chunk(cfg->csize)) return CHESSFAD_ERR_CHUNK;
+    const bool own = csize_hint == 0 && (!cfg || (!cfg->csize && !cfg->threads_per_row && !cfg->block_threads &&
+                                                  !cfg->method && !cfg->threads_per_point));
+    if (hvp && own) {
+        if (batch == 0) return CHESSFAD_SUCCESS;
+        if (!x || !out || !v) return CHESSFAD_ERR_NULL;
+        return launch_structured(fn, n, batch, x, v, out, params, prec, stream);
+    }
     const chessfad_config c = resolve(fn, n, batch, prec, cfg, csize_hint, hvp);
     st = check_config(c);
     if (st) return st;

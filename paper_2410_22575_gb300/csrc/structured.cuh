@@ -1,0 +1,722 @@
+// structured.cuh -- Hessian-vector products and Hessians of the built-in
+// functions by the hDual rules applied to the components that the seeding
+// makes nonzero.
+//
+// The dense sweeps (sweep.cuh) evaluate f once per (row i, chunk) on hDuals
+// in which every variable but x_i and the chunk's has a zero derivative part;
+// almost all of their arithmetic is products with those seed zeros.  Here the
+// rules of hdual.cuh are applied to the nonzero components only, and for a
+// product H v the seed of d1 is the direction v itself: with d1 seeded by v_k
+// instead of [k == i], the h component of variable l is (H v)_l directly, so
+// one pass over a point replaces its n rows.
+//
+//   Rosenbrock       row l holds three entries (two neighbouring terms);
+//                    their products with v are summed as the dense row is.
+//   Ackley           the two sums under sqrt and exp carry
+//                    d1 = sum_k x_k v_k and sum_k phi'(x_k) v_k; the tail's
+//                    unary rules then give each (H v)_l from g and h of its
+//                    own variable.
+//   Fletcher-Powell  residual r_m carries its FP64 value and
+//                    d1_m = -(J v)_m; the squares' rule needs sum_m d1_m g_ml
+//                    and sum_m r_m h_ml, four transposed products with A, B.
+//
+// A product with a seed zero is an exact zero unless its other factor is Inf
+// or NaN, and there the dense method returns NaN.  Points whose result is not
+// finite are therefore evaluated again entry by entry with the dense method's
+// propagation (the *_dense_* functions below), so non-finite inputs and
+// overflow give what the dense sweeps give.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <math_constants.h>
+
+#include "hdual.cuh"
+#include "sweep.cuh"
+
+namespace chessfad {
+
+template <typename T>
+__device__ __forceinline__ bool not_finite(T x)
+{
+    return !(fabs(x) <= (sizeof(T) == 8 ? (T)1.7976931348623157e308 : (T)3.402823466e38f));
+}
+
+__device__ __forceinline__ float nan_of(float) { return CUDART_NAN_F; }
+__device__ __forceinline__ double nan_of(double) { return CUDART_NAN; }
+
+// float -> double through the integer pipe (exact for normal floats; zeros,
+// subnormals, Inf and NaN take the conversion instruction): the conversion
+// instruction runs at the FP64 pipe's rate, 1/64 of FP32's.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    if (((b >> 23) + 1u & 0xffu) > 1u) {  // exponent field 1 .. 254
+        const unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
+        return __hiloint2double((int)hi, (int)(b << 29));
+    }
+    return (double)x;
+}
+
+// The row-times-v sum of the dense sweeps: Dot2 in compensated FP32, FMAs in
+// FP64.
+template <typename T>
+struct RowSum;
+template <>
+struct RowSum<float> {
+    CSum s{0.f, 0.f};
+    __device__ __forceinline__ void add(float a, float b) { cdot_add(s, a, b); }
+    __device__ __forceinline__ float value() const { return csum_value(s); }
+    __device__ __forceinline__ void merge_xor(int off)
+    {
+        CSum o;
+        o.s = __shfl_xor_sync(0xffffffffu, s.s, off);
+        o.e = __shfl_xor_sync(0xffffffffu, s.e, off);
+        s = csum_merge(s, o);
+    }
+};
+template <>
+struct RowSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { s = __fma_rn(a, b, s); }
+    __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ void merge_xor(int off) { s += __shfl_xor_sync(0xffffffffu, s, off); }
+};
+
+// Row s of a point evaluated densely: sum_j entry(s, j) v_j over every j.
+// wide: the dense HVP of this size adds its rows in FP64 (SymStage) instead
+// of as a Dot2.
+template <typename T, typename IO, typename F>
+__device__ __forceinline__ T dense_row(const IO *v, int n, int s, bool wide, F &&entry)
+{
+    if (IsComp<T>::value && wide) {
+        double d = 0.0;
+        for (int j = 0; j < n; ++j) d = fma((double)entry(s, j), (double)v[j], d);
+        return (T)d;
+    }
+    RowSum<T> d;
+    for (int j = 0; j < n; ++j) d.add(entry(s, j), (T)v[j]);
+    return d.value();
+}
+
+// ------------------------------------------------------------------ Rosenbrock
+// Row l of the Hessian from the terms k = l - 1 (as its y_{k+1}: d.d1 = d.g =
+// 1) and k = l (as its y_k: d.d1 = d.g = -2 x_l, d.h = -2), each square by the
+// unary rule; the rounding is the dense sweep's.
+template <typename T>
+struct RosRow {
+    T lo, diag, up;  // entries (l, l-1), (l, l), (l, l+1)
+};
+template <typename T>
+__device__ __forceinline__ RosRow<T> ros_row(T xm, T x0, T xp, int l, int n)
+{
+    RosRow<T> r;
+    r.lo = T(0);
+    r.diag = T(0);
+    r.up = T(0);
+    if (l > 0) {
+        r.lo = T(200) * (T(-2) * xm);
+        r.diag = T(200);
+    }
+    if (l < n - 1) {
+        const T g = T(-2) * x0;
+        const T dv = fma_(T(-1), x0 * x0, xp);
+        r.up = T(200) * g;
+        r.diag = fma_(r.up, g, r.diag);
+        r.diag = fma_(T(200) * dv, T(-2), r.diag);
+        r.diag = r.diag + T(2);
+    }
+    return r;
+}
+
+// What non-finite terms do to the dense entries.  A term whose x_k is not
+// finite multiplies seed zeros of every component: every entry is NaN.  A
+// term whose residual 200 d overflows (x_k finite) multiplies only second
+// derivatives, zero except at (k, k): every other entry is NaN.
+struct RosBad {
+    int count, at;  // residual-overflow terms, the last one's index
+    bool all;
+};
+template <typename T, typename IO>
+__device__ __forceinline__ RosBad ros_bad(const IO *x, int n)
+{
+    RosBad b{0, -1, false};
+    for (int k = 0; k + 1 < n; ++k) {
+        const T x0 = (T)x[k], dv = fma_(T(-1), x0 * x0, (T)x[k + 1]);
+        if (not_finite(x0)) b.all = true;
+        else if (not_finite(T(200) * dv)) {
+            ++b.count;
+            b.at = k;
+        }
+    }
+    return b;
+}
+template <typename T, typename IO>
+__device__ __forceinline__ T ros_dense_entry(const IO *x, int n, const RosBad &b, int i, int j)
+{
+    if (b.all || (b.count > 0 && !(b.count == 1 && i == j && b.at == i))) return nan_of(T(0));
+    if (i - j > 1 || j - i > 1) return T(0);
+    const RosRow<T> r = ros_row<T>(i > 0 ? (T)x[i - 1] : T(0), (T)x[i], i + 1 < n ? (T)x[i + 1] : T(0), i, n);
+    return j < i ? r.lo : j == i ? r.diag : r.up;
+}
+template <typename T, typename IO>
+__device__ __noinline__ void ros_dense_hvp(const IO *x, const IO *v, IO *out, int n, int t, int G, bool wide)
+{
+    const RosBad b = ros_bad<T>(x, n);
+    for (int s = t; s < n; s += G)
+        out[s] = (IO)dense_row<T>(v, n, s, wide, [&](int i, int j) { return ros_dense_entry<T>(x, n, b, i, j); });
+}
+
+// H v of one point by the G lanes t = 0 .. G-1 of an aligned group of its
+// warp (every lane of the warp calls it; idle groups pass active = false).
+template <typename T, typename IO>
+__device__ __forceinline__ void ros_point(const IO *__restrict__ x, const IO *__restrict__ v, IO *__restrict__ out,
+                                          int n, int t, int G, bool active, bool wide)
+{
+    bool bad = false;
+    if (active) {
+#pragma unroll 4
+        for (int l = t; l < n; l += G) {
+            const bool lo = l > 0, hi = l < n - 1;
+            const T xm = lo ? (T)x[l - 1] : T(0), x0 = (T)x[l], xp = hi ? (T)x[l + 1] : T(0);
+            const T vm = lo ? (T)v[l - 1] : T(0), v0 = (T)v[l], vp = hi ? (T)v[l + 1] : T(0);
+            const RosRow<T> r = ros_row<T>(xm, x0, xp, l, n);
+            RowSum<T> d;
+            d.add(r.lo, vm);
+            d.add(r.diag, v0);
+            d.add(r.up, vp);
+            const T o = d.value();
+            bad |= not_finite(o);
+            out[l] = (IO)o;
+        }
+    }
+    // a not finite x, v or residual makes its own row's product not finite
+    const unsigned votes = __ballot_sync(0xffffffffu, bad);
+    const unsigned mask = (G == 32 ? 0xffffffffu : ((1u << G) - 1u)) << ((threadIdx.x & 31) - t);
+    if (votes & mask) {
+        __syncwarp(mask);
+        ros_dense_hvp<T>(x, v, out, n, t, G, wide);
+    }
+}
+
+// ------------------------------------------------------------------ Ackley
+template <typename T>
+__device__ __forceinline__ void sincos_2pi(T x, T &s, T &c);
+template <>
+__device__ __forceinline__ void sincos_2pi<float>(float x, float &s, float &c) { sincospif(2.0f * x, &s, &c); }
+template <>
+__device__ __forceinline__ void sincos_2pi<double>(double x, double &s, double &c) { sincospi(2.0 * x, &s, &c); }
+
+// The tail's derivative factors of one point, from S = sum x^2 and
+// C = sum cos 2 pi x (both FP64): r = sqrt(S/n) as a function of S/2,
+// -20 exp(-0.2 r) as a function of r, -exp(C/n) as a function of C.
+template <typename T>
+struct AckTail {
+    T r1, r2;  // r', r''
+    T p1, p2;  // of -20 exp(-0.2 r)
+    T q1, q2;  // of -exp(C/n)
+};
+// The scalar functions in FP64, or, for compensated FP32, in FP32 from the
+// correctly rounded FP64 sums.
+__device__ __forceinline__ AckTail<double> ack_tail(double S, double C, double inv_n, double)
+{
+    AckTail<double> k;
+    const double a0 = S * inv_n, sq = sqrt(a0), k2 = 2.0 * inv_n;
+    const double e1 = exp(-0.2 * sq), e2 = exp(C * inv_n);
+    k.r1 = k2 * (0.5 / sq);
+    k.r2 = (k2 * k2) * (-0.25 / (sq * a0));
+    k.p1 = 4.0 * e1;
+    k.p2 = -0.8 * e1;
+    k.q1 = -inv_n * e2;
+    k.q2 = -(inv_n * inv_n) * e2;
+    return k;
+}
+__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, double inv_n, float)
+{
+    AckTail<float> k;
+    const float a0 = (float)(S * inv_n), sq = sqrtf(a0), in = (float)inv_n, k2 = 2.0f * in;
+    const float e1 = expf(-0.2f * sq), e2 = expf((float)(C * inv_n));
+    k.r1 = k2 * (0.5f / sq);
+    k.r2 = (k2 * k2) * (-0.25f / (sq * a0));
+    k.p1 = 4.0f * e1;
+    k.p2 = -0.8f * e1;
+    k.q1 = -in * e2;
+    k.q2 = -(in * in) * e2;
+    return k;
+}
+
+// One variable's h component of the whole tail: S/2 carries (d1 = sd, g = x,
+// h = sh), C carries (d1 = cd, g = cg, h = ch).
+template <typename T>
+__device__ __forceinline__ T ack_tail_h(const AckTail<T> &k, T sd, T x, T sh, T cd, T cg, T ch)
+{
+    HD<T, 1> a, b;
+    a.v = b.v = T(0);
+    a.d1 = sd;
+    a.g[0] = x;
+    a.h[0] = sh;
+    b.d1 = cd;
+    b.g[0] = cg;
+    b.h[0] = ch;
+    const HD<T, 1> r = unary(a, T(0), k.r1, k.r2);
+    HD<T, 1> f = unary(r, T(0), k.p1, k.p2);
+    add_unary<false>(f, b, T(0), k.q1, k.q2);
+    return f.h[0];
+}
+
+// A point evaluated as the dense sweeps propagate non-finite values: a not
+// finite x_k multiplies seed zeros in S of every component.
+template <typename T, typename IO>
+struct AckDense {
+    const IO *x;
+    bool poison;
+    AckTail<T> k;
+    __device__ __forceinline__ AckDense(const IO *x_, int n) : x(x_), poison(false)
+    {
+        double S = 0.0, C = 0.0;
+        for (int j = 0; j < n; ++j) {
+            T s, c;
+            const T xj = (T)x[j];
+            sincos_2pi<T>(xj, s, c);
+            poison |= not_finite(xj);
+            S = fma((double)xj, (double)xj, S);
+            C += (double)c;
+        }
+        k = ack_tail(S, C, 1.0 / n, T(0));
+    }
+    __device__ __forceinline__ T entry(int i, int j) const
+    {
+        if (poison) return nan_of(T(0));
+        T si, ci, sj, cj;
+        sincos_2pi<T>((T)x[i], si, ci);
+        sincos_2pi<T>((T)x[j], sj, cj);
+        const T m2p = T(-2.0 * CUDART_PI), m4p = T(-4.0 * CUDART_PI * CUDART_PI);
+        return ack_tail_h<T>(k, (T)x[i], (T)x[j], i == j ? T(1) : T(0), m2p * si, m2p * sj, i == j ? m4p * cj : T(0));
+    }
+};
+template <typename T, typename IO>
+__device__ __noinline__ void ack_dense_hvp(const IO *x, const IO *v, IO *out, int n, int t, int G, bool wide)
+{
+    const AckDense<T, IO> d(x, n);
+    for (int s = t; s < n; s += G)
+        out[s] = (IO)dense_row<T>(v, n, s, wide, [&](int i, int j) { return d.entry(i, j); });
+}
+
+// H v of one point by the G lanes of an aligned group of its warp, EPL
+// variables per lane (variable t + G j), n <= G EPL.
+template <typename T, typename IO, int EPL>
+__device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__restrict__ v, IO *__restrict__ out,
+                                          int n, int t, int G, bool active, bool wide, double inv_n)
+{
+    const int m = active ? n : 0;
+    T xs[EPL], vs[EPL], sn[EPL], cs[EPL];
+    double S = 0.0, C = 0.0;
+    RowSum<T> xv, sv;
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) {
+        const int k = t + G * j;
+        xs[j] = T(0);
+        vs[j] = T(0);
+        if (k < m) {
+            xs[j] = (T)x[k];
+            vs[j] = (T)v[k];
+        }
+    }
+    const T m2p = T(-2.0 * CUDART_PI), m4p = T(-4.0 * CUDART_PI * CUDART_PI);
+#pragma unroll
+    for (int j = 0; j < EPL; ++j) {
+        if (G * j < n) {  // uniform in the group
+            sincos_2pi<T>(xs[j], sn[j], cs[j]);
+            if (t + G * j < m) {
+                const double xd = widen(xs[j]);
+                S = fma(xd, xd, S);
+                C += widen(cs[j]);
+                sn[j] = m2p * sn[j];
+                xv.add(xs[j], vs[j]);
+                sv.add(sn[j], vs[j]);
+            }
+        }
+    }
+    for (int off = G >> 1; off > 0; off >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, off);
+        C += __shfl_xor_sync(0xffffffffu, C, off);
+        xv.merge_xor(off);
+        sv.merge_xor(off);
+    }
+    bool bad = false;
+    if (active) {
+        const AckTail<T> k = ack_tail(S, C, inv_n, T(0));
+        const T xd = xv.value(), sd = sv.value();
+#pragma unroll
+        for (int j = 0; j < EPL; ++j) {
+            if (t + G * j < n) {
+                const T o = ack_tail_h<T>(k, xd, xs[j], vs[j], sd, sn[j], (m4p * cs[j]) * vs[j]);
+                bad |= not_finite(o);
+                out[t + G * j] = (IO)o;
+            }
+        }
+    }
+    // a not finite x makes S or C, a not finite v its own row, not finite
+    const unsigned votes = __ballot_sync(0xffffffffu, bad);
+    const unsigned mask = (G == 32 ? 0xffffffffu : ((1u << G) - 1u)) << ((threadIdx.x & 31) - t);
+    if (votes & mask) {
+        __syncwarp(mask);
+        ack_dense_hvp<T>(x, v, out, n, t, G, wide);
+    }
+}
+
+// ------------------------------------------------------------------ Fletcher-Powell
+// A CTA of kFpThreads holds up to kFpPairs (point, variable) pairs, points
+// q < P of sizes n_q packed one after the other (pair base_q + j).
+//   pass 1  r_m = E_m - sum_j (A_mj sin x_j + B_mj cos x_j) in FP64 and
+//           d1_m = -sum_j (A_mj cos x_j - B_mj sin x_j) v_j, for the rows m of
+//           an A/B tile in shared memory, L lanes per (point, row);
+//   pass 2  sum_m A_ml d1_m, B_ml d1_m, A_ml r_m, B_ml r_m of every pair, kept
+//           in registers across the tiles, kFpNpt pairs per thread.
+// In compensated FP32 only the residual is FP64 (2 of the 8 FMAs of an (m, j)
+// pair); the other sums add blocks of plain FP32 FMAs with TwoSum.
+constexpr int kFpThreads = 256;
+constexpr int kFpNpt = 2;
+constexpr int kFpPairs = kFpThreads * kFpNpt;
+constexpr int kFpMaxPts = 128;
+
+struct FpShape {
+    int nmax;  // largest n of the tile's points
+    int mt;    // rows of A, B per shared-memory tile
+    int lanes; // lanes per (point, row) in pass 1, a power of two <= 32
+};
+
+// Shared-memory layout (bytes) of a CTA.
+template <typename T>
+struct FpSmem {
+    size_t zs, zc, ts, tc, r, d, a, b, af, bf, q, base, n, xoff, eoff, total;
+};
+// Row stride of the tiles: odd, so lanes on different rows (pass 1) hit
+// different banks.
+__host__ __device__ inline int fp_stride(int nmax) { return nmax | 1; }
+
+template <typename T>
+__host__ __device__ inline FpSmem<T> fp_smem(int nmax, int mt)
+{
+    FpSmem<T> s{};
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off = align_up(off + bytes, 16);
+        return at;
+    };
+    const size_t tile = (size_t)mt * fp_stride(nmax);
+    s.xoff = take(kFpMaxPts * sizeof(long long));
+    s.eoff = take(kFpMaxPts * sizeof(long long));
+    s.zs = take(kFpPairs * sizeof(double));
+    s.zc = take(kFpPairs * sizeof(double));
+    s.ts = take(kFpPairs * sizeof(T));
+    s.tc = take(kFpPairs * sizeof(T));
+    s.r = take(kFpPairs * sizeof(T));
+    s.d = take(kFpPairs * sizeof(T));
+    s.a = take(tile * sizeof(double));
+    s.b = take(tile * sizeof(double));
+    s.af = s.a;
+    s.bf = s.b;
+    if (sizeof(T) == 4) {
+        s.af = take(tile * sizeof(T));
+        s.bf = take(tile * sizeof(T));
+    }
+    s.n = take(kFpMaxPts * sizeof(int));
+    s.base = take((kFpMaxPts + 1) * sizeof(int));
+    s.q = take(kFpPairs);
+    s.total = off;
+    return s;
+}
+
+// Sums of pass 2 for one pair, and of pass 1 for one (point, row).
+template <typename T, int N>
+struct FpSums;
+template <int N>
+struct FpSums<double, N> {
+    double s[N];
+    __device__ __forceinline__ void init()
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) s[i] = 0.0;
+    }
+    __device__ __forceinline__ void fma_to(int i, double a, double b) { s[i] = __fma_rn(a, b, s[i]); }
+    __device__ __forceinline__ void flush() {}
+    __device__ __forceinline__ double value(int i) const { return s[i]; }
+    __device__ __forceinline__ void merge_xor(int off)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
+    }
+};
+template <int N>
+struct FpSums<float, N> {
+    CSum s[N];
+    float p[N];
+    __device__ __forceinline__ void init()
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            s[i] = CSum{0.f, 0.f};
+            p[i] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void fma_to(int i, float a, float b) { p[i] = __fmaf_rn(a, b, p[i]); }
+    // the block's partial sums enter the compensated pairs
+    __device__ __forceinline__ void flush()
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            csum_add(s[i], p[i]);
+            p[i] = 0.f;
+        }
+    }
+    __device__ __forceinline__ float value(int i) const { return csum_value(s[i]); }
+    __device__ __forceinline__ void merge_xor(int off)
+    {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            CSum o;
+            o.s = __shfl_xor_sync(0xffffffffu, s[i].s, off);
+            o.e = __shfl_xor_sync(0xffffffffu, s[i].e, off);
+            s[i] = csum_merge(s[i], o);
+        }
+    }
+};
+constexpr int kFpBlock = 4;  // (m, j) pairs per FP32 block partial
+
+struct FpArgs {
+    const double *A, *B, *E;
+    int ld;
+};
+
+// One tile of points.  The caller has filled, in shared memory, n[q], base[q]
+// (base[P] = the pair count), xoff[q] and eoff[q], and synchronised.
+// Afterwards sums[i] holds the four pass-2 sums of pair tid + i kFpThreads
+// over the rows m0 <= m < m1.
+template <typename T, typename IO>
+struct FpTile {
+    const FpArgs a;
+    const IO *x, *v;
+    unsigned char *smem;
+    const FpShape sh;
+    const FpSmem<T> L;
+    const int P, npairs;
+    double *zs, *zc, *ta, *tb;
+    T *ts, *tc, *rr, *dd, *fa, *fb;
+    unsigned char *qs;
+    int *ns, *base;
+    long long *xoff, *eoff;
+
+    __device__ __forceinline__ FpTile(const FpArgs &a_, const IO *x_, const IO *v_, unsigned char *sm,
+                                      const FpShape &s, int P_, int npairs_)
+        : a(a_), x(x_), v(v_), smem(sm), sh(s), L(fp_smem<T>(s.nmax, s.mt)), P(P_), npairs(npairs_)
+    {
+        zs = reinterpret_cast<double *>(sm + L.zs);
+        zc = reinterpret_cast<double *>(sm + L.zc);
+        ta = reinterpret_cast<double *>(sm + L.a);
+        tb = reinterpret_cast<double *>(sm + L.b);
+        ts = reinterpret_cast<T *>(sm + L.ts);
+        tc = reinterpret_cast<T *>(sm + L.tc);
+        rr = reinterpret_cast<T *>(sm + L.r);
+        dd = reinterpret_cast<T *>(sm + L.d);
+        fa = reinterpret_cast<T *>(sm + L.af);
+        fb = reinterpret_cast<T *>(sm + L.bf);
+        qs = sm + L.q;
+        ns = reinterpret_cast<int *>(sm + L.n);
+        base = reinterpret_cast<int *>(sm + L.base);
+        xoff = reinterpret_cast<long long *>(sm + L.xoff);
+        eoff = reinterpret_cast<long long *>(sm + L.eoff);
+    }
+
+    // sin, cos (FP64) and their products with v of every pair
+    __device__ __forceinline__ void stage()
+    {
+        for (int u = threadIdx.x; u < npairs; u += kFpThreads) {
+            int lo = 0, hi = P - 1;  // the pair's point: base[lo] <= u < base[lo + 1]
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (base[mid] <= u) lo = mid;
+                else hi = mid - 1;
+            }
+            qs[u] = (unsigned char)lo;
+            const long long o = xoff[lo] + (u - base[lo]);
+            double s, c;
+            sincos((double)x[o], &s, &c);
+            const T vv = (T)v[o];
+            zs[u] = s;
+            zc[u] = c;
+            ts[u] = (T)s * vv;
+            tc[u] = (T)c * vv;
+        }
+    }
+
+    __device__ __forceinline__ void load_tile(int mb, int mend)
+    {
+        const int w = fp_stride(sh.nmax), cnt = (mend - mb) * sh.nmax;
+        for (int e = threadIdx.x; e < cnt; e += kFpThreads) {
+            const int mm = e / sh.nmax, j = e - mm * sh.nmax;
+            const double av = __ldg(&a.A[(size_t)(mb + mm) * a.ld + j]), bv = __ldg(&a.B[(size_t)(mb + mm) * a.ld + j]);
+            ta[mm * w + j] = av;
+            tb[mm * w + j] = bv;
+            if constexpr (sizeof(T) == 4) {
+                fa[mm * w + j] = (T)av;
+                fb[mm * w + j] = (T)bv;
+            }
+        }
+    }
+
+    // pass 1 over the tile's rows [mb, mend); every lane of a warp runs the
+    // same number of items (the shuffles)
+    __device__ __forceinline__ void residuals(int mb, int mend)
+    {
+        const int w = fp_stride(sh.nmax), mt = mend - mb, lanes = sh.lanes;
+        const int lane = threadIdx.x & (lanes - 1), items = P * mt, groups = kFpThreads / lanes;
+        const int iters = (items + groups - 1) / groups;
+        for (int it = 0; it < iters; ++it) {
+            const int idx = threadIdx.x / lanes + it * groups;
+            int q = 0, mm = 0, n = 0;
+            if (idx < items) {
+                q = idx / mt;
+                mm = idx - q * mt;
+                if (mb + mm < ns[q]) n = ns[q];
+            }
+            const int z0 = base[q], row = mm * w;
+            double s = 0.0;
+            FpSums<T, 1> d;
+            d.init();
+            int blk = 0;
+            for (int j = lane; j < n; j += lanes) {
+                s = fma(ta[row + j], zs[z0 + j], fma(tb[row + j], zc[z0 + j], s));
+                d.fma_to(0, fa[row + j], tc[z0 + j]);
+                d.fma_to(0, -fb[row + j], ts[z0 + j]);
+                if (++blk == kFpBlock) {
+                    d.flush();
+                    blk = 0;
+                }
+            }
+            d.flush();
+            for (int off = lanes >> 1; off > 0; off >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, off);
+                d.merge_xor(off);
+            }
+            if (n > 0 && lane == 0) {
+                rr[z0 + mb + mm] = (T)(a.E[eoff[q] + mb + mm] - s);
+                dd[z0 + mb + mm] = -d.value(0);
+            }
+        }
+    }
+
+    // pass 2 over the tile's rows
+    __device__ __forceinline__ void transposed(int mb, int mend, FpSums<T, 4> (&sums)[kFpNpt])
+    {
+        const int w = fp_stride(sh.nmax);
+#pragma unroll
+        for (int i = 0; i < kFpNpt; ++i) {
+            const int u = threadIdx.x + i * kFpThreads;
+            if (u >= npairs) break;
+            const int q = qs[u], z0 = base[q], l = u - z0, end = min(mend, ns[q]);
+            int blk = 0;
+            for (int m = mb; m < end; ++m) {
+                const T av = fa[(m - mb) * w + l], bv = fb[(m - mb) * w + l], dv = dd[z0 + m], rv = rr[z0 + m];
+                sums[i].fma_to(0, av, dv);
+                sums[i].fma_to(1, bv, dv);
+                sums[i].fma_to(2, av, rv);
+                sums[i].fma_to(3, bv, rv);
+                if (++blk == 2 * kFpBlock) {
+                    sums[i].flush();
+                    blk = 0;
+                }
+            }
+            sums[i].flush();
+        }
+    }
+
+    __device__ __forceinline__ void run(int m0, int m1, FpSums<T, 4> (&sums)[kFpNpt])
+    {
+#pragma unroll
+        for (int i = 0; i < kFpNpt; ++i) sums[i].init();
+        stage();
+        for (int mb = m0; mb < m1; mb += sh.mt) {
+            const int mend = min(mb + sh.mt, m1);
+            load_tile(mb, mend);
+            __syncthreads();
+            residuals(mb, mend);
+            __syncthreads();
+            transposed(mb, mend, sums);
+            __syncthreads();
+        }
+    }
+
+    // (H v)_l = 2 sum_m [d1_m g_ml + r_m h_ml], g_ml = -(A_ml cos - B_ml sin),
+    // h_ml = (A_ml sin + B_ml cos) v_l
+    __device__ __forceinline__ T combine(int u, T ad, T bd, T ar, T br) const
+    {
+        const T s = (T)zs[u], c = (T)zc[u], vv = (T)v[xoff[qs[u]] + (u - base[qs[u]])];
+        RowSum<T> o;
+        o.add(-c, ad);
+        o.add(s, bd);
+        o.add(s * vv, ar);
+        o.add(c * vv, br);
+        return T(2) * o.value();
+    }
+
+    // The dense propagation for point q (r_m of every m in rr): an x, A
+    // or B that is not finite multiplies seed zeros in some residual of every
+    // component.
+    __device__ __forceinline__ T dense_entry(int q, bool poison, int i, int j) const
+    {
+        if (poison) return nan_of(T(0));
+        const int z0 = base[q];
+        const T si = (T)zs[z0 + i], ci = (T)zc[z0 + i], sj = (T)zs[z0 + j], cj = (T)zc[z0 + j];
+        const T hs = i == j ? -sj : T(0), hc = i == j ? -cj : T(0);
+        TermSum<T, 1, IsComp<T>::value> acc;
+        acc.init();
+        for (int m = 0; m < ns[q]; ++m) {
+            const double *Ar = a.A + (size_t)m * a.ld, *Br = a.B + (size_t)m * a.ld;
+            HD<T, 1> r;
+            r.v = rr[z0 + m];
+            r.d1 = -fma_((T)Br[i], -si, (T)Ar[i] * ci);
+            r.g[0] = -fma_((T)Br[j], -sj, (T)Ar[j] * cj);
+            r.h[0] = -fma_((T)Br[j], hc, (T)Ar[j] * hs);
+            acc.add_sq(r);
+        }
+        return acc.value().h[0];
+    }
+};
+
+// Points whose fast result is not finite, evaluated densely by the CTA; every
+// thread calls it after its outputs are written.
+template <typename T, typename IO>
+__device__ __noinline__ void fp_dense_points(const FpTile<T, IO> t, IO *out, bool wide)
+{
+    for (int q = 0; q < t.P; ++q) {
+        const int n = t.ns[q], z0 = t.base[q];
+        bool bad = false, poison = false;
+        for (int l = threadIdx.x; l < n; l += kFpThreads) {
+            bad |= not_finite((T)out[t.xoff[q] + l]);
+            poison |= not_finite((T)t.x[t.xoff[q] + l]);
+        }
+        if (!__syncthreads_or(bad)) continue;
+        for (int e = threadIdx.x; e < n * n; e += kFpThreads) {
+            const size_t at = (size_t)(e / n) * t.a.ld + e % n;
+            poison |= not_finite((T)t.a.A[at]) || not_finite((T)t.a.B[at]);
+        }
+        poison = __syncthreads_or(poison);
+        // the residuals, again: with the rows split over CTAs rr holds a part
+        for (int m = threadIdx.x; m < n; m += kFpThreads) {
+            double s = 0.0;
+            for (int j = 0; j < n; ++j)
+                s = fma(t.a.A[(size_t)m * t.a.ld + j], t.zs[z0 + j], fma(t.a.B[(size_t)m * t.a.ld + j], t.zc[z0 + j], s));
+            t.rr[z0 + m] = (T)(t.a.E[t.eoff[q] + m] - s);
+        }
+        __syncthreads();
+        const IO *v = t.v + t.xoff[q];
+        for (int s = threadIdx.x; s < n; s += kFpThreads)
+            out[t.xoff[q] + s] =
+                (IO)dense_row<T>(v, n, s, wide, [&](int i, int j) { return t.dense_entry(q, poison, i, j); });
+        __syncthreads();
+    }
+}
+
+}  // namespace chessfad

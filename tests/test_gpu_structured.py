@@ -1,0 +1,105 @@
+"""The structured evaluation (calls that name neither a chunk size nor a
+method) against the oracle and against the dense symmetric method: sizes at
+the edges of its lane groups, shared-memory tiles and pair limits, batches
+that leave a ragged last CTA, and non-finite or overflowing points, which must
+give what the dense method gives."""
+import numpy as np
+import pytest
+
+import paper_2410_22575_gb300 as cf
+from paper_2410_22575_gb300 import workloads as W
+
+from gpu_helpers import BOUND, Dev, hvp_err
+
+pytestmark = pytest.mark.gpu
+
+FNS = [W.ROSENBROCK, W.ACKLEY, W.FLETCHER_POWELL]
+PRECS = [cf.FP64, cf.FP32_COMP]
+
+
+@pytest.mark.parametrize("fn", FNS)
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("n,batch", [(1, 700), (2, 1), (2, 3001), (3, 257), (4, 130), (7, 1000), (8, 33), (9, 70),
+                                     (16, 5), (31, 77), (33, 40), (64, 333), (65, 9), (127, 5), (129, 3), (200, 3),
+                                     (257, 2), (511, 2), (512, 1)])
+def test_hvp_sizes(fn, prec, n, batch):
+    d = Dev(W.make_batch(fn, n, batch, seed=2000 + n), prec)
+    out = d.hvp()
+    e = hvp_err(d, out)
+    assert e.max() <= BOUND[prec], (e.max(), np.median(e))
+    assert np.array_equal(out, d.hvp())
+
+
+def _same(a, b, bound, scale):
+    """Equal NaN and Inf entries, finite entries within bound * scale."""
+    assert np.array_equal(np.isnan(a), np.isnan(b))
+    inf = np.isinf(b)
+    assert np.array_equal(np.isinf(a), inf) and np.array_equal(a[inf], b[inf])
+    ok = np.isfinite(b)
+    assert np.all(np.abs(a[ok] - b[ok]) <= bound * scale)
+
+
+@pytest.mark.parametrize("fn", FNS)
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("n", [2, 3, 5, 21, 64, 300])
+def test_non_finite_points_equal_the_dense_method(fn, prec, n):
+    """NaN and Inf in x, in v and in both, v = 0 beside them, x at the origin
+    (Ackley's square root) and x whose squares overflow: the default call
+    against the dense method it stands for (plain below n = 4)."""
+    bad = [np.nan, np.inf, -np.inf]
+    huge = 1e30 if prec == cf.FP32_COMP else 1e200
+    b = W.make_batch(fn, n, 24, seed=77 + n)
+    for k, val in enumerate(bad):
+        b.x[k, n // 2] = val
+        b.x[3 + k, n - 1] = val
+        b.v[6 + k, n // 2] = val
+        b.x[9 + k, 0] = val
+        b.v[9 + k, n - 1] = bad[(k + 1) % 3]
+        b.x[18 + k, 0] = val
+        b.v[18 + k] = 0.0
+    b.v[12, 0], b.v[12, n - 1] = np.inf, -np.inf
+    b.x[13] = 0.0
+    if fn != W.FLETCHER_POWELL:  # sin and cos of huge arguments: compared through Rosenbrock and Ackley
+        b.x[14, n // 2] = huge
+        b.x[15, 0] = b.x[15, n - 1] = -huge
+        b.x[16, n - 1] = huge
+        b.x[17, n - 2] = huge
+    d = Dev(b, prec)
+    dense = d.hvp(cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 0) if n >= 4 else cf.Config(2, 1, 256))
+    got = d.hvp()
+    fine = np.isfinite(dense)
+    scale = np.max(np.abs(np.where(fine, dense, 0.0)), axis=1, keepdims=True) * np.ones_like(dense)
+    tol = 4e-12 if prec == cf.FP64 else 4e-5
+    _same(got, dense, tol, scale[fine])
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_non_finite_parameters_equal_the_dense_method(prec):
+    import torch
+
+    for which in range(3):
+        b = W.make_batch(W.FLETCHER_POWELL, 13, 50, seed=5)
+        (b.fp.A, b.fp.B, b.fp.E)[which].flat[7] = np.inf
+        d = Dev(b, prec)
+        dense = d.hvp(cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 0))
+        assert np.array_equal(np.isnan(d.hvp()), np.isnan(dense)) and np.all(~np.isfinite(dense))
+
+
+@pytest.mark.parametrize("fn", FNS)
+def test_points_are_independent(fn):
+    """A permuted batch gives the permuted outputs bit for bit, also beside a
+    non-finite point; an offset, 8-byte aligned view gives the same values."""
+    import torch
+
+    b = W.make_batch(fn, 19, 300, seed=8)
+    b.x[100, 3] = np.nan
+    d = Dev(b, cf.FP64)
+    a = d.hvp()
+    perm = np.random.Generator(np.random.PCG64(1)).permutation(300)
+    dp = Dev(W.Batch("p", fn, 19, b.x[perm], b.v[perm], b.fp), cf.FP64)
+    assert np.array_equal(dp.hvp(), a[perm], equal_nan=True)
+    flat = torch.empty(300 * 19 + 1, dtype=torch.float64, device="cuda")
+    view = flat[1:].view(300, 19)
+    view.copy_(d.x)
+    out = cf.hvp(fn, view, d.v, params=d.params)
+    assert np.array_equal(out.cpu().numpy(), a, equal_nan=True)
