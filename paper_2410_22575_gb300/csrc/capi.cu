@@ -310,7 +310,7 @@ static bool dense_rows_in_fp64(int fn, int n, int prec)
 // The library's own choice of evaluation, for calls that name neither a chunk
 // size nor a method: the structured evaluation.
 static int launch_structured(int fn, int n, long long batch, const void *x, const void *v, void *out,
-                             const chessfad_fp_params *params, int prec, cudaStream_t stream)
+                             const chessfad_fp_params *params, int prec, bool hvp, cudaStream_t stream)
 {
     StructArgs a{};
     a.x = x;
@@ -325,7 +325,8 @@ static int launch_structured(int fn, int n, long long batch, const void *x, cons
     a.batch = batch;
     a.n = n;
     a.wide = dense_rows_in_fp64(fn, n, prec);
-    const cudaError_t e = structured_hvp(fn, prec == CHESSFAD_FP64, a, stream);
+    const bool f64 = prec == CHESSFAD_FP64;
+    const cudaError_t e = hvp ? structured_hvp(fn, f64, a, stream) : structured_hessian(fn, f64, a, stream);
     if (e == cudaErrorInvalidConfiguration) return CHESSFAD_ERR_BATCH;
     return e == cudaSuccess ? CHESSFAD_SUCCESS : CHESSFAD_ERR_CUDA;
 }
@@ -346,10 +347,10 @@ static int run(int fn, int n, long long batch, const chessfad_config *cfg, int c
     if (cfg && cfg->csize != 0 && !valid_chunk(cfg->csize)) return CHESSFAD_ERR_CHUNK;
     const bool own = csize_hint == 0 && (!cfg || (!cfg->csize && !cfg->threads_per_row && !cfg->block_threads &&
                                                   !cfg->method && !cfg->threads_per_point));
-    if (hvp && own) {
+    if (own) {
         if (batch == 0) return CHESSFAD_SUCCESS;
-        if (!x || !out || !v) return CHESSFAD_ERR_NULL;
-        return launch_structured(fn, n, batch, x, v, out, params, prec, stream);
+        if (!x || !out || (hvp && !v)) return CHESSFAD_ERR_NULL;
+        return launch_structured(fn, n, batch, x, v, out, params, prec, hvp, stream);
     }
     const chessfad_config c = resolve(fn, n, batch, prec, cfg, csize_hint, hvp);
     st = check_config(c);

@@ -6,6 +6,10 @@
 //   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.35 ms
 //   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.100 ms
 //   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.119 ms
+// Hessians:
+//   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.084 ms (6.4 TB/s written)
+//   Ackley n = 33, FP32-comp, 20000                0.178 ms -> 0.045 ms
+//   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.120 ms
 // The Rosenbrock kernel streams x and v; the other two are bound by the FP64
 // pipe (sin, cos and the sums under sqrt and exp; the residuals), in
 // compensated FP32 too.
@@ -14,19 +18,13 @@
 
 #include "structured.cuh"
 #include "structured.h"
+#include "structured_tune.h"
 
 namespace chessfad {
 namespace {
 
 constexpr int kThreads = 256;
 constexpr long long kMaxBlocks = 0x7fffffffLL;
-
-int pow2_ceil(int v)
-{
-    int p = 1;
-    while (p < v) p <<= 1;
-    return p;
-}
 
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kThreads) ros_hvp_kernel(const StructArgs a, int G)
@@ -40,14 +38,14 @@ __global__ void __launch_bounds__(kThreads) ros_hvp_kernel(const StructArgs a, i
 }
 
 template <typename T, typename IO, int EPL>
-__global__ void __launch_bounds__(kThreads) ack_hvp_kernel(const StructArgs a, int G, double inv_n)
+__global__ void __launch_bounds__(kThreads) ack_hvp_kernel(const StructArgs a, int G, const AckConst nc)
 {
     const long long p = ((long long)blockIdx.x * kThreads + threadIdx.x) / G;
     const int t = threadIdx.x & (G - 1);
     const bool active = p < a.batch;
     const size_t o = active ? (size_t)p * a.n : 0;
     ack_point<T, IO, EPL>(static_cast<const IO *>(a.x) + o, static_cast<const IO *>(a.v) + o,
-                          static_cast<IO *>(a.out) + o, a.n, t, G, active, a.wide, inv_n);
+                          static_cast<IO *>(a.out) + o, a.n, t, G, active, a.wide, nc);
 }
 
 template <typename T, typename IO>
@@ -59,7 +57,7 @@ __global__ void __launch_bounds__(kFpThreads) fp_hvp_kernel(const StructArgs a, 
     const int P = (int)min((long long)ppb, a.batch - p0);
     const FpArgs fa{a.A, a.B, a.E, a.ld};
     IO *out = static_cast<IO *>(a.out);
-    FpTile<T, IO> tile(fa, static_cast<const IO *>(a.x), static_cast<const IO *>(a.v), smem_raw, sh, P, P * n);
+    FpTile<T, IO, true> tile(fa, static_cast<const IO *>(a.x), static_cast<const IO *>(a.v), smem_raw, sh, P, P * n);
     for (int q = threadIdx.x; q <= P; q += kFpThreads) {
         tile.base[q] = q * n;
         if (q < P) {
@@ -76,85 +74,400 @@ __global__ void __launch_bounds__(kFpThreads) fp_hvp_kernel(const StructArgs a, 
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
         if (u >= P * n) break;
-        const T o = tile.combine(u, sums[i].value(0), sums[i].value(1), sums[i].value(2), sums[i].value(3));
+        const FpSums<T, 4> &f = sums[i];
+        const T o = tile.combine(u, f.value(0), f.value(1), f.value(2), f.value(3));
         bad |= not_finite(o);
         out[p0 * n + u] = (IO)o;
     }
-    if (__syncthreads_or(bad)) fp_dense_points<T, IO>(tile, out, a.wide);
+    if (__syncthreads_or(bad)) fp_dense_points<T, IO>(tile, out, a.wide ? 0 : n + 1);
 }
 
-// Lanes per point of the Rosenbrock kernel: about four variables per lane
-// (independent loads in flight), at least 8 lanes where n has them (a warp's
-// loads then cover whole 32-byte sectors).
-int ros_lanes(int n)
-{
-    return std::min(32, std::max(pow2_ceil((n + 3) / 4), std::min(8, pow2_ceil(n))));
-}
+// ---- Hessians
 
-// Lanes per point of the Ackley kernel.  Each lane pays for the cross-lane
-// sums and the tail's scalar functions about as much as for `over` variables,
-// so few lanes with many variables each (at most 16) do least work; a batch
-// too small to fill the GPU that way takes more lanes.
-int ack_lanes(int n, long long batch, bool f64)
+// `rows` rows of the batch's row space per CTA; a row has three entries, the
+// rest of it is the zeros of a terms' independent variables.  Bound by the
+// stores.
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kThreads) ros_hessian_kernel(const StructArgs a, int rows, FastDiv fd)
 {
-    const double over = f64 ? 2.0 : 1.0;
-    int best = 1;
-    double best_cost = 1e300;
-    for (int g = 1; g <= 32; g <<= 1) {
-        const int it = (n + g - 1) / g;
-        if (it > 16 || (g > 1 && g >= 2 * n)) continue;
-        const double waves = std::max(1.0, (double)batch * g / (152.0 * 512.0));
-        const double cost = (it + over) * waves;
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = g;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n;
+    const long long row0 = (long long)blockIdx.x * rows, total = a.batch * n;
+    const int cnt = (int)min((long long)rows, total - row0);
+    T *lo = reinterpret_cast<T *>(smem_raw), *diag = lo + rows, *up = diag + rows;
+    short *ls = reinterpret_cast<short *>(up + rows);
+    const long long p0 = row0 / n;
+    const int l0 = (int)(row0 - p0 * n);
+    const int npts = (l0 + cnt - 1) / n + 1;
+    const IO *x = static_cast<const IO *>(a.x) + p0 * n;  // the first touched point
+    IO *H = static_cast<IO *>(a.out) + (size_t)row0 * n;
+    bool bad = false;
+    for (int e = threadIdx.x; e < npts * n; e += kThreads) {
+        const int l = e - fd.div(e) * n, r = e - l0;
+        const T x0 = (T)x[e], xp = l + 1 < n ? (T)x[e + 1] : T(0);
+        if (l + 1 < n) bad |= not_finite(x0) || not_finite(T(200) * fma_(T(-1), x0 * x0, xp));
+        if (r >= 0 && r < cnt) {
+            const RosRow<T> w = ros_row<T>(l > 0 ? (T)x[e - 1] : T(0), x0, xp, l, n);
+            lo[r] = w.lo;
+            diag[r] = w.diag;
+            up[r] = w.up;
+            ls[r] = (short)l;
+            bad |= not_finite(w.diag) || not_finite(w.up);
         }
     }
-    return best;
+    if (__syncthreads_or(bad)) {  // dense propagation (equal to the rows below for finite points)
+        for (int q = 0; q < npts; ++q) {
+            const int r0 = max(0, l0 - q * n), r1 = min(n, l0 + cnt - q * n);
+            ros_dense_rows<T, IO>(x + (size_t)q * n, static_cast<IO *>(a.out) + (size_t)(p0 + q) * n * n, n, r0, r1);
+        }
+        return;
+    }
+    stream_rows(H, cnt, n, fd, [&](int r, int j) {
+        const int d = j - ls[r] + 1;
+        T v = T(0);
+        if ((unsigned)d <= 2u) v = d == 1 ? diag[r] : d == 2 ? up[r] : lo[r];
+        return v;
+    });
+}
+
+// ppc whole points per CTA, or, split > 1, one of `split` parts of one
+// point's rows.  Entry (i, j) is (K x_i) x_j + (G s_i) s_j, K = p1 r2 + p2 r1^2
+// and G = q2 the second derivatives of the tail in its two sums, s = sin 2 pi x;
+// the diagonal adds p1 r1 + q1 cos 2 pi x.  Bound by the stores and the
+// products that feed them.
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs a, int ppc, int split, FastDiv fd,
+                                                               const AckConst nc)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    struct alignas(2 * sizeof(T)) Pair {
+        T x, s;
+    };
+    const int n = a.n;
+    const long long p0 = split > 1 ? blockIdx.x / split : (long long)blockIdx.x * ppc;
+    const int part = split > 1 ? (int)(blockIdx.x % split) : 0;
+    const int npts = (int)min((long long)ppc, a.batch - p0), nv = npts * n;
+    const int r0 = n * part / split, r1 = split > 1 ? n * (part + 1) / split : nv;
+    Pair *xs = reinterpret_cast<Pair *>(smem_raw);  // x_j, s_j of every variable
+    Pair *ab = xs + ppc * n;                        // K x_i, G s_i
+    T *dg = reinterpret_cast<T *>(ab + ppc * n);    // cos 2 pi x_i, then the diagonal's addition
+    double *sums = reinterpret_cast<double *>(smem_raw + align_up((size_t)ppc * n * 5 * sizeof(T), 16));
+    int *flag = reinterpret_cast<int *>(sums + 2 * ppc);
+    const IO *x = static_cast<const IO *>(a.x) + p0 * n;
+    const int tid = threadIdx.x;
+    for (int u = tid; u < nv; u += kThreads) {
+        T s, c;
+        const T xv = (T)x[u];
+        sincos_2pi<T>(xv, s, c);
+        xs[u].x = xv;
+        xs[u].s = s;
+        dg[u] = c;
+    }
+    for (int q = tid; q < npts; q += kThreads) flag[q] = 0;
+    __syncthreads();
+    // S and C of each point in FP64: few variables by one thread, else a warp
+    const int G = n <= 16 ? 1 : 32, lane = tid & (G - 1);
+    for (int b = 0; b < npts; b += kThreads / G) {
+        const int q = b + tid / G;
+        double S = 0.0, C = 0.0;
+        for (int k = lane; k < n && q < npts; k += G) {
+            const double xd = widen(xs[q * n + k].x);
+            S = fma(xd, xd, S);
+            C += widen(dg[q * n + k]);
+        }
+        for (int off = G >> 1; off > 0; off >>= 1) {
+            S += __shfl_xor_sync(0xffffffffu, S, off);
+            C += __shfl_xor_sync(0xffffffffu, C, off);
+        }
+        if (q < npts && lane == 0) {
+            sums[2 * q] = S;
+            sums[2 * q + 1] = C;
+        }
+    }
+    __syncthreads();
+    // the tail's factors, one thread per point
+    T *tail = reinterpret_cast<T *>(flag + ppc + (ppc & 1));
+    for (int q = tid; q < npts; q += kThreads) {
+        const AckTail<T> k = ack_tail(sums[2 * q], sums[2 * q + 1], nc, T(0));
+        const double p1 = k.p1, r1 = k.r1;  // FP64: the factors are shared by every entry
+        tail[4 * q] = (T)fma(p1, (double)k.r2, ((double)k.p2 * r1) * r1);
+        tail[4 * q + 1] = k.q2;
+        tail[4 * q + 2] = (T)(p1 * r1);
+        tail[4 * q + 3] = k.q1;
+    }
+    __syncthreads();
+    for (int u = tid; u < nv; u += kThreads) {
+        const int q = fd.div(u);
+        const Pair e = xs[u];
+        Pair f;
+        f.x = tail[4 * q] * e.x;
+        f.s = tail[4 * q + 1] * e.s;
+        const T d = fma_(tail[4 * q + 3], dg[u], tail[4 * q + 2]);
+        ab[u] = f;
+        dg[u] = d;
+        if (not_finite(e.x) || not_finite(f.x) || not_finite(f.s) || not_finite(d)) atomicOr(&flag[q], 1);
+    }
+    __syncthreads();
+    IO *H = static_cast<IO *>(a.out) + ((size_t)p0 * n + r0) * n;
+    stream_rows(H, r1 - r0, n, fd, [&](int r, int j) {
+        const int u = r + r0, base = split > 1 ? 0 : fd.div(u) * n;
+        const int w = base + j;  // the smaller index's factors are the scaled ones: H is symmetric bit for bit
+        const Pair e = (w < u ? ab : xs)[w], f = (w < u ? xs : ab)[u];
+        T v = fma_(f.x, e.x, f.s * e.s);
+        if (w == u) v += dg[u];
+        return v;
+    });
+    bool any = false;
+    for (int q = tid; q < npts; q += kThreads) any |= flag[q] != 0;
+    if (__syncthreads_or(any))
+        for (int q = 0; q < npts; ++q)
+            if (flag[q])
+                ack_dense_rows<T, IO>(x + (size_t)q * n, static_cast<IO *>(a.out) + (size_t)(p0 + q) * n * n, n,
+                                      split > 1 ? r0 : 0, split > 1 ? r1 : n);
+}
+
+// Fletcher-Powell, first launch: the diagonal's curvature 2 sum_m r_m P_ml
+// (FP64 residuals), written to the diagonal of H.
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructArgs a, const FpShape sh, int ppb)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n;
+    const long long p0 = (long long)blockIdx.x * ppb;
+    const int P = (int)min((long long)ppb, a.batch - p0);
+    FpTile<T, IO, false> tile(FpArgs{a.A, a.B, a.E, a.ld}, static_cast<const IO *>(a.x), nullptr, smem_raw, sh, P,
+                              P * n);
+    for (int q = threadIdx.x; q <= P; q += kFpThreads) {
+        tile.base[q] = q * n;
+        if (q < P) {
+            tile.ns[q] = n;
+            tile.xoff[q] = (p0 + q) * n;
+            tile.eoff[q] = 0;
+        }
+    }
+    __syncthreads();
+    FpSums<T, 2> sums[kFpNpt];
+    tile.run(0, n, sums);
+#pragma unroll
+    for (int i = 0; i < kFpNpt; ++i) {
+        const int u = threadIdx.x + i * kFpThreads;
+        if (u >= P * n) break;
+        const int l = u - tile.base[tile.qs[u]];
+        static_cast<IO *>(a.out)[((size_t)p0 * n + u) * n + l] = (IO)tile.curvature(u, sums[i]);
+    }
+}
+
+// Second launch, n <= kGramSmall: ppc whole points per CTA, J in shared
+// memory, one 4 x 4 block on or above the diagonal per thread; the result is
+// staged in place of J and streamed out whole.
+constexpr int kGramSmall = 64;
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kThreads) fp_gram_small_kernel(const StructArgs a, int ppc, FastDiv fd)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n, nb = (n + 3) / 4, np = 4 * nb, nt = nb * (nb + 1) / 2, tid = threadIdx.x;
+    const long long p0 = (long long)blockIdx.x * ppc;
+    const int npts = (int)min((long long)ppc, a.batch - p0), nv = npts * n;
+    double *zs = reinterpret_cast<double *>(smem_raw), *zc = zs + n;  // dense propagation only
+    T *r = reinterpret_cast<T *>(zc + n);
+    T *J = reinterpret_cast<T *>(smem_raw + align_up((size_t)n * (2 * sizeof(double) + sizeof(T)), 16));
+    T *ts = J + (size_t)ppc * n * np, *tc = ts + ppc * n, *dg = tc + ppc * n;
+    const IO *x = static_cast<const IO *>(a.x) + p0 * n;
+    IO *H = static_cast<IO *>(a.out) + (size_t)p0 * n * n;
+    bool bad = false;
+    for (int u = tid; u < nv; u += kThreads) {
+        double s, c;
+        sincos((double)x[u], &s, &c);
+        ts[u] = (T)s;
+        tc[u] = (T)c;
+        dg[u] = (T)H[(size_t)u * n + (u - fd.div(u) * n)];
+        bad |= not_finite(dg[u]);
+    }
+    __syncthreads();
+    for (int e = tid; e < n * np; e += kThreads) {
+        const int m = e / np, j = e - m * np;
+        T av = T(0), bv = T(0);
+        if (j < n) {
+            av = narrow<T>(__ldg(&a.A[(size_t)m * a.ld + j]));
+            bv = narrow<T>(__ldg(&a.B[(size_t)m * a.ld + j]));
+        }
+        for (int q = 0; q < npts; ++q)
+            J[(size_t)q * n * np + e] = j < n ? fp_jacobian(av, bv, ts[q * n + j], tc[q * n + j]) : T(0);
+    }
+    __syncthreads();
+    // the thread's point and block (bi <= bj), blocks of a point row by row
+    const int q = tid / nt;
+    int bi = 0, bj = tid - q * nt;
+    while (bi < nb && bj >= nb - bi) {
+        bj -= nb - bi;
+        ++bi;
+    }
+    bj += bi;
+    Gram4<T> g;
+    g.init();
+    if (q < npts) {
+        const T *Jq = J + (size_t)q * n * np;
+        int blk = 0;
+        for (int m = 0; m < n; ++m) {
+            g.add(Jq + m * np + 4 * bi, Jq + m * np + 4 * bj);
+            if (++blk == kSumBlock) {
+                g.flush();
+                blk = 0;
+            }
+        }
+        g.flush();
+    }
+    __syncthreads();
+    if (q < npts) {
+        T *Hs = J + (size_t)q * n * np;  // row stride np
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int ri = 4 * bi + i, rj = 4 * bj + j;
+                if (ri >= n || rj >= n) continue;
+                T v = g.value(i, j);
+                if (ri == rj) v += dg[q * n + ri];
+                Hs[ri * np + rj] = v;
+                if (bi != bj) Hs[rj * np + ri] = v;
+            }
+    }
+    __syncthreads();
+    stream_rows(H, nv, n, fd, [&](int row, int j) { return J[(size_t)row * np + j]; });
+    if (__syncthreads_or(bad))
+        for (int k = 0; k < npts; ++k) {
+            bool b = false;
+            for (int l = tid; l < n; l += kThreads) b |= not_finite(dg[k * n + l]);
+            if (__syncthreads_or(b))
+                fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, x + (size_t)k * n, H + (size_t)k * n * n, n, zs,
+                                        zc, r);
+        }
+}
+
+// Second launch, n > kGramSmall: a CTA takes one 64 x 64 block (I <= J) of one
+// point, J formed for the two column ranges in tiles of kGramRows rows.
+constexpr int kGramTile = 64;
+constexpr int kGramRows = 16;
+template <typename T>
+__host__ __device__ constexpr size_t gram_smem()
+{
+    // two J tiles, the staged block, sin and cos of both ranges
+    return (size_t)(2 * kGramRows * kGramTile + kGramTile * (kGramTile + 1) + 4 * kGramTile) * sizeof(T);
+}
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kThreads) fp_gram_kernel(const StructArgs a, int nbk)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *JI = reinterpret_cast<T *>(smem_raw), *JJ = JI + kGramRows * kGramTile;
+    T *tile = JJ + kGramRows * kGramTile, *ts = tile + kGramTile * (kGramTile + 1), *tc = ts + 2 * kGramTile;
+    const int n = a.n, tid = threadIdx.x, nt = nbk * (nbk + 1) / 2;
+    const long long p = blockIdx.x / nt;
+    int bi = 0, bj = (int)(blockIdx.x % nt);
+    while (bj >= nbk - bi) {
+        bj -= nbk - bi;
+        ++bi;
+    }
+    bj += bi;
+    const int i0 = bi * kGramTile, j0 = bj * kGramTile;
+    const IO *x = static_cast<const IO *>(a.x) + p * n;
+    IO *H = static_cast<IO *>(a.out) + (size_t)p * n * n;
+    if (tid < 2 * kGramTile) {
+        const int col = tid < kGramTile ? i0 + tid : j0 + tid - kGramTile;
+        double s = 0.0, c = 0.0;
+        if (col < n) sincos((double)x[col], &s, &c);
+        ts[tid] = (T)s;
+        tc[tid] = (T)c;
+    }
+    const int ty = tid / 16, tx = tid % 16;
+    Gram4<T> g;
+    g.init();
+    for (int mb = 0; mb < n; mb += kGramRows) {
+        __syncthreads();
+        for (int e = tid; e < 2 * kGramRows * kGramTile; e += kThreads) {
+            const int half = e / (kGramRows * kGramTile), w = e % (kGramRows * kGramTile);
+            if (half && bi == bj) break;
+            const int m = mb + w / kGramTile, k = w % kGramTile, col = (half ? j0 : i0) + k;
+            T v = T(0);
+            if (m < n && col < n)
+                v = fp_jacobian(narrow<T>(__ldg(&a.A[(size_t)m * a.ld + col])),
+                                narrow<T>(__ldg(&a.B[(size_t)m * a.ld + col])), ts[half * kGramTile + k],
+                                tc[half * kGramTile + k]);
+            (half ? JJ : JI)[w] = v;
+        }
+        __syncthreads();
+        const T *Q = bi == bj ? JI : JJ;
+#pragma unroll
+        for (int m = 0; m < kGramRows; ++m) {
+            g.add(JI + m * kGramTile + 4 * ty, Q + m * kGramTile + 4 * tx);
+            if (m % kSumBlock == kSumBlock - 1) g.flush();
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int ri = 4 * ty + i, rj = 4 * tx + j;
+            T v = g.value(i, j);
+            if (bi == bj && ri == rj && i0 + ri < n) v += (T)H[(size_t)(i0 + ri) * n + i0 + ri];
+            tile[ri * (kGramTile + 1) + rj] = v;
+        }
+    __syncthreads();
+    for (int e = tid; e < kGramTile * kGramTile; e += kThreads) {
+        const int u = e / kGramTile, w = e % kGramTile;
+        if (i0 + u < n && j0 + w < n) H[(size_t)(i0 + u) * n + j0 + w] = (IO)tile[u * (kGramTile + 1) + w];
+        if (bi != bj && j0 + u < n && i0 + w < n) H[(size_t)(j0 + u) * n + i0 + w] = (IO)tile[w * (kGramTile + 1) + u];
+    }
+}
+
+// Third launch, n > kGramSmall: points whose residuals are not finite (their
+// whole diagonal is not) by the dense propagation.
+template <typename T, typename IO>
+__global__ void __launch_bounds__(kThreads) fp_hessian_fix_kernel(const StructArgs a)
+{
+    __shared__ double zs[kMaxVars], zc[kMaxVars];
+    __shared__ T r[kMaxVars];
+    __shared__ bool todo[kThreads];
+    const size_t nn = (size_t)a.n * a.n;
+    const long long p0 = (long long)blockIdx.x * kThreads, p = p0 + threadIdx.x;
+    IO *H = static_cast<IO *>(a.out);
+    todo[threadIdx.x] = p < a.batch && not_finite((T)H[(size_t)p * nn]);
+    if (!__syncthreads_or(todo[threadIdx.x])) return;
+    for (int k = 0; k < kThreads; ++k)
+        if (todo[k])
+            fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, static_cast<const IO *>(a.x) + (p0 + k) * a.n,
+                                    H + (size_t)(p0 + k) * nn, a.n, zs, zc, r);
 }
 
 template <typename T, typename IO>
 cudaError_t ack_launch(const StructArgs &a, int G, unsigned blocks, cudaStream_t s)
 {
     const int it = (a.n + G - 1) / G;
-    const double inv_n = 1.0 / a.n;
-    if (it <= 1) ack_hvp_kernel<T, IO, 1><<<blocks, kThreads, 0, s>>>(a, G, inv_n);
-    else if (it <= 2) ack_hvp_kernel<T, IO, 2><<<blocks, kThreads, 0, s>>>(a, G, inv_n);
-    else if (it <= 4) ack_hvp_kernel<T, IO, 4><<<blocks, kThreads, 0, s>>>(a, G, inv_n);
-    else if (it <= 8) ack_hvp_kernel<T, IO, 8><<<blocks, kThreads, 0, s>>>(a, G, inv_n);
-    else ack_hvp_kernel<T, IO, 16><<<blocks, kThreads, 0, s>>>(a, G, inv_n);
+    const AckConst nc = ack_const(a.n);
+    if (it <= 1) ack_hvp_kernel<T, IO, 1><<<blocks, kThreads, 0, s>>>(a, G, nc);
+    else if (it <= 2) ack_hvp_kernel<T, IO, 2><<<blocks, kThreads, 0, s>>>(a, G, nc);
+    else if (it <= 4) ack_hvp_kernel<T, IO, 4><<<blocks, kThreads, 0, s>>>(a, G, nc);
+    else if (it <= 8) ack_hvp_kernel<T, IO, 8><<<blocks, kThreads, 0, s>>>(a, G, nc);
+    else ack_hvp_kernel<T, IO, 16><<<blocks, kThreads, 0, s>>>(a, G, nc);
     return cudaGetLastError();
 }
 
-// Rows of A and B per tile: all of them within 64 KiB (two or more CTAs per
-// SM hide the barriers between the passes), else even parts of the rows.
-template <typename T>
-FpShape fp_shape(int nmax, int rows, int P)
+// Points per CTA of an FpTile kernel: as many pairs as its threads hold,
+// fewer when the batch would leave SMs without a CTA.
+int fp_points(int n, long long batch)
 {
-    const size_t row = (size_t)fp_stride(nmax) * 2 * (sizeof(double) + (sizeof(T) == 4 ? sizeof(float) : 0));
-    const int most = std::max(1, (int)(64 * 1024 / row));
-    const int tiles = (rows + most - 1) / most;
-    FpShape s;
-    s.nmax = nmax;
-    s.mt = (rows + tiles - 1) / tiles;
-    // pass 1: enough lanes per (point, row) to occupy the CTA's threads
-    s.lanes = 1;
-    while (s.lanes < 32 && s.lanes < nmax && P * s.mt * s.lanes < kFpThreads) s.lanes <<= 1;
-    return s;
+    const int most = std::max(1, std::min(kFpMaxPts, kFpPairs / n));
+    return (int)std::min<long long>(most, std::max<long long>(1, (batch + 303) / 304));
 }
 
-template <typename T, typename IO>
+template <typename T, typename IO, bool kHvp>
 cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
 {
-    // Points per CTA: as many pairs as its threads hold, fewer when the batch
-    // would leave SMs without a CTA.
-    int ppb = std::max(1, std::min(kFpMaxPts, kFpPairs / a.n));
-    ppb = (int)std::min<long long>(ppb, std::max<long long>(1, (a.batch + 303) / 304));
+    const int ppb = fp_points(a.n, a.batch);
     const FpShape sh = fp_shape<T>(a.n, a.n, ppb);
     const size_t bytes = fp_smem<T>(sh.nmax, sh.mt).total;
     const long long blocks = (a.batch + ppb - 1) / ppb;
     if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
-    auto kern = fp_hvp_kernel<T, IO>;
+    auto kern = kHvp ? fp_hvp_kernel<T, IO> : fp_curvature_kernel<T, IO>;
     static std::atomic<int> configured[64];
     const cudaError_t e = opt_in_smem(kern, bytes, configured);
     if (e != cudaSuccess) return e;
@@ -165,12 +478,77 @@ cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
 template <typename T, typename IO>
 cudaError_t hvp(int fn, const StructArgs &a, cudaStream_t s)
 {
-    if (fn == FN_FP) return fp_launch<T, IO>(a, s);
+    if (fn == FN_FP) return fp_launch<T, IO, true>(a, s);
     const int G = fn == FN_ROSENBROCK ? ros_lanes(a.n) : ack_lanes(a.n, a.batch, sizeof(T) == 8);
     const long long ppb = kThreads / G, blocks = (a.batch + ppb - 1) / ppb;
     if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
     if (fn == FN_ACKLEY) return ack_launch<T, IO>(a, G, (unsigned)blocks, s);
     ros_hvp_kernel<T, IO><<<(unsigned)blocks, kThreads, 0, s>>>(a, G);
+    return cudaGetLastError();
+}
+
+// Output elements per CTA of the streaming Hessian kernels: enough to hide a
+// CTA's start, few enough for several CTAs per SM.
+constexpr int kHessElems = 16384;
+
+template <typename T, typename IO>
+cudaError_t fp_hessian(const StructArgs &a, FastDiv fd, cudaStream_t s)
+{
+    const int n = a.n;
+    const int nbk = (n + kGramTile - 1) / kGramTile, nt = nbk * (nbk + 1) / 2;
+    if (n > kGramSmall && a.batch > kMaxBlocks / nt) return cudaErrorInvalidConfiguration;
+    cudaError_t e = fp_launch<T, IO, false>(a, s);
+    if (e != cudaSuccess) return e;
+    static std::atomic<int> small_smem[64], gram_attr[64];
+    if (n <= kGramSmall) {
+        const int nb = (n + 3) / 4, np = 4 * nb, tiles = nb * (nb + 1) / 2;
+        // points per CTA: one 4 x 4 block per thread, at most 64 KiB of J
+        const size_t per = (size_t)n * (np + 3) * sizeof(T);
+        int ppc = std::max(1, std::min(kThreads / tiles, (int)(64 * 1024 / per)));
+        ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 303) / 304));
+        const size_t bytes = align_up((size_t)n * (2 * sizeof(double) + sizeof(T)), 16) + ppc * per;
+        const long long blocks = (a.batch + ppc - 1) / ppc;
+        if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
+        auto kern = fp_gram_small_kernel<T, IO>;
+        e = opt_in_smem(kern, bytes, small_smem);
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)blocks, kThreads, bytes, s>>>(a, ppc, fd);
+        return cudaGetLastError();
+    }
+    auto kern = fp_gram_kernel<T, IO>;
+    e = opt_in_smem(kern, gram_smem<T>(), gram_attr);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(a.batch * nt), kThreads, gram_smem<T>(), s>>>(a, nbk);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    fp_hessian_fix_kernel<T, IO><<<(unsigned)((a.batch + kThreads - 1) / kThreads), kThreads, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename T, typename IO>
+cudaError_t hessian(int fn, const StructArgs &a, cudaStream_t s)
+{
+    const int n = a.n;
+    const FastDiv fd{n == 1 ? 0u : (unsigned)((1ull << 32) / (unsigned)n + 1)};
+    if (fn == FN_FP) return fp_hessian<T, IO>(a, fd, s);
+    if (fn == FN_ROSENBROCK) {
+        const long long total = a.batch * n;
+        int rows = std::max(1, std::min(1024, kHessElems / n));
+        rows = (int)std::min<long long>(rows, std::max<long long>(8, total / 304));
+        const long long blocks = (total + rows - 1) / rows;
+        if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
+        const size_t bytes = (size_t)rows * (3 * sizeof(T) + sizeof(short));
+        ros_hessian_kernel<T, IO><<<(unsigned)blocks, kThreads, bytes, s>>>(a, rows, fd);
+        return cudaGetLastError();
+    }
+    const int split = std::max(1, (n * n + kHessElems - 1) / kHessElems);
+    int ppc = split > 1 ? 1 : std::max(1, std::min(512 / n, kHessElems / (n * n)));
+    ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 303) / 304));
+    const long long ctas = (a.batch + ppc - 1) / ppc;
+    if (ctas > kMaxBlocks / split) return cudaErrorInvalidConfiguration;
+    const size_t bytes = align_up((size_t)ppc * n * 5 * sizeof(T), 16) + ppc * (2 * sizeof(double) + 4 * sizeof(T)) +
+                         (ppc + (ppc & 1)) * sizeof(int);
+    ack_hessian_kernel<T, IO><<<(unsigned)(ctas * split), kThreads, bytes, s>>>(a, ppc, split, fd, ack_const(n));
     return cudaGetLastError();
 }
 
@@ -180,6 +558,12 @@ cudaError_t structured_hvp(int fn, bool f64, const StructArgs &a, cudaStream_t s
 {
     if (f64) return hvp<double, double>(fn, a, stream);
     return a.n == 1 ? hvp<double, float>(fn, a, stream) : hvp<float, float>(fn, a, stream);
+}
+
+cudaError_t structured_hessian(int fn, bool f64, const StructArgs &a, cudaStream_t stream)
+{
+    if (f64) return hessian<double, double>(fn, a, stream);
+    return a.n == 1 ? hessian<double, float>(fn, a, stream) : hessian<float, float>(fn, a, stream);
 }
 
 }  // namespace chessfad

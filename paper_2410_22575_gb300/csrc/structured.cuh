@@ -58,6 +58,23 @@ __device__ __forceinline__ double widen(float x)
     return (double)x;
 }
 
+// double -> float, round to nearest even, through the integer pipe for results
+// in the normal float range (others take the conversion instruction).
+template <typename T>
+__device__ __forceinline__ T narrow(double x);
+template <>
+__device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float narrow<float>(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
+    if (m - (897ull << 52) < (253ull << 52)) {  // 2^-126 <= |x| < 2^127
+        const unsigned r = (unsigned)((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23);
+        return __uint_as_float(r | (unsigned)(b >> 63) << 31);
+    }
+    return (float)x;
+}
+
 // The row-times-v sum of the dense sweeps: Dot2 in compensated FP32, FMAs in
 // FP64.
 template <typename T>
@@ -157,7 +174,9 @@ __device__ __forceinline__ T ros_dense_entry(const IO *x, int n, const RosBad &b
     if (b.all || (b.count > 0 && !(b.count == 1 && i == j && b.at == i))) return nan_of(T(0));
     if (i - j > 1 || j - i > 1) return T(0);
     const RosRow<T> r = ros_row<T>(i > 0 ? (T)x[i - 1] : T(0), (T)x[i], i + 1 < n ? (T)x[i + 1] : T(0), i, n);
-    return j < i ? r.lo : j == i ? r.diag : r.up;
+    const T v = j < i ? r.lo : j == i ? r.diag : r.up;
+    // an infinite term leaves a NaN in the TwoSum of compensated FP32
+    return IsComp<T>::value && not_finite(v) ? nan_of(T(0)) : v;
 }
 template <typename T, typename IO>
 __device__ __noinline__ void ros_dense_hvp(const IO *x, const IO *v, IO *out, int n, int t, int G, bool wide)
@@ -214,39 +233,65 @@ template <typename T>
 struct AckTail {
     T r1, r2;  // r', r''
     T p1, p2;  // of -20 exp(-0.2 r)
-    T q1, q2;  // of -exp(C/n)
+    T q1, q2;  // of -exp(C/n), times -4 pi^2 and 4 pi^2: the factors that
+               // cos 2 pi x's phi'' = -4 pi^2 cos and phi' = -2 pi sin (twice)
+               // leave when C's components are taken as plain cos and sin
 };
+// The constant factors of n variables: 1/n, 1/n^2, 4 pi^2/n and -4 pi^2/n^2,
+// in compensated FP32 as unevaluated pairs (the rounded constant alone would
+// put the same error into every point).  One per launch.
+struct AckConst {
+    double inv_n, k[4];
+    float hi[4], lo[4];
+};
+__host__ __device__ inline AckConst ack_const(int n)
+{
+    AckConst c;
+    const double four_pi_sq = 39.478417604357434475337963999504604541254797628963;
+    c.inv_n = 1.0 / n;
+    c.k[0] = c.inv_n;
+    c.k[1] = 1.0 / ((double)n * n);
+    c.k[2] = four_pi_sq * c.k[0];
+    c.k[3] = -four_pi_sq * c.k[1];
+    for (int i = 0; i < 4; ++i) {
+        c.hi[i] = (float)c.k[i];
+        c.lo[i] = (float)(c.k[i] - (double)c.hi[i]);
+    }
+    return c;
+}
+
 // The scalar functions in FP64, or, for compensated FP32, in FP32 from the
 // correctly rounded FP64 sums.
-__device__ __forceinline__ AckTail<double> ack_tail(double S, double C, double inv_n, double)
+__device__ __forceinline__ AckTail<double> ack_tail(double S, double C, const AckConst &n, double)
 {
     AckTail<double> k;
-    const double a0 = S * inv_n, sq = sqrt(a0), k2 = 2.0 * inv_n;
-    const double e1 = exp(-0.2 * sq), e2 = exp(C * inv_n);
-    k.r1 = k2 * (0.5 / sq);
-    k.r2 = (k2 * k2) * (-0.25 / (sq * a0));
+    const double a0 = S * n.inv_n, sq = sqrt(a0), e1 = exp(-0.2 * sq), e2 = exp(C * n.inv_n);
+    k.r1 = n.k[0] / sq;
+    k.r2 = -n.k[1] / (sq * a0);
     k.p1 = 4.0 * e1;
     k.p2 = -0.8 * e1;
-    k.q1 = -inv_n * e2;
-    k.q2 = -(inv_n * inv_n) * e2;
+    k.q1 = n.k[2] * e2;
+    k.q2 = n.k[3] * e2;
     return k;
 }
-__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, double inv_n, float)
+__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const AckConst &n, float)
 {
     AckTail<float> k;
-    const float a0 = (float)(S * inv_n), sq = sqrtf(a0), in = (float)inv_n, k2 = 2.0f * in;
-    const float e1 = expf(-0.2f * sq), e2 = expf((float)(C * inv_n));
-    k.r1 = k2 * (0.5f / sq);
-    k.r2 = (k2 * k2) * (-0.25f / (sq * a0));
+    const float a0 = (float)(S * n.inv_n), sq = sqrtf(a0);
+    const float e1 = expf(-0.2f * sq), e2 = expf((float)(C * n.inv_n));
+    const float d1 = 1.0f / sq, d2 = -1.0f / (sq * a0);
+    auto times = [&](int i, float y) { return __fmaf_rn(n.hi[i], y, n.lo[i] * y); };
+    k.r1 = times(0, d1);
+    k.r2 = times(1, d2);
     k.p1 = 4.0f * e1;
     k.p2 = -0.8f * e1;
-    k.q1 = -in * e2;
-    k.q2 = -(in * in) * e2;
+    k.q1 = times(2, e2);
+    k.q2 = times(3, e2);
     return k;
 }
 
 // One variable's h component of the whole tail: S/2 carries (d1 = sd, g = x,
-// h = sh), C carries (d1 = cd, g = cg, h = ch).
+// h = sh), C carries (d1 = cd, g = cg, h = ch) in the units of q1, q2.
 template <typename T>
 __device__ __forceinline__ T ack_tail_h(const AckTail<T> &k, T sd, T x, T sh, T cd, T cg, T ch)
 {
@@ -282,7 +327,7 @@ struct AckDense {
             S = fma((double)xj, (double)xj, S);
             C += (double)c;
         }
-        k = ack_tail(S, C, 1.0 / n, T(0));
+        k = ack_tail(S, C, ack_const(n), T(0));
     }
     __device__ __forceinline__ T entry(int i, int j) const
     {
@@ -290,8 +335,7 @@ struct AckDense {
         T si, ci, sj, cj;
         sincos_2pi<T>((T)x[i], si, ci);
         sincos_2pi<T>((T)x[j], sj, cj);
-        const T m2p = T(-2.0 * CUDART_PI), m4p = T(-4.0 * CUDART_PI * CUDART_PI);
-        return ack_tail_h<T>(k, (T)x[i], (T)x[j], i == j ? T(1) : T(0), m2p * si, m2p * sj, i == j ? m4p * cj : T(0));
+        return ack_tail_h<T>(k, (T)x[i], (T)x[j], i == j ? T(1) : T(0), si, sj, i == j ? cj : T(0));
     }
 };
 template <typename T, typename IO>
@@ -306,7 +350,8 @@ __device__ __noinline__ void ack_dense_hvp(const IO *x, const IO *v, IO *out, in
 // variables per lane (variable t + G j), n <= G EPL.
 template <typename T, typename IO, int EPL>
 __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__restrict__ v, IO *__restrict__ out,
-                                          int n, int t, int G, bool active, bool wide, double inv_n)
+                                          int n, int t, int G, bool active, bool wide,
+                                          const AckConst &nc)
 {
     const int m = active ? n : 0;
     T xs[EPL], vs[EPL], sn[EPL], cs[EPL];
@@ -322,7 +367,6 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
             vs[j] = (T)v[k];
         }
     }
-    const T m2p = T(-2.0 * CUDART_PI), m4p = T(-4.0 * CUDART_PI * CUDART_PI);
 #pragma unroll
     for (int j = 0; j < EPL; ++j) {
         if (G * j < n) {  // uniform in the group
@@ -331,7 +375,6 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
                 const double xd = widen(xs[j]);
                 S = fma(xd, xd, S);
                 C += widen(cs[j]);
-                sn[j] = m2p * sn[j];
                 xv.add(xs[j], vs[j]);
                 sv.add(sn[j], vs[j]);
             }
@@ -345,12 +388,12 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
     }
     bool bad = false;
     if (active) {
-        const AckTail<T> k = ack_tail(S, C, inv_n, T(0));
+        const AckTail<T> k = ack_tail(S, C, nc, T(0));
         const T xd = xv.value(), sd = sv.value();
 #pragma unroll
         for (int j = 0; j < EPL; ++j) {
             if (t + G * j < n) {
-                const T o = ack_tail_h<T>(k, xd, xs[j], vs[j], sd, sn[j], (m4p * cs[j]) * vs[j]);
+                const T o = ack_tail_h<T>(k, xd, xs[j], vs[j], sd, sn[j], cs[j] * vs[j]);
                 bad |= not_finite(o);
                 out[t + G * j] = (IO)o;
             }
@@ -443,6 +486,7 @@ struct FpSums<double, N> {
     __device__ __forceinline__ void fma_to(int i, double a, double b) { s[i] = __fma_rn(a, b, s[i]); }
     __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value(int i) const { return s[i]; }
+    __device__ __forceinline__ double wide(int i) const { return s[i]; }
     __device__ __forceinline__ void merge_xor(int off)
     {
 #pragma unroll
@@ -472,6 +516,7 @@ struct FpSums<float, N> {
         }
     }
     __device__ __forceinline__ float value(int i) const { return csum_value(s[i]); }
+    __device__ __forceinline__ double wide(int i) const { return widen(s[i].s) + widen(s[i].e); }
     __device__ __forceinline__ void merge_xor(int off)
     {
 #pragma unroll
@@ -494,8 +539,11 @@ struct FpArgs {
 // (base[P] = the pair count), xoff[q] and eoff[q], and synchronised.
 // Afterwards sums[i] holds the four pass-2 sums of pair tid + i kFpThreads
 // over the rows m0 <= m < m1.
-template <typename T, typename IO>
+// kDir: with the direction v (products H v); without it only r_m and the two
+// sums over it (the Hessian's diagonal part).
+template <typename T, typename IO, bool kDir>
 struct FpTile {
+    static constexpr int NS = kDir ? 4 : 2;
     const FpArgs a;
     const IO *x, *v;
     unsigned char *smem;
@@ -543,11 +591,13 @@ struct FpTile {
             const long long o = xoff[lo] + (u - base[lo]);
             double s, c;
             sincos((double)x[o], &s, &c);
-            const T vv = (T)v[o];
             zs[u] = s;
             zc[u] = c;
-            ts[u] = (T)s * vv;
-            tc[u] = (T)c * vv;
+            if constexpr (kDir) {
+                const T vv = (T)v[o];
+                ts[u] = (T)s * vv;
+                tc[u] = (T)c * vv;
+            }
         }
     }
 
@@ -560,8 +610,8 @@ struct FpTile {
             ta[mm * w + j] = av;
             tb[mm * w + j] = bv;
             if constexpr (sizeof(T) == 4) {
-                fa[mm * w + j] = (T)av;
-                fb[mm * w + j] = (T)bv;
+                fa[mm * w + j] = narrow<T>(av);
+                fb[mm * w + j] = narrow<T>(bv);
             }
         }
     }
@@ -588,27 +638,29 @@ struct FpTile {
             int blk = 0;
             for (int j = lane; j < n; j += lanes) {
                 s = fma(ta[row + j], zs[z0 + j], fma(tb[row + j], zc[z0 + j], s));
-                d.fma_to(0, fa[row + j], tc[z0 + j]);
-                d.fma_to(0, -fb[row + j], ts[z0 + j]);
-                if (++blk == kFpBlock) {
-                    d.flush();
-                    blk = 0;
+                if constexpr (kDir) {
+                    d.fma_to(0, fa[row + j], tc[z0 + j]);
+                    d.fma_to(0, -fb[row + j], ts[z0 + j]);
+                    if (++blk == kFpBlock) {
+                        d.flush();
+                        blk = 0;
+                    }
                 }
             }
             d.flush();
             for (int off = lanes >> 1; off > 0; off >>= 1) {
                 s += __shfl_xor_sync(0xffffffffu, s, off);
-                d.merge_xor(off);
+                if constexpr (kDir) d.merge_xor(off);
             }
             if (n > 0 && lane == 0) {
                 rr[z0 + mb + mm] = (T)(a.E[eoff[q] + mb + mm] - s);
-                dd[z0 + mb + mm] = -d.value(0);
+                if constexpr (kDir) dd[z0 + mb + mm] = -d.value(0);
             }
         }
     }
 
     // pass 2 over the tile's rows
-    __device__ __forceinline__ void transposed(int mb, int mend, FpSums<T, 4> (&sums)[kFpNpt])
+    __device__ __forceinline__ void transposed(int mb, int mend, FpSums<T, NS> (&sums)[kFpNpt])
     {
         const int w = fp_stride(sh.nmax);
 #pragma unroll
@@ -618,11 +670,14 @@ struct FpTile {
             const int q = qs[u], z0 = base[q], l = u - z0, end = min(mend, ns[q]);
             int blk = 0;
             for (int m = mb; m < end; ++m) {
-                const T av = fa[(m - mb) * w + l], bv = fb[(m - mb) * w + l], dv = dd[z0 + m], rv = rr[z0 + m];
-                sums[i].fma_to(0, av, dv);
-                sums[i].fma_to(1, bv, dv);
-                sums[i].fma_to(2, av, rv);
-                sums[i].fma_to(3, bv, rv);
+                const T av = fa[(m - mb) * w + l], bv = fb[(m - mb) * w + l], rv = rr[z0 + m];
+                sums[i].fma_to(0, av, rv);
+                sums[i].fma_to(1, bv, rv);
+                if constexpr (kDir) {
+                    const T dv = dd[z0 + m];
+                    sums[i].fma_to(2, av, dv);
+                    sums[i].fma_to(3, bv, dv);
+                }
                 if (++blk == 2 * kFpBlock) {
                     sums[i].flush();
                     blk = 0;
@@ -632,7 +687,7 @@ struct FpTile {
         }
     }
 
-    __device__ __forceinline__ void run(int m0, int m1, FpSums<T, 4> (&sums)[kFpNpt])
+    __device__ __forceinline__ void run(int m0, int m1, FpSums<T, NS> (&sums)[kFpNpt])
     {
 #pragma unroll
         for (int i = 0; i < kFpNpt; ++i) sums[i].init();
@@ -650,7 +705,7 @@ struct FpTile {
 
     // (H v)_l = 2 sum_m [d1_m g_ml + r_m h_ml], g_ml = -(A_ml cos - B_ml sin),
     // h_ml = (A_ml sin + B_ml cos) v_l
-    __device__ __forceinline__ T combine(int u, T ad, T bd, T ar, T br) const
+    __device__ __forceinline__ T combine(int u, T ar, T br, T ad, T bd) const
     {
         const T s = (T)zs[u], c = (T)zc[u], vv = (T)v[xoff[qs[u]] + (u - base[qs[u]])];
         RowSum<T> o;
@@ -660,63 +715,245 @@ struct FpTile {
         o.add(c * vv, br);
         return T(2) * o.value();
     }
+    // the diagonal's second-derivative part, 2 sum_m r_m (A_ml sin + B_ml cos)
+    __device__ __forceinline__ T curvature(int u, const FpSums<T, 2> &sum) const
+    {
+        RowSum<T> o;
+        o.add((T)zs[u], sum.value(0));
+        o.add((T)zc[u], sum.value(1));
+        return T(2) * o.value();
+    }
+};
 
-    // The dense propagation for point q (r_m of every m in rr): an x, A
-    // or B that is not finite multiplies seed zeros in some residual of every
-    // component.
-    __device__ __forceinline__ T dense_entry(int q, bool poison, int i, int j) const
+// One point for the dense propagation: sin, cos (FP64) and the residuals of
+// every variable.  An x, A or B that is not finite multiplies seed zeros in
+// some residual of every component (poison).
+template <typename T>
+struct FpDense {
+    const double *A, *B;
+    int ld, n;
+    const double *zs, *zc;
+    const T *r;
+    bool poison;
+    __device__ __forceinline__ T entry(int i, int j) const
     {
         if (poison) return nan_of(T(0));
-        const int z0 = base[q];
-        const T si = (T)zs[z0 + i], ci = (T)zc[z0 + i], sj = (T)zs[z0 + j], cj = (T)zc[z0 + j];
+        const T si = (T)zs[i], ci = (T)zc[i], sj = (T)zs[j], cj = (T)zc[j];
         const T hs = i == j ? -sj : T(0), hc = i == j ? -cj : T(0);
         TermSum<T, 1, IsComp<T>::value> acc;
         acc.init();
-        for (int m = 0; m < ns[q]; ++m) {
-            const double *Ar = a.A + (size_t)m * a.ld, *Br = a.B + (size_t)m * a.ld;
-            HD<T, 1> r;
-            r.v = rr[z0 + m];
-            r.d1 = -fma_((T)Br[i], -si, (T)Ar[i] * ci);
-            r.g[0] = -fma_((T)Br[j], -sj, (T)Ar[j] * cj);
-            r.h[0] = -fma_((T)Br[j], hc, (T)Ar[j] * hs);
-            acc.add_sq(r);
+        for (int m = 0; m < n; ++m) {
+            const double *Ar = A + (size_t)m * ld, *Br = B + (size_t)m * ld;
+            HD<T, 1> t;
+            t.v = r[m];
+            t.d1 = -fma_((T)Br[i], -si, (T)Ar[i] * ci);
+            t.g[0] = -fma_((T)Br[j], -sj, (T)Ar[j] * cj);
+            t.h[0] = -fma_((T)Br[j], hc, (T)Ar[j] * hs);
+            acc.add_sq(t);
         }
         return acc.value().h[0];
     }
 };
 
-// Points whose fast result is not finite, evaluated densely by the CTA; every
-// thread calls it after its outputs are written.
+// Whether x or the leading n x n block of A or B holds a value that is not
+// finite in T; every thread of the CTA calls it.
 template <typename T, typename IO>
-__device__ __noinline__ void fp_dense_points(const FpTile<T, IO> t, IO *out, bool wide)
+__device__ __forceinline__ bool fp_poison(const FpArgs &a, const IO *x, int n)
+{
+    bool p = false;
+    for (int l = threadIdx.x; l < n; l += blockDim.x) p |= not_finite((T)x[l]);
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+        const size_t at = (size_t)(e / n) * a.ld + e % n;
+        p |= not_finite((T)a.A[at]) || not_finite((T)a.B[at]);
+    }
+    return __syncthreads_or(p);
+}
+
+// r_m of every m from the staged sin and cos; every thread calls it.
+template <typename T>
+__device__ __forceinline__ void fp_residuals(const FpArgs &a, const double *E, int n, const double *zs,
+                                             const double *zc, T *r)
+{
+    for (int m = threadIdx.x; m < n; m += blockDim.x) {
+        double s = 0.0;
+        for (int j = 0; j < n; ++j) s = fma(a.A[(size_t)m * a.ld + j], zs[j], fma(a.B[(size_t)m * a.ld + j], zc[j], s));
+        r[m] = (T)(E[m] - s);
+    }
+    __syncthreads();
+}
+
+// Points whose fast result is not finite, evaluated densely by the CTA; every
+// thread calls it after its outputs are written.  The dense HVP of n >=
+// wide_from variables adds its rows in FP64.
+template <typename T, typename IO>
+__device__ __noinline__ void fp_dense_points(const FpTile<T, IO, true> t, IO *out, int wide_from)
 {
     for (int q = 0; q < t.P; ++q) {
         const int n = t.ns[q], z0 = t.base[q];
-        bool bad = false, poison = false;
-        for (int l = threadIdx.x; l < n; l += kFpThreads) {
-            bad |= not_finite((T)out[t.xoff[q] + l]);
-            poison |= not_finite((T)t.x[t.xoff[q] + l]);
-        }
+        IO *o = out + t.xoff[q];
+        bool bad = false;
+        for (int l = threadIdx.x; l < n; l += kFpThreads) bad |= not_finite((T)o[l]);
         if (!__syncthreads_or(bad)) continue;
-        for (int e = threadIdx.x; e < n * n; e += kFpThreads) {
-            const size_t at = (size_t)(e / n) * t.a.ld + e % n;
-            poison |= not_finite((T)t.a.A[at]) || not_finite((T)t.a.B[at]);
-        }
-        poison = __syncthreads_or(poison);
-        // the residuals, again: with the rows split over CTAs rr holds a part
-        for (int m = threadIdx.x; m < n; m += kFpThreads) {
-            double s = 0.0;
-            for (int j = 0; j < n; ++j)
-                s = fma(t.a.A[(size_t)m * t.a.ld + j], t.zs[z0 + j], fma(t.a.B[(size_t)m * t.a.ld + j], t.zc[z0 + j], s));
-            t.rr[z0 + m] = (T)(t.a.E[t.eoff[q] + m] - s);
-        }
-        __syncthreads();
-        const IO *v = t.v + t.xoff[q];
+        const bool poison = fp_poison<T>(t.a, t.x + t.xoff[q], n);
+        fp_residuals<T>(t.a, t.a.E + t.eoff[q], n, t.zs + z0, t.zc + z0, t.rr + z0);
+        const FpDense<T> d{t.a.A, t.a.B, t.a.ld, n, t.zs + z0, t.zc + z0, t.rr + z0, poison};
         for (int s = threadIdx.x; s < n; s += kFpThreads)
-            out[t.xoff[q] + s] =
-                (IO)dense_row<T>(v, n, s, wide, [&](int i, int j) { return t.dense_entry(q, poison, i, j); });
+            o[s] = (IO)dense_row<T>(t.v + t.xoff[q], n, s, n >= wide_from, [&](int i, int j) { return d.entry(i, j); });
         __syncthreads();
     }
+}
+
+// ------------------------------------------------------------------ Hessians
+// e / n for 0 <= e < 2^32 / n: a multiplication by magic = floor(2^32 / n) + 1
+// (n = 1: magic 0).
+struct FastDiv {
+    unsigned magic;
+    __device__ __forceinline__ int div(int e) const { return magic ? (int)__umulhi((unsigned)e, magic) : e; }
+};
+
+// The elements of `rows` consecutive Hessian rows of n, out[r n + j] =
+// val(r, j), with 16-byte streaming stores where the address allows.  Every
+// thread of the CTA calls it.
+template <typename IO, typename F>
+__device__ __forceinline__ void stream_rows(IO *out, int rows, int n, FastDiv fd, F &&val)
+{
+    using Vec = typename std::conditional<sizeof(IO) == 8, double2, float4>::type;
+    constexpr int V = 16 / (int)sizeof(IO);
+    const int cnt = rows * n;
+    const int mis = (int)(((16 - ((size_t)out & 15)) & 15) / sizeof(IO));
+    const int head = mis < cnt ? mis : cnt, nvec = (cnt - head) / V;
+    auto one = [&](int e) {
+        const int r = fd.div(e);
+        out[e] = (IO)val(r, e - r * n);
+    };
+    for (int e = threadIdx.x; e < head; e += blockDim.x) one(e);
+    for (int w = threadIdx.x; w < nvec; w += blockDim.x) {
+        const int e = head + w * V;
+        int r = fd.div(e), j = e - r * n;
+        IO q[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            q[i] = (IO)val(r, j);
+            if (++j == n) {
+                j = 0;
+                ++r;
+            }
+        }
+        Vec o;
+        if constexpr (V == 2) {
+            o.x = q[0];
+            o.y = q[1];
+        } else {
+            o.x = q[0];
+            o.y = q[1];
+            o.z = q[2];
+            o.w = q[3];
+        }
+        __stcs(reinterpret_cast<Vec *>(out + e), o);
+    }
+    for (int e = head + nvec * V + threadIdx.x; e < cnt; e += blockDim.x) one(e);
+}
+
+// The Hessian rows [r0, r1) of one point by the dense propagation; the CTA's
+// threads take whole rows.
+template <typename T, typename IO>
+__device__ __noinline__ void ros_dense_rows(const IO *x, IO *H, int n, int r0, int r1)
+{
+    const RosBad b = ros_bad<T>(x, n);
+    for (int i = r0 + (int)threadIdx.x; i < r1; i += blockDim.x)
+        for (int j = 0; j < n; ++j) H[(size_t)i * n + j] = (IO)ros_dense_entry<T>(x, n, b, i, j);
+}
+template <typename T, typename IO>
+__device__ __noinline__ void ack_dense_rows(const IO *x, IO *H, int n, int r0, int r1)
+{
+    const AckDense<T, IO> d(x, n);
+    for (int i = r0 + (int)threadIdx.x; i < r1; i += blockDim.x)
+        for (int j = 0; j < n; ++j) H[(size_t)i * n + j] = (IO)d.entry(i, j);
+}
+// zs, zc, r: shared scratch of n elements each
+template <typename T, typename IO>
+__device__ __noinline__ void fp_dense_hessian(const FpArgs a, const IO *x, IO *H, int n, double *zs, double *zc, T *r)
+{
+    __syncthreads();
+    for (int l = threadIdx.x; l < n; l += blockDim.x) sincos((double)x[l], &zs[l], &zc[l]);
+    const bool poison = fp_poison<T>(a, x, n);
+    fp_residuals<T>(a, a.E, n, zs, zc, r);
+    const FpDense<T> d{a.A, a.B, a.ld, n, zs, zc, r, poison};
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) H[e] = (IO)d.entry(e / n, e % n);
+    __syncthreads();
+}
+
+// Fletcher-Powell, f_ij = 2 sum_m J_mi J_mj (+ the curvature on the diagonal):
+// a 4 x 4 block of one point's products J^T J in registers, compensated FP32 as
+// blocked Sum2 (plain FMAs over kSumBlock rows, then TwoSum), as the dense
+// sweep's sum over terms.
+template <typename T>
+struct Gram4;
+template <>
+struct Gram4<double> {
+    double s[4][4];
+    __device__ __forceinline__ void init()
+    {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) s[i / 4][i % 4] = 0.0;
+    }
+    __device__ __forceinline__ void add(const double *p, const double *q)
+    {
+        double u[4], w[4];
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            const double2 a = *reinterpret_cast<const double2 *>(p + i), b = *reinterpret_cast<const double2 *>(q + i);
+            u[i] = a.x;
+            u[i + 1] = a.y;
+            w[i] = b.x;
+            w[i + 1] = b.y;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] = __fma_rn(u[i], w[j], s[i][j]);
+    }
+    __device__ __forceinline__ void flush() {}
+    __device__ __forceinline__ double value(int i, int j) const { return 2.0 * s[i][j]; }
+};
+template <>
+struct Gram4<float> {
+    CSum s[4][4];
+    float p[4][4];
+    __device__ __forceinline__ void init()
+    {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            s[i / 4][i % 4] = CSum{0.f, 0.f};
+            p[i / 4][i % 4] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void add(const float *a, const float *b)
+    {
+        const float4 x = *reinterpret_cast<const float4 *>(a), y = *reinterpret_cast<const float4 *>(b);
+        const float u[4] = {x.x, x.y, x.z, x.w};
+        const float w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) vfma(u[i], w, p[i]);
+    }
+    __device__ __forceinline__ void flush()
+    {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                csum_add(s[i][j], p[i][j]);
+                p[i][j] = 0.f;
+            }
+    }
+    __device__ __forceinline__ float value(int i, int j) const { return 2.0f * csum_value(s[i][j]); }
+};
+
+// J_mj = A_mj cos x_j - B_mj sin x_j, as the dense sweep rounds it
+template <typename T>
+__device__ __forceinline__ T fp_jacobian(T a, T b, T s, T c)
+{
+    return fma_(b, -s, a * c);
 }
 
 }  // namespace chessfad

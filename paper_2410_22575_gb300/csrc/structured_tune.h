@@ -1,0 +1,66 @@
+// structured_tune.h -- host-side shapes of the structured kernels, shared by
+// the contiguous launches (structured.cu) and the uneven-batch plan
+// (ragged_structured.cu).
+#pragma once
+
+#include <algorithm>
+
+#include "structured.cuh"
+
+namespace chessfad {
+
+inline int pow2_ceil(int v)
+{
+    int p = 1;
+    while (p < v) p <<= 1;
+    return p;
+}
+
+// Lanes per point of the Rosenbrock kernel: about four variables per lane
+// (independent loads in flight), at least 8 lanes where n has them (a warp's
+// loads then cover whole 32-byte sectors).
+inline int ros_lanes(int n)
+{
+    return std::min(32, std::max(pow2_ceil((n + 3) / 4), std::min(8, pow2_ceil(n))));
+}
+
+// Lanes per point of the Ackley kernel.  Each lane pays for the cross-lane
+// sums and the tail's scalar functions about as much as for `over` variables,
+// so few lanes with many variables each (at most 16) do least work; a batch
+// too small to fill the GPU that way takes more lanes.
+inline int ack_lanes(int n, long long batch, bool f64)
+{
+    const double over = f64 ? 2.0 : 1.0;
+    int best = 1;
+    double best_cost = 1e300;
+    for (int g = 1; g <= 32; g <<= 1) {
+        const int it = (n + g - 1) / g;
+        if (it > 16 || (g > 1 && g >= 2 * n) || (!f64 && g < 8 && it > 1)) continue;
+        const double waves = std::max(1.0, (double)batch * g / (152.0 * 512.0));
+        const double cost = (it + over) * waves;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = g;
+        }
+    }
+    return best;
+}
+
+// Rows of A and B per tile: all of them within 64 KiB (two or more CTAs per
+// SM hide the barriers between the passes), else even parts of the rows.
+template <typename T>
+inline FpShape fp_shape(int nmax, int rows, int P)
+{
+    const size_t row = (size_t)fp_stride(nmax) * 2 * (sizeof(double) + (sizeof(T) == 4 ? sizeof(float) : 0));
+    const int most = std::max(1, (int)(64 * 1024 / row));
+    const int tiles = (rows + most - 1) / most;
+    FpShape s;
+    s.nmax = nmax;
+    s.mt = (rows + tiles - 1) / tiles;
+    // pass 1: enough lanes per (point, row) to occupy the CTA's threads
+    s.lanes = 1;
+    while (s.lanes < 32 && s.lanes < nmax && P * s.mt * s.lanes < kFpThreads) s.lanes <<= 1;
+    return s;
+}
+
+}  // namespace chessfad

@@ -9,7 +9,7 @@ import pytest
 import paper_2410_22575_gb300 as cf
 from paper_2410_22575_gb300 import workloads as W
 
-from gpu_helpers import BOUND, Dev, hvp_err
+from gpu_helpers import BOUND, Dev, hessian_err, hvp_err
 
 pytestmark = pytest.mark.gpu
 
@@ -28,6 +28,20 @@ def test_hvp_sizes(fn, prec, n, batch):
     e = hvp_err(d, out)
     assert e.max() <= BOUND[prec], (e.max(), np.median(e))
     assert np.array_equal(out, d.hvp())
+
+
+@pytest.mark.parametrize("fn", FNS)
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("n,batch", [(1, 700), (2, 1), (2, 3001), (3, 257), (4, 130), (7, 600), (16, 5), (17, 77),
+                                     (33, 40), (63, 7), (64, 30), (65, 9), (127, 5), (128, 2), (129, 3), (200, 3),
+                                     (511, 1), (512, 1)])
+def test_hessian_sizes(fn, prec, n, batch):
+    d = Dev(W.make_batch(fn, n, batch, seed=3000 + n), prec)
+    H = d.hessian()
+    e = hessian_err(d, H)
+    assert e.max() <= BOUND[prec], (e.max(), np.median(e))
+    assert np.array_equal(H, np.swapaxes(H, 1, 2))
+    assert np.array_equal(H, d.hessian())
 
 
 def _same(a, b, bound, scale):
@@ -71,6 +85,11 @@ def test_non_finite_points_equal_the_dense_method(fn, prec, n):
     scale = np.max(np.abs(np.where(fine, dense, 0.0)), axis=1, keepdims=True) * np.ones_like(dense)
     tol = 4e-12 if prec == cf.FP64 else 4e-5
     _same(got, dense, tol, scale[fine])
+    dense = d.hessian(cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 0) if n >= 4 else cf.Config(2, 1, 256))
+    got = d.hessian()
+    fine = np.isfinite(dense)
+    scale = np.max(np.abs(np.where(fine, dense, 0.0)), axis=(1, 2), keepdims=True) * np.ones_like(dense)
+    _same(got, dense, tol, scale[fine])
 
 
 @pytest.mark.parametrize("prec", PRECS)
@@ -83,6 +102,9 @@ def test_non_finite_parameters_equal_the_dense_method(prec):
         d = Dev(b, prec)
         dense = d.hvp(cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 0))
         assert np.array_equal(np.isnan(d.hvp()), np.isnan(dense)) and np.all(~np.isfinite(dense))
+        Hd, H = d.hessian(cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 0)), d.hessian()
+        assert np.array_equal(np.isnan(H), np.isnan(Hd))
+        assert np.array_equal(np.isinf(H), np.isinf(Hd)) and np.all(~np.isfinite(Hd))
 
 
 @pytest.mark.parametrize("fn", FNS)
@@ -103,3 +125,87 @@ def test_points_are_independent(fn):
     view.copy_(d.x)
     out = cf.hvp(fn, view, d.v, params=d.params)
     assert np.array_equal(out.cpu().numpy(), a, equal_nan=True)
+    assert np.array_equal(dp.hessian(), d.hessian()[perm], equal_nan=True)
+    Hflat = torch.empty(300 * 19 * 19 + 1, dtype=torch.float64, device="cuda")
+    Hv = cf.hessian(fn, view, params=d.params, out=Hflat[1:].view(300, 19, 19))
+    assert np.array_equal(Hv.cpu().numpy(), d.hessian(), equal_nan=True)
+
+
+class _Uneven:
+    """An uneven batch of the given functions and sizes and its plan (csize 0)."""
+
+    def __init__(self, fns, ns, prec, seed=3):
+        import torch
+
+        self.fns, self.ns, self.prec = np.asarray(fns, np.int32), np.asarray(ns, np.int32), prec
+        rng = np.random.Generator(np.random.PCG64(seed))
+        self.fp = W.draw_fp_instance(rng, int(self.ns.max()))
+        self.offs = np.concatenate([[0], np.cumsum(self.ns[:-1], dtype=np.int64)])
+        x = np.concatenate([rng.uniform(*W.X_RANGE[int(f)], int(n)) for f, n in zip(fns, ns)])
+        v = rng.uniform(-1, 1, int(self.ns.sum()))
+        first, E, pos = {}, [], 0
+        for n in sorted(set(self.ns.tolist())):
+            E.append(W.fp_rhs(self.fp.A[:n, :n], self.fp.B[:n, :n], self.fp.alpha[:n]))
+            first[n], pos = pos, pos + n
+        self.eoffs = np.array([first[int(n)] for n in self.ns], np.int64)
+        self.Epack = np.concatenate(E)
+        dt = torch.float64 if prec == cf.FP64 else torch.float32
+        self.x, self.v = torch.tensor(x, dtype=dt, device="cuda"), torch.tensor(v, dtype=dt, device="cuda")
+        self.keep = [torch.tensor(t, device="cuda") for t in (self.fp.A, self.fp.B, self.Epack)]
+        self.params = cf.fp_params(*self.keep)
+
+    def reqs(self):
+        return cf.requests(self.fns, self.ns, self.offs, self.eoffs)
+
+    def run(self, csize=0):
+        import torch
+
+        plan = cf.RaggedPlan(self.reqs(), self.prec, csize)
+        out = torch.full_like(self.x, 7.0)
+        plan.run(self.x, self.v, out, self.params)
+        torch.cuda.synchronize()
+        first = out.double().cpu().numpy()
+        plan.run(self.x, self.v, out, self.params)
+        torch.cuda.synchronize()
+        assert np.array_equal(first, out.double().cpu().numpy(), equal_nan=True)
+        return first
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_uneven_batch_tiles(prec):
+    """Requests at the edges of the tiles: one variable, groups that end inside
+    a tile, sizes that differ by more than a tile may mix, a few large
+    Fletcher-Powell requests that are split over tiles; every request against
+    the oracle, and a second run equal bit for bit."""
+    import oracle
+    from paper_2410_22575_gb300 import metrics
+
+    F, R, A = W.FLETCHER_POWELL, W.ROSENBROCK, W.ACKLEY
+    sizes = [1, 1, 2, 3, 5, 8, 9, 16, 17, 31, 32, 33, 64, 65, 100, 127, 128, 129, 200, 256, 257, 300, 511, 512]
+    fns, ns = [], []
+    for k, n in enumerate(sizes):
+        for f in (F, R, A):
+            fns += [f] * (1 + (k * 7 + f) % 3)
+            ns += [n] * (1 + (k * 7 + f) % 3)
+    order = np.random.Generator(np.random.PCG64(1)).permutation(len(ns))
+    u = _Uneven(np.array(fns)[order], np.array(ns)[order], prec)
+    got = u.run()
+    xh, vh = u.x.double().cpu().numpy(), u.v.double().cpu().numpy()
+    ref, hn = oracle.hvp_ragged(u.fns, u.ns, u.offs, u.eoffs, xh, vh, u.fp.A, u.fp.B, u.Epack, u.fp.A.shape[1])
+    e = metrics.ragged_hvp_errors(got, ref, hn, vh, u.ns, u.offs)
+    assert e.max() <= BOUND[prec], (e.max(), np.median(e))
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_uneven_non_finite_requests_equal_the_dense_evaluation(prec):
+    F, R, A = W.FLETCHER_POWELL, W.ROSENBROCK, W.ACKLEY
+    fns = [F, R, A] * 8
+    ns = [1] * 3 + [5] * 6 + [40] * 6 + [140] * 9
+    u = _Uneven(fns, ns, prec)
+    for k in range(0, 24, 2):
+        t = u.x if k % 4 else u.v
+        t[int(u.offs[k]) + u.ns[k] // 2] = (np.nan, np.inf, -np.inf)[k % 3]
+    dense, got = u.run(8), u.run()
+    fine = np.isfinite(dense)
+    _same(got, dense, 4e-12 if prec == cf.FP64 else 4e-5, np.repeat(
+        [np.max(np.abs(np.where(fine, dense, 0.0)[o:o + n]), initial=1.0) for o, n in zip(u.offs, u.ns)], u.ns)[fine])
