@@ -342,12 +342,10 @@ typedef struct chessfad_ragged_plan_s *chessfad_ragged_plan;
 
 /* Build a plan (host memory, owned by the caller until
  * chessfad_ragged_plan_destroy) from a host array of nreq requests for
- * precision prec.  csize 8 or 16: every (function, n) group uses that chunk
- * size and the default lanes per row; csize 0: each group takes the chunk
- * size and lanes per row that chessfad_ragged_autotune stored for its
- * (precision, function, n range), else the defaults (chunk 16 for compensated
- * FP32, 8 for FP64; lanes per row min(32, pow2_floor(ceil(n/C) / 8))).  The
- * n ranges are the powers of two, 2^b <= n < 2^(b+1) (n = 512 with 256..511).
+ * precision prec.  csize 8 or 16: the dense chunked evaluation, every
+ * (function, n) group with that chunk size and the default lanes per row;
+ * csize 0: the structured evaluation (see conventions), the same results to
+ * rounding.
  * Validates every request: CHESSFAD_ERR_FUNCTION / _SIZE for a bad fn or n,
  * CHESSFAD_ERR_PLAN for a negative offset.  Launches nothing. */
 CHESSFAD_API int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, int prec, int csize,
@@ -355,21 +353,28 @@ CHESSFAD_API int chessfad_ragged_plan_create(const chessfad_request *reqs, long 
 CHESSFAD_API int chessfad_ragged_plan_destroy(chessfad_ragged_plan plan);
 
 /* Device workspace bytes the plan needs (tile table, request list, offsets,
- * the queue counter, a tile counter per request and, for the Fletcher-Powell
- * requests with n >= 128, one FP64 partial row vector per tile), the number
+ * the queue counter, tile counters and, for the Fletcher-Powell requests
+ * whose work is split over tiles, FP64 partial sums per tile), the number
  * of tiles and the dynamic shared memory per CTA.  Any pointer may be NULL. */
 CHESSFAD_API int chessfad_ragged_plan_info(chessfad_ragged_plan plan, size_t *workspace_bytes, long long *ntiles,
                                            size_t *smem_bytes);
 
 /* The chunk size, lanes per row and Fletcher-Powell A/B tile height (rows of
- * A and B staged per shared-memory tile; 8 for the other functions) the plan
- * uses for requests of function fn and size n (CHESSFAD_ERR_SIZE if it holds
- * no such request).  Any output pointer may be NULL.  Host only. */
+ * A and B staged per shared-memory tile; 8 for the other functions) of the
+ * dense evaluation of the plan's requests of function fn and size n
+ * (CHESSFAD_ERR_SIZE if it holds no such request): the plan's chunk size and
+ * the default lanes per row, or, for a plan of csize 0, the chunk size and
+ * lanes that chessfad_ragged_autotune stored for the (precision, function, n
+ * range), else the defaults (chunk 16 for compensated FP32, 8 for FP64; lanes
+ * per row min(32, pow2_floor(ceil(n/C) / 8))).  The n ranges are the powers
+ * of two, 2^b <= n < 2^(b+1) (n = 512 with 256..511).  Any output pointer may
+ * be NULL.  Host only. */
 CHESSFAD_API int chessfad_ragged_plan_group_config(chessfad_ragged_plan plan, int fn, int n, int *csize,
                                                    int *threads_per_row, int *tile_rows);
 
-/* Autotune the uneven batch: for every (function, n range) group of the
- * requests (ranges as for chessfad_ragged_plan_create), run the persistent
+/* Autotune the dense evaluation of the uneven batch: for every (function, n
+ * range) group of the requests (ranges as for
+ * chessfad_ragged_plan_group_config), run the persistent
  * kernel on a sample of the group's requests (in table order, enough rows to
  * fill the GPU about four times) for every chunk size (16, 8), lanes per
  * row (1 .. 32; for the symmetric Fletcher-Powell tiles, whose (row, chunk)
@@ -380,8 +385,7 @@ CHESSFAD_API int chessfad_ragged_plan_group_config(chessfad_ragged_plan plan, in
  * measuring the SM cycles its tiles take, summed over the CTAs (the group's
  * throughput inside a large mixed run, free of the small sample's own tail),
  * and store the cheapest per (prec, function, n range) in the process-wide
- * table
- * that chessfad_ragged_plan_create(..., csize = 0, ...) reads.  xpack, vpack,
+ * table that chessfad_ragged_plan_group_config reports from.  xpack, vpack,
  * outpack, params as for chessfad_hvp_ragged (outpack of the sampled requests
  * is overwritten); workspace: device scratch of workspace_bytes (candidates
  * whose trial plan needs more, plus 256 bytes for the cycle counter, are
@@ -407,13 +411,14 @@ CHESSFAD_API int chessfad_ragged_plan_upload(chessfad_ragged_plan plan, void *wo
 /* Run the plan: reset the queue counter and the per-request tile counters in
  * the workspace (one cudaMemsetAsync) and launch one persistent kernel, both
  * on stream; no host synchronisation, no allocation, so the call can be
- * captured into a CUDA graph and replayed.  Fletcher-Powell requests with
- * n >= 128 use the symmetric method (SC-HESS-VEC, Alg. 8; about half the
- * evaluations): each entry right of a row's diagonal chunk also updates the
+ * captured into a CUDA graph and replayed.  In the dense evaluation,
+ * Fletcher-Powell requests with n >= 128 use the symmetric method
+ * (SC-HESS-VEC, Alg. 8; about half the evaluations): each entry right of a row's diagonal chunk also updates the
  * row it mirrors, usually in another tile; every tile adds its rows'
  * contributions in a fixed order into a partial row vector of its own (FP64)
  * and the tile that completes a request adds the request's partial vectors
- * in tile order, so every result is bitwise reproducible from run to run.
+ * in tile order; the structured evaluation's split requests are added the
+ * same way.  Every result is bitwise reproducible from run to run.
  * xpack, vpack, outpack: device, float (FP32_COMP) or double (FP64) by the
  * plan's precision.  params: required when the plan holds Fletcher-Powell
  * requests (ld >= their largest n).  Runs that share a workspace must not

@@ -9,7 +9,10 @@
 // ones fill the tail.  The chunk size and the lanes per row are chosen per
 // (function, n range): from the table chessfad_ragged_autotune fills, else by
 // default.  The tables (tiles, request list, offsets) live in a
-// caller-provided device workspace together with a queue counter.
+// caller-provided device workspace together with a queue counter.  That is
+// the dense chunked evaluation, of a plan built with a chunk size; a plan
+// built without one is evaluated structurally (ragged_structured.cu), with
+// the same workspace, counter and launch scheme.
 //
 // Device side: a persistent kernel, a few CTAs per SM, whose CTAs take tile
 // after tile from the counter with atomicAdd and run the tile's sweeps.  No
@@ -43,6 +46,7 @@
 
 #include "../../include/chessfad.h"
 #include "dispatch.h"
+#include "structured.h"
 
 namespace chessfad {
 
@@ -311,6 +315,11 @@ struct chessfad_ragged_plan_s {
     std::vector<int> list;
     std::vector<long long> offs, eoffs, soffs;
     long long slot_elems = 0;  // FP64 partial rows of the symmetric tiles
+    // csize 0: the structured evaluation's tiles in place of the dense ones,
+    // and one dense tile per group for chessfad_ragged_plan_group_config
+    bool structured = false;
+    SPlan sp;
+    size_t off_n = 0, off_base = 0;
     // device workspace layout (bytes): tables (uploaded), then the queue
     // counter and the per-request tile counters (zeroed every run), then the
     // symmetric tiles' slots (written before they are read)
@@ -402,6 +411,34 @@ struct PlanOptions {
     const std::map<std::pair<int, int>, GroupCfg> *force = nullptr;  // (fn, bucket) -> forced config
 };
 
+// Workspace of a structured plan: tiles | off | eoff | n | base (the tables),
+// then counter | done (zeroed by every run), then the slots.
+int layout_structured(chessfad_ragged_plan_s *pl)
+{
+    const SPlan &sp = pl->sp;
+    const size_t nreq = sp.n.size();
+    if (sp.tiles.size() > (size_t)0x7fffffff) return CHESSFAD_ERR_BATCH;
+    pl->smem = sp.smem;
+    pl->off_tiles = 0;
+    pl->off_offs = align256(sp.tiles.size() * sizeof(STile));
+    pl->off_eoffs = align256(pl->off_offs + nreq * sizeof(long long));
+    pl->off_n = align256(pl->off_eoffs + nreq * sizeof(long long));
+    pl->off_base = align256(pl->off_n + nreq * sizeof(int));
+    pl->table_bytes = align256(pl->off_base + nreq * sizeof(int));
+    pl->off_counter = pl->table_bytes;
+    pl->off_done = align256(pl->off_counter + sizeof(int));
+    pl->off_slots = align256(pl->off_done + (size_t)sp.ndone * sizeof(int));
+    pl->total = align256(pl->off_slots + (size_t)sp.slot_elems * sizeof(double));
+    pl->image.assign(pl->table_bytes, 0);
+    if (nreq == 0) return CHESSFAD_SUCCESS;
+    std::memcpy(&pl->image[pl->off_tiles], sp.tiles.data(), sp.tiles.size() * sizeof(STile));
+    std::memcpy(&pl->image[pl->off_offs], sp.off.data(), nreq * sizeof(long long));
+    std::memcpy(&pl->image[pl->off_eoffs], sp.eoff.data(), nreq * sizeof(long long));
+    std::memcpy(&pl->image[pl->off_n], sp.n.data(), nreq * sizeof(int));
+    std::memcpy(&pl->image[pl->off_base], sp.base.data(), nreq * sizeof(int));
+    return CHESSFAD_SUCCESS;
+}
+
 int build_plan(const chessfad_request *reqs, long long nreq, int prec, const PlanOptions &opt,
                chessfad_ragged_plan_s *pl)
 {
@@ -422,6 +459,7 @@ int build_plan(const chessfad_request *reqs, long long nreq, int prec, const Pla
     }
     std::vector<std::pair<double, RTile>> work;
     size_t smem = 0;
+    pl->structured = opt.csize == 0 && !opt.force;
     for (auto &g : groups) {
         const int fn = g.first.first, n = g.first.second;
         GroupCfg gc;
@@ -445,6 +483,16 @@ int build_plan(const chessfad_request *reqs, long long nreq, int prec, const Pla
         const size_t ab = (size_t)(gc.ab_kib ? gc.ab_kib : kAbDefaultKiB) * 1024;
         const int mt = (fn == CHESSFAD_FLETCHER_POWELL) ? fp_tile_rows_ragged(n, prec, (C == 1) ? 8 : mb, ab) : 8;
         if (fn == CHESSFAD_FLETCHER_POWELL) pl->max_fp_n = std::max(pl->max_fp_n, n);
+        if (pl->structured) {
+            RTile t{};
+            t.fn = fn;
+            t.n = n;
+            t.C = C;
+            t.tpr = fn == CHESSFAD_FLETCHER_POWELL && n >= kSymMinN ? sym_tpr(tpr, n) : tpr;
+            t.mt = mt;
+            pl->tiles.push_back(t);
+            continue;
+        }
         const bool f64sweep = (prec == CHESSFAD_FP64) || n == 1;
         const size_t bytes = f64sweep ? smem_layout<double>(fn, true, n, maxpts, mt).total
                                       : smem_layout<float>(fn, true, n, maxpts, mt).total;
@@ -512,6 +560,10 @@ int build_plan(const chessfad_request *reqs, long long nreq, int prec, const Pla
             work.push_back({cost, t});
             pl->est_cost += cost;
         }
+    }
+    if (pl->structured) {
+        structured_plan(reqs, nreq, prec, pl->sp);
+        return layout_structured(pl);
     }
     if (work.size() > (size_t)0x7fffffff) return CHESSFAD_ERR_BATCH;
     std::stable_sort(work.begin(), work.end(),
@@ -591,6 +643,44 @@ cudaError_t launch_ragged(chessfad_ragged_plan_s *pl, const RaggedArgs &a, cudaS
     return cudaGetLastError();
 }
 
+int run_structured(chessfad_ragged_plan_s *plan, unsigned char *ws, const void *xpack, const void *vpack,
+                   void *outpack, const chessfad_fp_params *params, cudaStream_t stream)
+{
+    SRaggedArgs a{};
+    a.x = xpack;
+    a.v = vpack;
+    a.out = outpack;
+    if (params) {
+        a.A = params->A;
+        a.B = params->B;
+        a.Epack = params->E;
+        a.ld = params->ld;
+    }
+    a.ntiles = (int)plan->sp.tiles.size();
+    a.tiles = reinterpret_cast<const STile *>(ws + plan->off_tiles);
+    a.off = reinterpret_cast<const long long *>(ws + plan->off_offs);
+    a.eoff = reinterpret_cast<const long long *>(ws + plan->off_eoffs);
+    a.n = reinterpret_cast<const int *>(ws + plan->off_n);
+    a.base = reinterpret_cast<const int *>(ws + plan->off_base);
+    a.counter = reinterpret_cast<int *>(ws + plan->off_counter);
+    a.done = reinterpret_cast<int *>(ws + plan->off_done);
+    a.slots = reinterpret_cast<double *>(ws + plan->off_slots);
+    const bool f64 = plan->prec == CHESSFAD_FP64;
+    int dev = 0, grid = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return CHESSFAD_ERR_CUDA;
+    {
+        std::lock_guard<std::mutex> lk(plan->mu);
+        if (plan->grid_dev != dev) {
+            if (structured_ragged_grid(f64, plan->smem, &plan->grid) != cudaSuccess) return CHESSFAD_ERR_CUDA;
+            plan->grid_dev = dev;
+        }
+        grid = plan->grid;
+    }
+    if (cudaMemsetAsync(a.counter, 0, plan->off_slots - plan->off_counter, stream) != cudaSuccess)
+        return CHESSFAD_ERR_CUDA;
+    return structured_ragged(f64, a, plan->smem, grid, stream) == cudaSuccess ? CHESSFAD_SUCCESS : CHESSFAD_ERR_CUDA;
+}
+
 RaggedArgs ragged_args(const chessfad_ragged_plan_s *plan, unsigned char *ws, const void *xpack, const void *vpack,
                        void *outpack, const chessfad_fp_params *params)
 {
@@ -619,6 +709,7 @@ RaggedArgs ragged_args(const chessfad_ragged_plan_s *plan, unsigned char *ws, co
 int run_plan(chessfad_ragged_plan_s *plan, unsigned char *ws, const void *xpack, const void *vpack, void *outpack,
              const chessfad_fp_params *params, cudaStream_t s, unsigned long long *busy = nullptr)
 {
+    if (plan->structured) return run_structured(plan, ws, xpack, vpack, outpack, params, s);
     RaggedArgs a = ragged_args(plan, ws, xpack, vpack, outpack, params);
     a.busy = busy;
     const cudaError_t e =
@@ -672,7 +763,7 @@ int chessfad_ragged_plan_info(chessfad_ragged_plan plan, size_t *workspace_bytes
 {
     if (!plan) return CHESSFAD_ERR_PLAN;
     if (workspace_bytes) *workspace_bytes = plan->total;
-    if (ntiles) *ntiles = (long long)plan->tiles.size();
+    if (ntiles) *ntiles = (long long)(plan->structured ? plan->sp.tiles.size() : plan->tiles.size());
     if (smem_bytes) *smem_bytes = plan->smem;
     return CHESSFAD_SUCCESS;
 }
