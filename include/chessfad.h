@@ -487,12 +487,15 @@ CHESSFAD_API int chessfad_version(void);
  * +1, and a comparison of values (the branch taken is differentiated as it
  * stands).  params is the caller's device pointer, passed through (may be
  * NULL).  The arithmetic of f runs in the handle's precision: FP64, or FP32
- * (CHESSFAD_FP32_COMP: only the row-times-v reduction is compensated; the
- * function's own sums are plain FP32 as written; at n = 1, where the Hessian
+ * (CHESSFAD_FP32_COMP: the function's own sums are plain FP32 as written; the
+ * plain and symmetric methods' row-times-v reduction is compensated, the
+ * default HVP has none; at n = 1, where the Hessian
  * is one entry whose terms can cancel, the arithmetic is FP64 with float
  * inputs and outputs).
  *
- * Two decompositions, as for the built-in functions: plain (CHESS-VEC,
+ * The default HVP evaluates f once per chunk with d1 seeded by v, so that the
+ * h components are the chunk's rows of H v.  Two decompositions by rows, as for
+ * the built-in functions: plain (CHESS-VEC,
  * Alg. 7 / CHUNK-HESS, Alg. 5: one thread per (point, Hessian row), sweeping
  * the row's ceil(n/csize) chunks) and symmetric (SC-HESS-VEC, Alg. 8 /
  * SCHUNK-HESS, Alg. 6: threads_per_point threads share a point's (row, chunk
@@ -524,9 +527,10 @@ CHESSFAD_API int chessfad_user_fn_info(const chessfad_user_fn *fn, int hvp, int 
                                        int *local_bytes);
 
 /* out[p] = H(x_p) v_p for the user's f, p < batch; types by the handle's
- * precision (double, or float for CHESSFAD_FP32_COMP), by the symmetric
- * method with 32 threads per point.  Asynchronous on `stream`; allocates nothing.  The first symmetric
- * launch on a device that needs more than 48 KiB of shared memory raises the
+ * precision (double, or float for CHESSFAD_FP32_COMP): one evaluation of f
+ * per chunk with d1 seeded by v (rows that are not finite, and points whose v
+ * is not, by the plain method).  Asynchronous on `stream`; allocates nothing.
+ * The first symmetric launch on a device that needs more than 48 KiB of shared memory raises the
  * kernel's limit (a host call; make it before capturing a CUDA graph). */
 CHESSFAD_API int chessfad_user_hvp(chessfad_user_fn *fn, int n, long long batch, const void *x, const void *v,
                                    void *out, const double *params, chessfad_stream_t stream);
@@ -538,7 +542,8 @@ CHESSFAD_API int chessfad_user_hessian(chessfad_user_fn *fn, int n, long long ba
                                        const double *params, chessfad_stream_t stream);
 
 /* As chessfad_user_hvp / chessfad_user_hessian with an explicit
- * configuration (cfg may be NULL = the defaults above): csize 0 or the
+ * configuration (cfg may be NULL = the defaults above, and for a Hessian the
+ * symmetric method with 32 threads per point): csize 0 or the
  * handle's (else CHESSFAD_ERR_CHUNK); method CHESSFAD_METHOD_PLAIN or
  * _SYMMETRIC (else CHESSFAD_ERR_CONFIG); threads_per_row 0 or 1;
  * block_threads 0 (= 256) or 32..256, a multiple of 32; threads_per_point 0

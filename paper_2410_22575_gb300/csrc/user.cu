@@ -29,6 +29,7 @@ struct chessfad_user_fn {
     cudaKernel_t hessian = nullptr;      // plain (CHUNK-HESS, Alg. 5)
     cudaKernel_t sym_hvp = nullptr;      // symmetric (SC-HESS-VEC, Alg. 8)
     cudaKernel_t sym_hessian = nullptr;  // symmetric (SCHUNK-HESS, Alg. 6)
+    cudaKernel_t dir_hvp = nullptr;      // directional (the default HVP)
     cudaKernel_t hvp_n1 = nullptr;       // FP32 handles, n = 1: FP64 arithmetic, float I/O
     cudaKernel_t hessian_n1 = nullptr;
     int csize = 0;
@@ -212,6 +213,14 @@ int launch(chessfad_user_fn *fn, const chessfad_config *cfg, bool hvp, int n, lo
         block = (unsigned)b;
         smem = (size_t)args.maxpts * 2 * sizeof(double);
         k = hvp ? fn->hvp_n1 : fn->hessian_n1;
+    } else if (hvp && !cfg) {
+        // the default: one thread per (point, chunk); CTAs of 128, so that
+        // small batches reach more SMs
+        const long long nch = (n + fn->csize - 1) / fn->csize;
+        block = 128;
+        grid = (batch * nch + block - 1) / block;
+        smem = 0;
+        k = fn->dir_hvp;
     } else if (method == CHESSFAD_METHOD_SYMMETRIC) {
         grid = (batch + ppb - 1) / ppb;
         block = (unsigned)(ppb * tpp);
@@ -309,6 +318,7 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->hessian, fn->lib, "chessfad_user_hessian");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hvp, fn->lib, "chessfad_user_sym_hvp");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hessian, fn->lib, "chessfad_user_sym_hessian");
+    if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->dir_hvp, fn->lib, "chessfad_user_dir_hvp");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP) e = cudaLibraryGetKernel(&fn->hvp_n1, fn->lib, "chessfad_user_hvp_n1");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP)
         e = cudaLibraryGetKernel(&fn->hessian_n1, fn->lib, "chessfad_user_hessian_n1");

@@ -15,7 +15,11 @@
 //    floor(i/C)) are dealt round-robin to its threads.  The Hessian writes
 //    each chunk and its mirror image; the HVP stages the chunks in shared
 //    memory (compact upper-block layout) and, after one barrier, every thread
-//    sums whole rows, each off-diagonal-chunk entry serving both r_i and r_j.
+//    sums whole rows, each off-diagonal-chunk entry serving both r_i and r_j;
+//  directional (HVP, the default): one thread per (point, chunk), a single
+//    evaluation with d1 seeded by v gives the chunk's rows of H v (ceil(n/C)
+//    evaluations per point instead of n ceil(n/C)); rows that are not finite,
+//    and points whose v is not, are evaluated again by the plain method.
 // FP32: the row-times-v products are summed as a Dot2 (TwoProd by FMA plus
 // TwoSum); the function's own arithmetic is plain FP32, as written by the
 // user, except at n = 1 (FP64 arithmetic, float I/O).  FP64: fused
@@ -235,8 +239,61 @@ __device__ __forceinline__ void user_sym(const UserArgs &a)
     }
 }
 
+// Rows cstart .. cstart + C - 1 of H v by the plain method (Alg. 7).
+template <typename T, int C>
+__device__ __noinline__ void user_dense_rows(const T *xp, const T *vp, T *out, int n, int cstart, const double *params)
+{
+    const SeedK<T> z = seed_constants<T>();
+    for (int i = cstart; i < cstart + C && i < n; ++i) {
+        RowDot<T> dot;
+        for (int c0 = 0; c0 < n; c0 += C) {
+            const Vars<T, C> x{xp, i, c0, z};
+            const Num<T, C> r = ::CHESSFAD_USER_FN<Num<T, C>, Vars<T, C>>(x, n, params);
+#pragma unroll
+            for (int l = 0; l < C; ++l)
+                if (c0 + l < n) dot.add(r.a.h[l], vp[c0 + l]);
+        }
+        out[i] = dot.value();
+    }
+}
+
+// Bound by the arithmetic of f on 2C + 2 components (FP64 pipe or FMA issue);
+// x and v come from L1 (the lanes of a point read the same element).  The
+// extended-operator test function, n = 64, C = 8, FP64, 4096 points: symmetric
+// method 100.7 ms, here 2.83 ms.  Errors against the oracle (FP32, n = 19 and
+// 64, rms over the test functions): 1.0 to 1.24 times the symmetric method's,
+// below 1.7e-7.
+template <typename T, int C>
+__device__ __forceinline__ void user_directional(const UserArgs &a)
+{
+    const int n = a.n, nch = (n + C - 1) / C;
+    const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (item >= a.batch * nch) return;
+    const long long p = item / nch;
+    const int cstart = (int)(item - p * nch) * C;
+    const T *xp = static_cast<const T *>(a.x) + p * n, *vp = static_cast<const T *>(a.v) + p * n;
+    T *out = static_cast<T *>(a.out) + p * n;
+    const DirVars<T, C> x{xp, vp, cstart, seed_constants<T>()};
+    const Num<T, C> r = ::CHESSFAD_USER_FN<Num<T, C>, DirVars<T, C>>(x, n, a.params);
+    T zero = T(0);  // stays 0 while every value is finite
+#pragma unroll
+    for (int l = 0; l < C; ++l) {
+        if (cstart + l < n) {
+            out[cstart + l] = r.a.h[l];
+            zero += r.a.h[l] * T(0);
+        }
+    }
+    for (int k = 0; k < n; ++k) zero += vp[k] * T(0);
+    if (!(zero == T(0))) user_dense_rows<T, C>(xp, vp, out, n, cstart, a.params);
+}
+
 }  // namespace user
 }  // namespace chessfad
+
+extern "C" __global__ void __launch_bounds__(256) chessfad_user_dir_hvp(chessfad::user::UserArgs a)
+{
+    chessfad::user::user_directional<CHESSFAD_USER_T, CHESSFAD_USER_C>(a);
+}
 
 extern "C" __global__ void __launch_bounds__(256) chessfad_user_sym_hvp(chessfad::user::UserArgs a)
 {

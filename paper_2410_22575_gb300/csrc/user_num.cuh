@@ -215,5 +215,21 @@ struct Vars {
     __device__ __forceinline__ Num<T, C> operator[](int k) const { return Num<T, C>(seed<T, C>(x[k], k, i, cstart, z)); }
 };
 
+// The same for a product H v in one evaluation per chunk: d1 is seeded by the
+// direction v instead of the unit vector of a row, so the result's h
+// components are (H v)_(cstart + l).
+template <typename T, int C>
+struct DirVars {
+    const T *x, *v;
+    int cstart;
+    SeedK<T> z;
+    __device__ __forceinline__ Num<T, C> operator[](int k) const
+    {
+        HD<T, C> y = seed<T, C>(x[k], k, -1, cstart, z);
+        y.d1 = v[k];
+        return Num<T, C>(y);
+    }
+};
+
 }  // namespace user
 }  // namespace chessfad

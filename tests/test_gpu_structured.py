@@ -209,3 +209,30 @@ def test_uneven_non_finite_requests_equal_the_dense_evaluation(prec):
     fine = np.isfinite(dense)
     _same(got, dense, 4e-12 if prec == cf.FP64 else 4e-5, np.repeat(
         [np.max(np.abs(np.where(fine, dense, 0.0)[o:o + n]), initial=1.0) for o, n in zip(u.offs, u.ns)], u.ns)[fine])
+
+
+# ------------------------------------------------------------------ user functions
+@pytest.mark.parametrize("fn", [W.ROSENBROCK, W.ACKLEY, W.FLETCHER_POWELL, W.MIX])
+@pytest.mark.parametrize("prec", PRECS)
+def test_user_default_hvp(fn, prec):
+    """The default product of a user function (one evaluation per chunk with d1
+    seeded by v): chunk sizes that divide n, exceed it or leave a remainder, a
+    point per CTA edge, and non-finite x and v, where it equals the symmetric
+    method it replaces."""
+    from test_gpu_user import SYM, Case, user_fn
+
+    for c, n, batch in ((1, 5, 40), (8, 1, 300), (8, 8, 129), (8, 21, 50), (16, 7, 33), (16, 130, 3)):
+        f, k = user_fn(fn, c, prec), Case(fn, n, batch, 40 + n, prec)
+        out = f.hvp(k.x, k.v, k.params)
+        e = k.hvp_err(out)
+        assert e.max() <= BOUND[prec], (c, n, e.max())
+        assert np.array_equal(out.cpu().numpy(), f.hvp(k.x, k.v, k.params).cpu().numpy())
+    f, k = user_fn(fn, 8, prec), Case(fn, 21, 12, 7, prec)
+    k.x[1, 4], k.x[2, 20], k.x[3, 0] = np.nan, np.inf, -np.inf
+    k.v[4, 4], k.v[5, 20], k.v[6, 0] = np.nan, np.inf, -np.inf
+    k.x[7, 3], k.v[7] = np.nan, 0.0
+    got = f.hvp(k.x, k.v, k.params).double().cpu().numpy()
+    dense = f.hvp(k.x, k.v, k.params, cfg=SYM).double().cpu().numpy()
+    fine = np.isfinite(dense)
+    scale = np.max(np.abs(np.where(fine, dense, 0.0)), axis=1, keepdims=True) * np.ones_like(dense)
+    _same(got, dense, 4e-12 if prec == cf.FP64 else 4e-5, scale[fine])
