@@ -26,8 +26,10 @@ constexpr int kThreads = kFpThreads;
 // 4000 requests, n log-uniform in 2 .. 512, compensated FP32: dense 308 ms, here
 // 0.437 ms, bound by the FP64 residuals of the large Fletcher-Powell requests.
 
+// The tile functions are calls, so that each has registers of its own: inlined
+// into one kernel, the FP64 and many-variable variants made all of them spill.
 template <typename T, typename IO>
-__device__ __forceinline__ void lanes_tile(const SRaggedArgs &a, const STile &t)
+__device__ __noinline__ void lanes_tile(const SRaggedArgs &a, const STile &t)
 {
     const IO *x = static_cast<const IO *>(a.x), *v = static_cast<const IO *>(a.v);
     IO *out = static_cast<IO *>(a.out);
@@ -41,6 +43,10 @@ __device__ __forceinline__ void lanes_tile(const SRaggedArgs &a, const STile &t)
             ros_point<T, IO>(x + o, v + o, out + o, n, lane, G, active, false);
         } else {
             const AckConst nc = ack_const(n);
+            if constexpr (!std::is_same<T, IO>::value) {  // one variable
+                ack_point<T, IO, 1>(x + o, v + o, out + o, n, lane, G, active, false, nc);
+                continue;
+            }
             switch (t.epl) {
             case 1: ack_point<T, IO, 1>(x + o, v + o, out + o, n, lane, G, active, false, nc); break;
             case 4: ack_point<T, IO, 4>(x + o, v + o, out + o, n, lane, G, active, false, nc); break;
@@ -52,11 +58,11 @@ __device__ __forceinline__ void lanes_tile(const SRaggedArgs &a, const STile &t)
 }
 
 template <typename T, typename IO>
-__device__ __forceinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile &t, unsigned char *smem)
+__device__ __noinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile &t, unsigned char *smem)
 {
     __shared__ int s_last;
     IO *out = static_cast<IO *>(a.out);
-    const FpShape sh{t.nmax, t.mt, t.lanes};
+    const FpShape sh{t.nmax, t.mt, t.bufs, t.pairs, t.lanes};
     FpTile<T, IO, true> tile(FpArgs{a.A, a.B, a.Epack, a.ld}, static_cast<const IO *>(a.x),
                              static_cast<const IO *>(a.v), smem, sh, t.count, t.pairs);
     for (int q = threadIdx.x; q <= t.count; q += kThreads) {
@@ -71,7 +77,7 @@ __device__ __forceinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile
         }
     }
     __syncthreads();
-    FpSums<T, 4> sums[kFpNpt];
+    FpSums<T, 2> sums[kFpNpt];
     tile.run(t.m0, t.m1, sums);
     if (t.parts > 1) {
         double *slot = a.slots + t.slot + (long long)t.part * 4 * t.pairs;
@@ -113,7 +119,7 @@ __device__ __forceinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 2) structured_ragged_kernel(const SRaggedArgs a)
+__global__ void __launch_bounds__(kThreads, 2) structured_ragged_kernel(const __grid_constant__ SRaggedArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_tile;
@@ -195,11 +201,11 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
                 t.m0 = nmax * t.part / t.parts;
                 t.m1 = nmax * (t.part + 1) / t.parts;
                 const bool wide = f64 || t.f64;
-                const FpShape sh = wide ? fp_shape<double>(nmax, t.m1 - t.m0, t.count)
-                                        : fp_shape<float>(nmax, t.m1 - t.m0, t.count);
+                const FpShape sh = fp_shape(nmax, t.m1 - t.m0, t.count, t.pairs, wide);
                 t.mt = sh.mt;
+                t.bufs = sh.bufs;
                 t.lanes = sh.lanes;
-                pl.smem = std::max(pl.smem, wide ? fp_smem<double>(nmax, sh.mt).total : fp_smem<float>(nmax, sh.mt).total);
+                pl.smem = std::max(pl.smem, wide ? fp_smem<double>(sh).total : fp_smem<float>(sh).total);
                 work.push_back({cost / t.parts + 40.0 * t.pairs, t});
             }
             continue;

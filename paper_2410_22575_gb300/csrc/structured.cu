@@ -2,17 +2,19 @@
 // contiguous batch (structured.cuh).
 //
 // H v through the default call, GB300, dense symmetric method -> here:
-//   Ackley n = 64, FP64, 65536 points            102.2 ms -> 0.39 ms
-//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.35 ms
-//   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.100 ms
-//   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.119 ms
+//   Ackley n = 64, FP64, 65536 points            102.2 ms -> 0.256 ms
+//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.197 ms
+//   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.086 ms
+//   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.115 ms
 // Hessians:
-//   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.084 ms (6.4 TB/s written)
-//   Ackley n = 33, FP32-comp, 20000                0.178 ms -> 0.045 ms
-//   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.120 ms
-// The Rosenbrock kernel streams x and v; the other two are bound by the FP64
-// pipe (sin, cos and the sums under sqrt and exp; the residuals), in
-// compensated FP32 too.
+//   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.082 ms (6.6 TB/s written)
+//   Ackley n = 33, FP32-comp, 20000                0.178 ms -> 0.035 ms
+//   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.111 ms
+// The Rosenbrock kernels stream; the others are bound by the FP64 pipe (sin,
+// cos and the sums under sqrt and exp; the residuals), in compensated FP32 too.
+// It takes one warp instruction per 16 clocks and SM, so what is not FP64
+// arithmetic stays off it: conversions and tests of FP64 values run on 32-bit
+// words, coefficients come from registers (fp64_sincos.cuh).
 #include <algorithm>
 #include <atomic>
 
@@ -67,14 +69,14 @@ __global__ void __launch_bounds__(kFpThreads) fp_hvp_kernel(const StructArgs a, 
         }
     }
     __syncthreads();
-    FpSums<T, 4> sums[kFpNpt];
+    FpSums<T, 2> sums[kFpNpt];
     tile.run(0, n, sums);
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
         if (u >= P * n) break;
-        const FpSums<T, 4> &f = sums[i];
+        const FpSums<T, 2> &f = sums[i];
         const T o = tile.combine(u, f.value(0), f.value(1), f.value(2), f.value(3));
         bad |= not_finite(o);
         out[p0 * n + u] = (IO)o;
@@ -122,12 +124,13 @@ __global__ void __launch_bounds__(kThreads) ros_hessian_kernel(const StructArgs 
         }
         return;
     }
-    stream_rows(H, cnt, n, fd, [&](int r, int j) {
+    auto val = [&](int r, int j) {
         const int d = j - ls[r] + 1;
         T v = T(0);
         if ((unsigned)d <= 2u) v = d == 1 ? diag[r] : d == 2 ? up[r] : lo[r];
         return v;
-    });
+    };
+    stream_rows(H, cnt, n, fd, val);
 }
 
 // ppc whole points per CTA, or, split > 1, one of `split` parts of one
@@ -155,18 +158,20 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
     int *flag = reinterpret_cast<int *>(sums + 2 * ppc);
     const IO *x = static_cast<const IO *>(a.x) + p0 * n;
     const int tid = threadIdx.x;
+    const Turn<T> turn;
     for (int u = tid; u < nv; u += kThreads) {
         T s, c;
         const T xv = (T)x[u];
-        sincos_2pi<T>(xv, s, c);
+        turn(xv, s, c);
         xs[u].x = xv;
         xs[u].s = s;
         dg[u] = c;
     }
     for (int q = tid; q < npts; q += kThreads) flag[q] = 0;
     __syncthreads();
-    // S and C of each point in FP64: few variables by one thread, else a warp
-    const int G = n <= 16 ? 1 : 32, lane = tid & (G - 1);
+    // S and C of each point in FP64, G lanes per point: few, so that few FP64
+    // additions go across lanes, but at most 16 variables per lane
+    const int G = n <= 8 ? 1 : n <= 128 ? 8 : 32, lane = tid & (G - 1);
     for (int b = 0; b < npts; b += kThreads / G) {
         const int q = b + tid / G;
         double S = 0.0, C = 0.0;
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
     // the tail's factors, one thread per point
     T *tail = reinterpret_cast<T *>(flag + ppc + (ppc & 1));
     for (int q = tid; q < npts; q += kThreads) {
-        const AckTail<T> k = ack_tail(sums[2 * q], sums[2 * q + 1], nc, T(0));
+        const AckTail<T> k = ack_tail(sums[2 * q], sums[2 * q + 1], nc, false, T(0));
         const double p1 = k.p1, r1 = k.r1;  // FP64: the factors are shared by every entry
         tail[4 * q] = (T)fma(p1, (double)k.r2, ((double)k.p2 * r1) * r1);
         tail[4 * q + 1] = k.q2;
@@ -209,14 +214,16 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
     }
     __syncthreads();
     IO *H = static_cast<IO *>(a.out) + ((size_t)p0 * n + r0) * n;
-    stream_rows(H, r1 - r0, n, fd, [&](int r, int j) {
-        const int u = r + r0, base = split > 1 ? 0 : fd.div(u) * n;
-        const int w = base + j;  // the smaller index's factors are the scaled ones: H is symmetric bit for bit
+    // The smaller index's factors are the scaled ones, so H is symmetric bit
+    // for bit.
+    auto val = [&](int r, int j) {
+        const int u = r + r0, w = (split > 1 ? 0 : fd.div(u) * n) + j;
         const Pair e = (w < u ? ab : xs)[w], f = (w < u ? xs : ab)[u];
         T v = fma_(f.x, e.x, f.s * e.s);
         if (w == u) v += dg[u];
         return v;
-    });
+    };
+    stream_rows(H, r1 - r0, n, fd, val);
     bool any = false;
     for (int q = tid; q < npts; q += kThreads) any |= flag[q] != 0;
     if (__syncthreads_or(any))
@@ -227,7 +234,12 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
 }
 
 // Fletcher-Powell, first launch: the diagonal's curvature 2 sum_m r_m P_ml
-// (FP64 residuals), written to the diagonal of H.
+// (FP64 residuals), written to the diagonal of H.  For 3 <= n <= kGramSmall it
+// also leaves sin x_l and cos x_l beside it, at columns l + 1 and l + 2 (mod
+// n), where the second launch reads them before it overwrites H: FP64 sin and
+// cos again would take that launch as long as its products.
+constexpr int kGramSmall = 64;
+__device__ __forceinline__ int beside(int l, int k, int n) { return l + k < n ? l + k : l + k - n; }
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructArgs a, const FpShape sh, int ppb)
 {
@@ -246,21 +258,25 @@ __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructAr
         }
     }
     __syncthreads();
-    FpSums<T, 2> sums[kFpNpt];
+    FpSums<T, 1> sums[kFpNpt];
     tile.run(0, n, sums);
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
         if (u >= P * n) break;
         const int l = u - tile.base[tile.qs[u]];
-        static_cast<IO *>(a.out)[((size_t)p0 * n + u) * n + l] = (IO)tile.curvature(u, sums[i]);
+        IO *row = static_cast<IO *>(a.out) + ((size_t)p0 * n + u) * n;
+        row[l] = (IO)tile.curvature(u, sums[i]);
+        if (n >= 3 && n <= kGramSmall) {
+            row[beside(l, 1, n)] = (IO)narrow<T>(tile.z[u].x);
+            row[beside(l, 2, n)] = (IO)narrow<T>(tile.z[u].y);
+        }
     }
 }
 
 // Second launch, n <= kGramSmall: ppc whole points per CTA, J in shared
 // memory, one 4 x 4 block on or above the diagonal per thread; the result is
 // staged in place of J and streamed out whole.
-constexpr int kGramSmall = 64;
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kThreads) fp_gram_small_kernel(const StructArgs a, int ppc, FastDiv fd)
 {
@@ -268,19 +284,26 @@ __global__ void __launch_bounds__(kThreads) fp_gram_small_kernel(const StructArg
     const int n = a.n, nb = (n + 3) / 4, np = 4 * nb, nt = nb * (nb + 1) / 2, tid = threadIdx.x;
     const long long p0 = (long long)blockIdx.x * ppc;
     const int npts = (int)min((long long)ppc, a.batch - p0), nv = npts * n;
-    double *zs = reinterpret_cast<double *>(smem_raw), *zc = zs + n;  // dense propagation only
-    T *r = reinterpret_cast<T *>(zc + n);
-    T *J = reinterpret_cast<T *>(smem_raw + align_up((size_t)n * (2 * sizeof(double) + sizeof(T)), 16));
+    Two<double> *z = reinterpret_cast<Two<double> *>(smem_raw);  // dense propagation only
+    Two<T> *r = reinterpret_cast<Two<T> *>(z + n);
+    T *J = reinterpret_cast<T *>(smem_raw + align_up((size_t)n * (sizeof(Two<double>) + sizeof(Two<T>)), 16));
     T *ts = J + (size_t)ppc * n * np, *tc = ts + ppc * n, *dg = tc + ppc * n;
     const IO *x = static_cast<const IO *>(a.x) + p0 * n;
     IO *H = static_cast<IO *>(a.out) + (size_t)p0 * n * n;
     bool bad = false;
     for (int u = tid; u < nv; u += kThreads) {
-        double s, c;
-        sincos((double)x[u], &s, &c);
-        ts[u] = (T)s;
-        tc[u] = (T)c;
-        dg[u] = (T)H[(size_t)u * n + (u - fd.div(u) * n)];
+        const int l = u - fd.div(u) * n;
+        const IO *row = H + (size_t)u * n;
+        if (n >= 3) {
+            ts[u] = (T)row[beside(l, 1, n)];
+            tc[u] = (T)row[beside(l, 2, n)];
+        } else {
+            double s, c;
+            sincos((double)x[u], &s, &c);
+            ts[u] = (T)s;
+            tc[u] = (T)c;
+        }
+        dg[u] = (T)row[l];
         bad |= not_finite(dg[u]);
     }
     __syncthreads();
@@ -339,8 +362,7 @@ __global__ void __launch_bounds__(kThreads) fp_gram_small_kernel(const StructArg
             bool b = false;
             for (int l = tid; l < n; l += kThreads) b |= not_finite(dg[k * n + l]);
             if (__syncthreads_or(b))
-                fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, x + (size_t)k * n, H + (size_t)k * n * n, n, zs,
-                                        zc, r);
+                fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, x + (size_t)k * n, H + (size_t)k * n * n, n, z, r);
         }
 }
 
@@ -374,7 +396,7 @@ __global__ void __launch_bounds__(kThreads) fp_gram_kernel(const StructArgs a, i
     if (tid < 2 * kGramTile) {
         const int col = tid < kGramTile ? i0 + tid : j0 + tid - kGramTile;
         double s = 0.0, c = 0.0;
-        if (col < n) sincos((double)x[col], &s, &c);
+        if (col < n) sincos_rad(sincos_k(0), (double)x[col], s, c);
         ts[tid] = (T)s;
         tc[tid] = (T)c;
     }
@@ -424,8 +446,8 @@ __global__ void __launch_bounds__(kThreads) fp_gram_kernel(const StructArgs a, i
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kThreads) fp_hessian_fix_kernel(const StructArgs a)
 {
-    __shared__ double zs[kMaxVars], zc[kMaxVars];
-    __shared__ T r[kMaxVars];
+    __shared__ Two<double> z[kMaxVars];
+    __shared__ Two<T> r[kMaxVars];
     __shared__ bool todo[kThreads];
     const size_t nn = (size_t)a.n * a.n;
     const long long p0 = (long long)blockIdx.x * kThreads, p = p0 + threadIdx.x;
@@ -435,7 +457,7 @@ __global__ void __launch_bounds__(kThreads) fp_hessian_fix_kernel(const StructAr
     for (int k = 0; k < kThreads; ++k)
         if (todo[k])
             fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, static_cast<const IO *>(a.x) + (p0 + k) * a.n,
-                                    H + (size_t)(p0 + k) * nn, a.n, zs, zc, r);
+                                    H + (size_t)(p0 + k) * nn, a.n, z, r);
 }
 
 template <typename T, typename IO>
@@ -451,20 +473,35 @@ cudaError_t ack_launch(const StructArgs &a, int G, unsigned blocks, cudaStream_t
     return cudaGetLastError();
 }
 
-// Points per CTA of an FpTile kernel: as many pairs as its threads hold,
-// fewer when the batch would leave SMs without a CTA.
-int fp_points(int n, long long batch)
+// Points per CTA of an FpTile kernel: at most as many pairs as its threads
+// hold, and such that the last round of CTAs leaves few SMs idle (the FP64 pipe
+// of an SM is the bound, 2 FMAs a clock, so the time is that of the SM with
+// most work).  fmas: FP64 FMAs per (m, j).  A CTA's own cost, what the load of
+// A and B and the barriers are not hidden by, is taken as 600 + n^2 / 10
+// clocks.  Fewer than 128 pairs leave half of its threads without one.
+int fp_points(int n, long long batch, int fmas)
 {
     const int most = std::max(1, std::min(kFpMaxPts, kFpPairs / n));
-    return (int)std::min<long long>(most, std::max<long long>(1, (batch + 303) / 304));
+    const double point = 0.5 * fmas * n * n + 10.0 * n, cta = 600.0 + 0.1 * n * n;
+    int best = most;
+    double best_cost = 1e300;
+    for (int p = std::min(most, (127 + n) / n); p <= most; ++p) {
+        const long long ctas = (batch + p - 1) / p, rounds = (ctas + 151) / 152;
+        const double cost = (double)rounds * (std::min<long long>(p, batch) * point + cta);
+        if (cost <= best_cost) {
+            best_cost = cost;
+            best = p;
+        }
+    }
+    return best;
 }
 
 template <typename T, typename IO, bool kHvp>
 cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
 {
-    const int ppb = fp_points(a.n, a.batch);
-    const FpShape sh = fp_shape<T>(a.n, a.n, ppb);
-    const size_t bytes = fp_smem<T>(sh.nmax, sh.mt).total;
+    const int ppb = fp_points(a.n, a.batch, sizeof(T) == 8 ? (kHvp ? 8 : 4) : 2);
+    const FpShape sh = fp_shape(a.n, a.n, ppb, ppb * a.n, sizeof(T) == 8);
+    const size_t bytes = fp_smem<T>(sh).total;
     const long long blocks = (a.batch + ppb - 1) / ppb;
     if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
     auto kern = kHvp ? fp_hvp_kernel<T, IO> : fp_curvature_kernel<T, IO>;
@@ -506,7 +543,7 @@ cudaError_t fp_hessian(const StructArgs &a, FastDiv fd, cudaStream_t s)
         const size_t per = (size_t)n * (np + 3) * sizeof(T);
         int ppc = std::max(1, std::min(kThreads / tiles, (int)(64 * 1024 / per)));
         ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 303) / 304));
-        const size_t bytes = align_up((size_t)n * (2 * sizeof(double) + sizeof(T)), 16) + ppc * per;
+        const size_t bytes = align_up((size_t)n * (sizeof(Two<double>) + sizeof(Two<T>)), 16) + ppc * per;
         const long long blocks = (a.batch + ppc - 1) / ppc;
         if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
         auto kern = fp_gram_small_kernel<T, IO>;

@@ -30,36 +30,39 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "fp64_sincos.cuh"
 #include "hdual.cuh"
 #include "sweep.cuh"
 
 namespace chessfad {
 
-template <typename T>
-__device__ __forceinline__ bool not_finite(T x)
+// Tests and conversions of FP64 values on 32-bit words: a comparison or an
+// absolute value (also a mask of the sign bit of the whole 64-bit word, which
+// the compiler makes one of) is an FP64 instruction.
+__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u; }
+__device__ __forceinline__ bool not_finite(double x)
 {
-    return !(fabs(x) <= (sizeof(T) == 8 ? (T)1.7976931348623157e308 : (T)3.402823466e38f));
+    return ((unsigned)__double2hiint(x) & 0x7ff00000u) == 0x7ff00000u;
 }
 
 __device__ __forceinline__ float nan_of(float) { return CUDART_NAN_F; }
 __device__ __forceinline__ double nan_of(double) { return CUDART_NAN; }
 
-// float -> double through the integer pipe (exact for normal floats; zeros,
-// subnormals, Inf and NaN take the conversion instruction): the conversion
-// instruction runs at the FP64 pipe's rate, 1/64 of FP32's.
+// float -> double through the integer pipe: the conversion instruction runs at
+// the FP64 pipe's rate, 1/64 of FP32's.  Exact for normal floats; zeros and
+// subnormals become 0, Inf and NaN a finite value (callers take points with
+// those another way).
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x)
 {
-    const unsigned b = __float_as_uint(x);
-    if (((b >> 23) + 1u & 0xffu) > 1u) {  // exponent field 1 .. 254
-        const unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
-        return __hiloint2double((int)hi, (int)(b << 29));
-    }
-    return (double)x;
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    const unsigned hi = (b & 0x80000000u) | ((m >> 3) + 0x38000000u);
+    const bool zero = m < 0x00800000u;
+    return __hiloint2double(zero ? 0 : (int)hi, zero ? 0 : (int)(b << 29));
 }
 
-// double -> float, round to nearest even, through the integer pipe for results
-// in the normal float range (others take the conversion instruction).
+// double -> float, round to nearest even, through the integer pipe; results
+// below the normal float range become 0.
 template <typename T>
 __device__ __forceinline__ T narrow(double x);
 template <>
@@ -67,12 +70,12 @@ __device__ __forceinline__ double narrow<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float narrow<float>(double x)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x), m = b & 0x7fffffffffffffffull;
-    if (m - (897ull << 52) < (253ull << 52)) {  // 2^-126 <= |x| < 2^127
-        const unsigned r = (unsigned)((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23);
-        return __uint_as_float(r | (unsigned)(b >> 63) << 31);
-    }
-    return (float)x;
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), h = hi & 0x7fffffffu;
+    unsigned r = __funnelshift_l(lo, h, 3);  // exponent and 23 bits; 29 bits of lo are dropped
+    r += (((lo & 0x1fffffffu) + 0x0fffffffu + (r & 1u)) >> 29) - (896u << 23);
+    if (h < (897u << 20)) r = 0u;
+    if (h >= (1151u << 20)) r = h > 0x7ff00000u || (h == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u;
+    return __uint_as_float(r | (hi & 0x80000000u));
 }
 
 // The row-times-v sum of the dense sweeps: Dot2 in compensated FP32, FMAs in
@@ -219,12 +222,18 @@ __device__ __forceinline__ void ros_point(const IO *__restrict__ x, const IO *__
 }
 
 // ------------------------------------------------------------------ Ackley
+// sin and cos of 2 pi x; the FP64 form keeps its coefficients in registers.
 template <typename T>
-__device__ __forceinline__ void sincos_2pi(T x, T &s, T &c);
+struct Turn;
 template <>
-__device__ __forceinline__ void sincos_2pi<float>(float x, float &s, float &c) { sincospif(2.0f * x, &s, &c); }
+struct Turn<float> {
+    __device__ __forceinline__ void operator()(float x, float &s, float &c) const { sincospif(2.0f * x, &s, &c); }
+};
 template <>
-__device__ __forceinline__ void sincos_2pi<double>(double x, double &s, double &c) { sincospi(2.0 * x, &s, &c); }
+struct Turn<double> {
+    SinCosK k = sincos_k(1);
+    __device__ __forceinline__ void operator()(double x, double &s, double &c) const { sincos_turn(k, x, s, c); }
+};
 
 // The tail's derivative factors of one point, from S = sum x^2 and
 // C = sum cos 2 pi x (both FP64): r = sqrt(S/n) as a function of S/2,
@@ -236,6 +245,9 @@ struct AckTail {
     T q1, q2;  // of -exp(C/n), times -4 pi^2 and 4 pi^2: the factors that
                // cos 2 pi x's phi'' = -4 pi^2 cos and phi' = -2 pi sin (twice)
                // leave when C's components are taken as plain cos and sin
+    // -20 exp(-0.2 r) as a function of S/2: the two unary rules composed
+    __device__ __forceinline__ T f1() const { return p1 * r1; }
+    __device__ __forceinline__ T f2() const { return fma_(p1, r2, (p2 * r1) * r1); }
 };
 // The constant factors of n variables: 1/n, 1/n^2, 4 pi^2/n and -4 pi^2/n^2,
 // in compensated FP32 as unevaluated pairs (the rounded constant alone would
@@ -261,24 +273,36 @@ __host__ __device__ inline AckConst ack_const(int n)
 }
 
 // The scalar functions in FP64, or, for compensated FP32, in FP32 from the
-// correctly rounded FP64 sums.
-__device__ __forceinline__ AckTail<double> ack_tail(double S, double C, const AckConst &n, double)
+// correctly rounded FP64 sums.  pair: the thread's neighbour (lane xor 1)
+// holds the same point and the two share the exponentials; every lane of the
+// warp calls it then.
+__device__ __forceinline__ AckTail<double> ack_tail(double S, double C, const AckConst &n, bool pair, double)
 {
     AckTail<double> k;
-    const double a0 = S * n.inv_n, sq = sqrt(a0), e1 = exp(-0.2 * sq), e2 = exp(C * n.inv_n);
-    k.r1 = n.k[0] / sq;
-    k.r2 = -n.k[1] / (sq * a0);
+    const double a0 = S * n.inv_n, sq = sqrt(a0), w = 1.0 / (sq * a0);
+    double e1, e2;
+    if (pair) {
+        const bool odd = threadIdx.x & 1;
+        const double e = exp(odd ? C * n.inv_n : -0.2 * sq), o = __shfl_xor_sync(0xffffffffu, e, 1);
+        e1 = odd ? o : e;
+        e2 = odd ? e : o;
+    } else {
+        e1 = exp(-0.2 * sq);
+        e2 = exp(C * n.inv_n);
+    }
+    k.r1 = (n.k[0] * a0) * w;
+    k.r2 = -n.k[1] * w;
     k.p1 = 4.0 * e1;
     k.p2 = -0.8 * e1;
     k.q1 = n.k[2] * e2;
     k.q2 = n.k[3] * e2;
     return k;
 }
-__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const AckConst &n, float)
+__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const AckConst &n, bool, float)
 {
     AckTail<float> k;
-    const float a0 = (float)(S * n.inv_n), sq = sqrtf(a0);
-    const float e1 = expf(-0.2f * sq), e2 = expf((float)(C * n.inv_n));
+    const float a0 = narrow<float>(S * n.inv_n), sq = sqrtf(a0);
+    const float e1 = expf(-0.2f * sq), e2 = expf(narrow<float>(C * n.inv_n));
     const float d1 = 1.0f / sq, d2 = -1.0f / (sq * a0);
     auto times = [&](int i, float y) { return __fmaf_rn(n.hi[i], y, n.lo[i] * y); };
     k.r1 = times(0, d1);
@@ -291,7 +315,8 @@ __device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const Ack
 }
 
 // One variable's h component of the whole tail: S/2 carries (d1 = sd, g = x,
-// h = sh), C carries (d1 = cd, g = cg, h = ch) in the units of q1, q2.
+// h = sh), C carries (d1 = cd, g = cg, h = ch) in the units of q1, q2.  As the
+// dense sweep composes it, rule by rule:
 template <typename T>
 __device__ __forceinline__ T ack_tail_h(const AckTail<T> &k, T sd, T x, T sh, T cd, T cg, T ch)
 {
@@ -318,23 +343,29 @@ struct AckDense {
     AckTail<T> k;
     __device__ __forceinline__ AckDense(const IO *x_, int n) : x(x_), poison(false)
     {
+        const Turn<T> turn;
         double S = 0.0, C = 0.0;
         for (int j = 0; j < n; ++j) {
             T s, c;
             const T xj = (T)x[j];
-            sincos_2pi<T>(xj, s, c);
+            turn(xj, s, c);
             poison |= not_finite(xj);
             S = fma((double)xj, (double)xj, S);
             C += (double)c;
         }
-        k = ack_tail(S, C, ack_const(n), T(0));
+        k = ack_tail(S, C, ack_const(n), false, T(0));
+        // the sqrt rule's factors at any S, as the dense prologue forms them
+        const T a0 = (T)(S / n), sq = sqrt(a0), k2 = T(2) * T(1.0 / n);
+        k.r1 = k2 * (T(0.5) / sq);
+        k.r2 = (k2 * k2) * (T(-0.25) / (sq * a0));
     }
     __device__ __forceinline__ T entry(int i, int j) const
     {
         if (poison) return nan_of(T(0));
+        const Turn<T> turn;
         T si, ci, sj, cj;
-        sincos_2pi<T>((T)x[i], si, ci);
-        sincos_2pi<T>((T)x[j], sj, cj);
+        turn((T)x[i], si, ci);
+        turn((T)x[j], sj, cj);
         return ack_tail_h<T>(k, (T)x[i], (T)x[j], i == j ? T(1) : T(0), si, sj, i == j ? cj : T(0));
     }
 };
@@ -354,6 +385,7 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
                                           const AckConst &nc)
 {
     const int m = active ? n : 0;
+    const Turn<T> turn;
     T xs[EPL], vs[EPL], sn[EPL], cs[EPL];
     double S = 0.0, C = 0.0;
     RowSum<T> xv, sv;
@@ -370,7 +402,7 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
 #pragma unroll
     for (int j = 0; j < EPL; ++j) {
         if (G * j < n) {  // uniform in the group
-            sincos_2pi<T>(xs[j], sn[j], cs[j]);
+            turn(xs[j], sn[j], cs[j]);
             if (t + G * j < m) {
                 const double xd = widen(xs[j]);
                 S = fma(xd, xd, S);
@@ -387,13 +419,16 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
         sv.merge_xor(off);
     }
     bool bad = false;
+    const AckTail<T> k = ack_tail(S, C, nc, G > 1, T(0));
     if (active) {
-        const AckTail<T> k = ack_tail(S, C, nc, T(0));
-        const T xd = xv.value(), sd = sv.value();
+        // f1 h + (f2 d1) g of S/2 plus q1 h + (q2 d1) g of C
+        const T f1 = k.f1(), fx = k.f2() * xv.value(), qs = k.q2 * sv.value();
 #pragma unroll
         for (int j = 0; j < EPL; ++j) {
             if (t + G * j < n) {
-                const T o = ack_tail_h<T>(k, xd, xs[j], vs[j], sd, sn[j], cs[j] * vs[j]);
+                T o = fma_(fx, xs[j], f1 * vs[j]);
+                o = fma_(qs, sn[j], o);
+                o = fma_(k.q1, cs[j] * vs[j], o);
                 bad |= not_finite(o);
                 out[t + G * j] = (IO)o;
             }
@@ -417,29 +452,40 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
 //   pass 2  sum_m A_ml d1_m, B_ml d1_m, A_ml r_m, B_ml r_m of every pair, kept
 //           in registers across the tiles, kFpNpt pairs per thread.
 // In compensated FP32 only the residual is FP64 (2 of the 8 FMAs of an (m, j)
-// pair); the other sums add blocks of plain FP32 FMAs with TwoSum.
+// pair), and the FP64 pipe is the bound all the same; the other sums add
+// blocks of plain FP32 FMAs with TwoSum.
 constexpr int kFpThreads = 256;
 constexpr int kFpNpt = 2;
 constexpr int kFpPairs = kFpThreads * kFpNpt;
 constexpr int kFpMaxPts = 128;
 
 struct FpShape {
-    int nmax;  // largest n of the tile's points
-    int mt;    // rows of A, B per shared-memory tile
-    int lanes; // lanes per (point, row) in pass 1, a power of two <= 32
+    int nmax;   // largest n of the tile's points
+    int mt;     // rows of A, B per shared-memory tile
+    int bufs;   // tile buffers: 2 when the rows take several tiles
+    int pairs;  // (point, variable) pairs the shared arrays hold
+    int lanes;  // lanes per (point, row) in pass 1, a power of two <= 32
 };
 
-// Shared-memory layout (bytes) of a CTA.
+// Two values read and multiplied together: (A, B) of one (m, j), (sin, cos)
+// of one variable.
+template <typename T>
+struct alignas(2 * sizeof(T)) Two {
+    T x, y;
+};
+
+// Shared-memory layout (bytes) of a CTA.  The A/B tile holds (A, B) pairs in
+// FP64 and, in compensated FP32, once more rounded, for the FP32 sums.
 template <typename T>
 struct FpSmem {
-    size_t zs, zc, ts, tc, r, d, a, b, af, bf, q, base, n, xoff, eoff, total;
+    size_t z, t, rd, ab, fab, q, base, n, xoff, eoff, total;
 };
-// Row stride of the tiles: odd, so lanes on different rows (pass 1) hit
-// different banks.
+// Row stride of the tiles in pairs: odd, so lanes on different rows (pass 1)
+// hit different banks.
 __host__ __device__ inline int fp_stride(int nmax) { return nmax | 1; }
 
 template <typename T>
-__host__ __device__ inline FpSmem<T> fp_smem(int nmax, int mt)
+__host__ __device__ inline FpSmem<T> fp_smem(const FpShape &sh)
 {
     FpSmem<T> s{};
     size_t off = 0;
@@ -448,87 +494,88 @@ __host__ __device__ inline FpSmem<T> fp_smem(int nmax, int mt)
         off = align_up(off + bytes, 16);
         return at;
     };
-    const size_t tile = (size_t)mt * fp_stride(nmax);
+    const size_t tile = (size_t)sh.bufs * sh.mt * fp_stride(sh.nmax), np = (size_t)sh.pairs;
     s.xoff = take(kFpMaxPts * sizeof(long long));
     s.eoff = take(kFpMaxPts * sizeof(long long));
-    s.zs = take(kFpPairs * sizeof(double));
-    s.zc = take(kFpPairs * sizeof(double));
-    s.ts = take(kFpPairs * sizeof(T));
-    s.tc = take(kFpPairs * sizeof(T));
-    s.r = take(kFpPairs * sizeof(T));
-    s.d = take(kFpPairs * sizeof(T));
-    s.a = take(tile * sizeof(double));
-    s.b = take(tile * sizeof(double));
-    s.af = s.a;
-    s.bf = s.b;
-    if (sizeof(T) == 4) {
-        s.af = take(tile * sizeof(T));
-        s.bf = take(tile * sizeof(T));
-    }
+    s.z = take(np * sizeof(Two<double>));
+    s.t = take(np * sizeof(Two<T>));
+    s.rd = take(np * sizeof(Two<T>));
+    s.ab = take(tile * sizeof(Two<double>));
+    s.fab = sizeof(T) == 4 ? take(tile * sizeof(Two<T>)) : s.ab;
     s.n = take(kFpMaxPts * sizeof(int));
     s.base = take((kFpMaxPts + 1) * sizeof(int));
-    s.q = take(kFpPairs);
+    s.q = take(np);
     s.total = off;
     return s;
 }
 
-// Sums of pass 2 for one pair, and of pass 1 for one (point, row).
+// N pairs of sums over products of a Two with a Two or with a scalar: pass 1's
+// one pair per (point, row), pass 2's per (point, variable).
 template <typename T, int N>
 struct FpSums;
 template <int N>
 struct FpSums<double, N> {
-    double s[N];
+    double s[2 * N];
     __device__ __forceinline__ void init()
     {
 #pragma unroll
-        for (int i = 0; i < N; ++i) s[i] = 0.0;
+        for (int i = 0; i < 2 * N; ++i) s[i] = 0.0;
     }
-    __device__ __forceinline__ void fma_to(int i, double a, double b) { s[i] = __fma_rn(a, b, s[i]); }
+    __device__ __forceinline__ void add(int i, const Two<double> &a, double x, double y)
+    {
+        s[2 * i] = __fma_rn(a.x, x, s[2 * i]);
+        s[2 * i + 1] = __fma_rn(a.y, y, s[2 * i + 1]);
+    }
     __device__ __forceinline__ void flush() {}
     __device__ __forceinline__ double value(int i) const { return s[i]; }
     __device__ __forceinline__ double wide(int i) const { return s[i]; }
-    __device__ __forceinline__ void merge_xor(int off)
+    __device__ __forceinline__ RowSum<double> both() const
     {
-#pragma unroll
-        for (int i = 0; i < N; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
+        RowSum<double> r;
+        r.s = s[0] + s[1];
+        return r;
     }
 };
+// Compensated FP32: packed FMAs into block partials p, which flush() adds into
+// the pairs (s, e) with TwoSum (a - b as the exact fma(-1, b, a)).
 template <int N>
 struct FpSums<float, N> {
-    CSum s[N];
-    float p[N];
+    float2 s[N], e[N], p[N];
     __device__ __forceinline__ void init()
     {
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            s[i] = CSum{0.f, 0.f};
-            p[i] = 0.f;
-        }
+        for (int i = 0; i < N; ++i) s[i] = e[i] = p[i] = make_float2(0.f, 0.f);
     }
-    __device__ __forceinline__ void fma_to(int i, float a, float b) { p[i] = __fmaf_rn(a, b, p[i]); }
-    // the block's partial sums enter the compensated pairs
+    __device__ __forceinline__ void add(int i, const Two<float> &a, float x, float y)
+    {
+        p[i] = __ffma2_rn(make_float2(a.x, a.y), make_float2(x, y), p[i]);
+    }
     __device__ __forceinline__ void flush()
     {
+        const float2 m1 = make_float2(-1.f, -1.f);
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-            csum_add(s[i], p[i]);
-            p[i] = 0.f;
+            const float2 t = __fadd2_rn(s[i], p[i]), bb = __ffma2_rn(m1, s[i], t);
+            const float2 x = __ffma2_rn(m1, __ffma2_rn(m1, bb, t), s[i]), y = __ffma2_rn(m1, bb, p[i]);
+            e[i] = __fadd2_rn(e[i], __fadd2_rn(x, y));
+            s[i] = t;
+            p[i] = make_float2(0.f, 0.f);
         }
     }
-    __device__ __forceinline__ float value(int i) const { return csum_value(s[i]); }
-    __device__ __forceinline__ double wide(int i) const { return widen(s[i].s) + widen(s[i].e); }
-    __device__ __forceinline__ void merge_xor(int off)
+    __device__ __forceinline__ CSum sum(int i) const
     {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            CSum o;
-            o.s = __shfl_xor_sync(0xffffffffu, s[i].s, off);
-            o.e = __shfl_xor_sync(0xffffffffu, s[i].e, off);
-            s[i] = csum_merge(s[i], o);
-        }
+        return i & 1 ? CSum{s[i / 2].y, e[i / 2].y} : CSum{s[i / 2].x, e[i / 2].x};
+    }
+    __device__ __forceinline__ float value(int i) const { return csum_value(sum(i)); }
+    __device__ __forceinline__ double wide(int i) const { return (double)sum(i).s + (double)sum(i).e; }
+    __device__ __forceinline__ RowSum<float> both() const
+    {
+        RowSum<float> r;
+        r.s = csum_merge(sum(0), sum(1));
+        return r;
     }
 };
-constexpr int kFpBlock = 4;  // (m, j) pairs per FP32 block partial
+// (a block partial is kSumBlock plain FP32 FMAs per sum)
 
 struct FpArgs {
     const double *A, *B, *E;
@@ -543,33 +590,28 @@ struct FpArgs {
 // sums over it (the Hessian's diagonal part).
 template <typename T, typename IO, bool kDir>
 struct FpTile {
-    static constexpr int NS = kDir ? 4 : 2;
+    static constexpr int NS = kDir ? 2 : 1;
     const FpArgs a;
     const IO *x, *v;
     unsigned char *smem;
     const FpShape sh;
     const FpSmem<T> L;
     const int P, npairs;
-    double *zs, *zc, *ta, *tb;
-    T *ts, *tc, *rr, *dd, *fa, *fb;
+    Two<double> *z, *ab;  // (sin, cos); (A, B)
+    Two<T> *t, *rd, *fab;  // v (cos, -sin); (r, d1); (A, B)
     unsigned char *qs;
     int *ns, *base;
     long long *xoff, *eoff;
 
     __device__ __forceinline__ FpTile(const FpArgs &a_, const IO *x_, const IO *v_, unsigned char *sm,
                                       const FpShape &s, int P_, int npairs_)
-        : a(a_), x(x_), v(v_), smem(sm), sh(s), L(fp_smem<T>(s.nmax, s.mt)), P(P_), npairs(npairs_)
+        : a(a_), x(x_), v(v_), smem(sm), sh(s), L(fp_smem<T>(s)), P(P_), npairs(npairs_)
     {
-        zs = reinterpret_cast<double *>(sm + L.zs);
-        zc = reinterpret_cast<double *>(sm + L.zc);
-        ta = reinterpret_cast<double *>(sm + L.a);
-        tb = reinterpret_cast<double *>(sm + L.b);
-        ts = reinterpret_cast<T *>(sm + L.ts);
-        tc = reinterpret_cast<T *>(sm + L.tc);
-        rr = reinterpret_cast<T *>(sm + L.r);
-        dd = reinterpret_cast<T *>(sm + L.d);
-        fa = reinterpret_cast<T *>(sm + L.af);
-        fb = reinterpret_cast<T *>(sm + L.bf);
+        z = reinterpret_cast<Two<double> *>(sm + L.z);
+        ab = reinterpret_cast<Two<double> *>(sm + L.ab);
+        t = reinterpret_cast<Two<T> *>(sm + L.t);
+        rd = reinterpret_cast<Two<T> *>(sm + L.rd);
+        fab = reinterpret_cast<Two<T> *>(sm + L.fab);
         qs = sm + L.q;
         ns = reinterpret_cast<int *>(sm + L.n);
         base = reinterpret_cast<int *>(sm + L.base);
@@ -580,6 +622,7 @@ struct FpTile {
     // sin, cos (FP64) and their products with v of every pair
     __device__ __forceinline__ void stage()
     {
+        const SinCosK k = sincos_k(0);
         for (int u = threadIdx.x; u < npairs; u += kFpThreads) {
             int lo = 0, hi = P - 1;  // the pair's point: base[lo] <= u < base[lo + 1]
             while (lo < hi) {
@@ -590,35 +633,44 @@ struct FpTile {
             qs[u] = (unsigned char)lo;
             const long long o = xoff[lo] + (u - base[lo]);
             double s, c;
-            sincos((double)x[o], &s, &c);
-            zs[u] = s;
-            zc[u] = c;
+            sincos_rad(k, (double)x[o], s, c);
+            z[u] = Two<double>{s, c};
             if constexpr (kDir) {
                 const T vv = (T)v[o];
-                ts[u] = (T)s * vv;
-                tc[u] = (T)c * vv;
+                t[u] = Two<T>{narrow<T>(c) * vv, -(narrow<T>(s) * vv)};
             }
         }
     }
 
-    __device__ __forceinline__ void load_tile(int mb, int mend)
+    // Start the copy of rows [mb, mend) of A and B into a tile buffer (8-byte
+    // cp.async: any leading dimension and base alignment).
+    __device__ __forceinline__ void load_tile(int buf, int mb, int mend)
     {
-        const int w = fp_stride(sh.nmax), cnt = (mend - mb) * sh.nmax;
+        const int w = fp_stride(sh.nmax), cnt = (mend - mb) * sh.nmax, o = buf * sh.mt * w;
         for (int e = threadIdx.x; e < cnt; e += kFpThreads) {
             const int mm = e / sh.nmax, j = e - mm * sh.nmax;
-            const double av = __ldg(&a.A[(size_t)(mb + mm) * a.ld + j]), bv = __ldg(&a.B[(size_t)(mb + mm) * a.ld + j]);
-            ta[mm * w + j] = av;
-            tb[mm * w + j] = bv;
-            if constexpr (sizeof(T) == 4) {
-                fa[mm * w + j] = narrow<T>(av);
-                fb[mm * w + j] = narrow<T>(bv);
+            const size_t g = (size_t)(mb + mm) * a.ld + j;
+            const unsigned d = (unsigned)__cvta_generic_to_shared(ab + o + mm * w + j);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(a.A + g));
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8u), "l"(a.B + g));
+        }
+        asm volatile("cp.async.commit_group;");
+    }
+    // Round what this thread copied, once it has arrived.
+    __device__ __forceinline__ void round_tile(int buf, int mb, int mend)
+    {
+        if constexpr (sizeof(T) == 4) {
+            const int w = fp_stride(sh.nmax), cnt = (mend - mb) * sh.nmax, o = buf * sh.mt * w;
+            for (int e = threadIdx.x; e < cnt; e += kFpThreads) {
+                const int mm = e / sh.nmax, d = o + mm * w + e - mm * sh.nmax;
+                fab[d] = Two<T>{narrow<T>(ab[d].x), narrow<T>(ab[d].y)};
             }
         }
     }
 
-    // pass 1 over the tile's rows [mb, mend); every lane of a warp runs the
-    // same number of items (the shuffles)
-    __device__ __forceinline__ void residuals(int mb, int mend)
+    // pass 1 over the rows [mb, mend) in a buffer; every lane of a warp runs
+    // the same number of items (the shuffles)
+    __device__ __forceinline__ void residuals(int buf, int mb, int mend)
     {
         const int w = fp_stride(sh.nmax), mt = mend - mb, lanes = sh.lanes;
         const int lane = threadIdx.x & (lanes - 1), items = P * mt, groups = kFpThreads / lanes;
@@ -631,83 +683,90 @@ struct FpTile {
                 mm = idx - q * mt;
                 if (mb + mm < ns[q]) n = ns[q];
             }
-            const int z0 = base[q], row = mm * w;
-            double s = 0.0;
+            const int z0 = base[q], row = (buf * sh.mt + mm) * w;
+            double s = 0.0, s2 = 0.0;  // two chains: the FP64 latency is several issue slots
             FpSums<T, 1> d;
             d.init();
-            int blk = 0;
-            for (int j = lane; j < n; j += lanes) {
-                s = fma(ta[row + j], zs[z0 + j], fma(tb[row + j], zc[z0 + j], s));
+            auto term = [&](int j) {
+                const Two<double> g = ab[row + j], zz = z[z0 + j];
+                s = fma(g.x, zz.x, s);
+                s2 = fma(g.y, zz.y, s2);
                 if constexpr (kDir) {
-                    d.fma_to(0, fa[row + j], tc[z0 + j]);
-                    d.fma_to(0, -fb[row + j], ts[z0 + j]);
-                    if (++blk == kFpBlock) {
-                        d.flush();
-                        blk = 0;
-                    }
+                    const Two<T> tt = t[z0 + j];
+                    d.add(0, fab[row + j], tt.x, tt.y);
                 }
+            };
+            int j = lane;
+            for (; j + (kSumBlock - 1) * lanes < n; j += kSumBlock * lanes) {
+#pragma unroll
+                for (int i = 0; i < kSumBlock; ++i) term(j + i * lanes);
+                if constexpr (kDir) d.flush();
             }
-            d.flush();
+            for (; j < n; j += lanes) term(j);
+            if constexpr (kDir) d.flush();
+            s += s2;
+            RowSum<T> d1 = d.both();
             for (int off = lanes >> 1; off > 0; off >>= 1) {
                 s += __shfl_xor_sync(0xffffffffu, s, off);
-                if constexpr (kDir) d.merge_xor(off);
+                if constexpr (kDir) d1.merge_xor(off);
             }
-            if (n > 0 && lane == 0) {
-                rr[z0 + mb + mm] = (T)(a.E[eoff[q] + mb + mm] - s);
-                if constexpr (kDir) dd[z0 + mb + mm] = -d.value(0);
-            }
+            if (n > 0 && lane == 0)
+                rd[z0 + mb + mm] = Two<T>{narrow<T>(a.E[eoff[q] + mb + mm] - s), kDir ? -d1.value() : T(0)};
         }
     }
 
-    // pass 2 over the tile's rows
-    __device__ __forceinline__ void transposed(int mb, int mend, FpSums<T, NS> (&sums)[kFpNpt])
+    // pass 2 over the rows in a buffer
+    __device__ __forceinline__ void transposed(int buf, int mb, int mend, FpSums<T, NS> (&sums)[kFpNpt])
     {
         const int w = fp_stride(sh.nmax);
 #pragma unroll
         for (int i = 0; i < kFpNpt; ++i) {
             const int u = threadIdx.x + i * kFpThreads;
             if (u >= npairs) break;
-            const int q = qs[u], z0 = base[q], l = u - z0, end = min(mend, ns[q]);
-            int blk = 0;
-            for (int m = mb; m < end; ++m) {
-                const T av = fa[(m - mb) * w + l], bv = fb[(m - mb) * w + l], rv = rr[z0 + m];
-                sums[i].fma_to(0, av, rv);
-                sums[i].fma_to(1, bv, rv);
-                if constexpr (kDir) {
-                    const T dv = dd[z0 + m];
-                    sums[i].fma_to(2, av, dv);
-                    sums[i].fma_to(3, bv, dv);
-                }
-                if (++blk == 2 * kFpBlock) {
-                    sums[i].flush();
-                    blk = 0;
-                }
+            const int q = qs[u], z0 = base[q], end = min(mend, ns[q]);
+            const Two<T> *g = fab + buf * sh.mt * w + (u - z0), *f = rd + z0;
+            auto term = [&](int m) {
+                const Two<T> gg = g[(m - mb) * w], ff = f[m];
+                sums[i].add(0, gg, ff.x, ff.x);
+                if constexpr (kDir) sums[i].add(1, gg, ff.y, ff.y);
+            };
+            int m = mb;
+            for (; m + kSumBlock <= end; m += kSumBlock) {
+#pragma unroll
+                for (int k = 0; k < kSumBlock; ++k) term(m + k);
+                sums[i].flush();
             }
+            for (; m < end; ++m) term(m);
             sums[i].flush();
         }
     }
 
+    // Rows m0 <= m < m1.  The next tile's copy runs under this tile's passes.
     __device__ __forceinline__ void run(int m0, int m1, FpSums<T, NS> (&sums)[kFpNpt])
     {
 #pragma unroll
         for (int i = 0; i < kFpNpt; ++i) sums[i].init();
+        load_tile(0, m0, min(m0 + sh.mt, m1));
         stage();
-        for (int mb = m0; mb < m1; mb += sh.mt) {
+        int buf = 0;
+        for (int mb = m0; mb < m1; mb += sh.mt, buf ^= 1) {
             const int mend = min(mb + sh.mt, m1);
-            load_tile(mb, mend);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            round_tile(buf, mb, mend);
+            __syncthreads();  // the tile has arrived, and the other buffer is read no more
+            if (mend < m1) load_tile(buf ^ 1, mend, min(mend + sh.mt, m1));
+            residuals(buf, mb, mend);
             __syncthreads();
-            residuals(mb, mend);
-            __syncthreads();
-            transposed(mb, mend, sums);
-            __syncthreads();
+            transposed(buf, mb, mend, sums);
         }
+        __syncthreads();
     }
 
     // (H v)_l = 2 sum_m [d1_m g_ml + r_m h_ml], g_ml = -(A_ml cos - B_ml sin),
     // h_ml = (A_ml sin + B_ml cos) v_l
     __device__ __forceinline__ T combine(int u, T ar, T br, T ad, T bd) const
     {
-        const T s = (T)zs[u], c = (T)zc[u], vv = (T)v[xoff[qs[u]] + (u - base[qs[u]])];
+        const T s = narrow<T>(z[u].x), c = narrow<T>(z[u].y), vv = (T)v[xoff[qs[u]] + (u - base[qs[u]])];
         RowSum<T> o;
         o.add(-c, ad);
         o.add(s, bd);
@@ -716,11 +775,11 @@ struct FpTile {
         return T(2) * o.value();
     }
     // the diagonal's second-derivative part, 2 sum_m r_m (A_ml sin + B_ml cos)
-    __device__ __forceinline__ T curvature(int u, const FpSums<T, 2> &sum) const
+    __device__ __forceinline__ T curvature(int u, const FpSums<T, 1> &sum) const
     {
         RowSum<T> o;
-        o.add((T)zs[u], sum.value(0));
-        o.add((T)zc[u], sum.value(1));
+        o.add(narrow<T>(z[u].x), sum.value(0));
+        o.add(narrow<T>(z[u].y), sum.value(1));
         return T(2) * o.value();
     }
 };
@@ -732,20 +791,20 @@ template <typename T>
 struct FpDense {
     const double *A, *B;
     int ld, n;
-    const double *zs, *zc;
-    const T *r;
+    const Two<double> *z;
+    const Two<T> *r;  // .x
     bool poison;
     __device__ __forceinline__ T entry(int i, int j) const
     {
         if (poison) return nan_of(T(0));
-        const T si = (T)zs[i], ci = (T)zc[i], sj = (T)zs[j], cj = (T)zc[j];
+        const T si = (T)z[i].x, ci = (T)z[i].y, sj = (T)z[j].x, cj = (T)z[j].y;
         const T hs = i == j ? -sj : T(0), hc = i == j ? -cj : T(0);
         TermSum<T, 1, IsComp<T>::value> acc;
         acc.init();
         for (int m = 0; m < n; ++m) {
             const double *Ar = A + (size_t)m * ld, *Br = B + (size_t)m * ld;
             HD<T, 1> t;
-            t.v = r[m];
+            t.v = r[m].x;
             t.d1 = -fma_((T)Br[i], -si, (T)Ar[i] * ci);
             t.g[0] = -fma_((T)Br[j], -sj, (T)Ar[j] * cj);
             t.h[0] = -fma_((T)Br[j], hc, (T)Ar[j] * hs);
@@ -771,13 +830,12 @@ __device__ __forceinline__ bool fp_poison(const FpArgs &a, const IO *x, int n)
 
 // r_m of every m from the staged sin and cos; every thread calls it.
 template <typename T>
-__device__ __forceinline__ void fp_residuals(const FpArgs &a, const double *E, int n, const double *zs,
-                                             const double *zc, T *r)
+__device__ __forceinline__ void fp_residuals(const FpArgs &a, const double *E, int n, const Two<double> *z, Two<T> *r)
 {
     for (int m = threadIdx.x; m < n; m += blockDim.x) {
         double s = 0.0;
-        for (int j = 0; j < n; ++j) s = fma(a.A[(size_t)m * a.ld + j], zs[j], fma(a.B[(size_t)m * a.ld + j], zc[j], s));
-        r[m] = (T)(E[m] - s);
+        for (int j = 0; j < n; ++j) s = fma(a.A[(size_t)m * a.ld + j], z[j].x, fma(a.B[(size_t)m * a.ld + j], z[j].y, s));
+        r[m].x = (T)(E[m] - s);
     }
     __syncthreads();
 }
@@ -795,8 +853,8 @@ __device__ __noinline__ void fp_dense_points(const FpTile<T, IO, true> t, IO *ou
         for (int l = threadIdx.x; l < n; l += kFpThreads) bad |= not_finite((T)o[l]);
         if (!__syncthreads_or(bad)) continue;
         const bool poison = fp_poison<T>(t.a, t.x + t.xoff[q], n);
-        fp_residuals<T>(t.a, t.a.E + t.eoff[q], n, t.zs + z0, t.zc + z0, t.rr + z0);
-        const FpDense<T> d{t.a.A, t.a.B, t.a.ld, n, t.zs + z0, t.zc + z0, t.rr + z0, poison};
+        fp_residuals<T>(t.a, t.a.E + t.eoff[q], n, t.z + z0, t.rd + z0);
+        const FpDense<T> d{t.a.A, t.a.B, t.a.ld, n, t.z + z0, t.rd + z0, poison};
         for (int s = threadIdx.x; s < n; s += kFpThreads)
             o[s] = (IO)dense_row<T>(t.v + t.xoff[q], n, s, n >= wide_from, [&](int i, int j) { return d.entry(i, j); });
         __syncthreads();
@@ -870,15 +928,16 @@ __device__ __noinline__ void ack_dense_rows(const IO *x, IO *H, int n, int r0, i
     for (int i = r0 + (int)threadIdx.x; i < r1; i += blockDim.x)
         for (int j = 0; j < n; ++j) H[(size_t)i * n + j] = (IO)d.entry(i, j);
 }
-// zs, zc, r: shared scratch of n elements each
+// z, r: shared scratch of n elements each
 template <typename T, typename IO>
-__device__ __noinline__ void fp_dense_hessian(const FpArgs a, const IO *x, IO *H, int n, double *zs, double *zc, T *r)
+__device__ __noinline__ void fp_dense_hessian(const FpArgs a, const IO *x, IO *H, int n, Two<double> *z, Two<T> *r)
 {
     __syncthreads();
-    for (int l = threadIdx.x; l < n; l += blockDim.x) sincos((double)x[l], &zs[l], &zc[l]);
+    const SinCosK k = sincos_k(0);
+    for (int l = threadIdx.x; l < n; l += blockDim.x) sincos_rad(k, (double)x[l], z[l].x, z[l].y);
     const bool poison = fp_poison<T>(a, x, n);
-    fp_residuals<T>(a, a.E, n, zs, zc, r);
-    const FpDense<T> d{a.A, a.B, a.ld, n, zs, zc, r, poison};
+    fp_residuals<T>(a, a.E, n, z, r);
+    const FpDense<T> d{a.A, a.B, a.ld, n, z, r, poison};
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) H[e] = (IO)d.entry(e / n, e % n);
     __syncthreads();
 }
@@ -936,14 +995,23 @@ struct Gram4<float> {
 #pragma unroll
         for (int i = 0; i < 4; ++i) vfma(u[i], w, p[i]);
     }
+    // csum_add of two neighbours at a time (packed; a - b as the exact
+    // fma(-1, b, a), each component rounding as csum_add's)
     __device__ __forceinline__ void flush()
     {
+        const float2 m1 = make_float2(-1.f, -1.f);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                csum_add(s[i][j], p[i][j]);
-                p[i][j] = 0.f;
+            for (int j = 0; j < 4; j += 2) {
+                const float2 a = make_float2(s[i][j].s, s[i][j + 1].s), b = make_float2(p[i][j], p[i][j + 1]);
+                const float2 e = make_float2(s[i][j].e, s[i][j + 1].e);
+                const float2 t = __fadd2_rn(a, b), bb = __ffma2_rn(m1, a, t);
+                const float2 x = __ffma2_rn(m1, __ffma2_rn(m1, bb, t), a), y = __ffma2_rn(m1, bb, b);
+                const float2 f = __fadd2_rn(e, __fadd2_rn(x, y));
+                s[i][j] = CSum{t.x, f.x};
+                s[i][j + 1] = CSum{t.y, f.y};
+                p[i][j] = p[i][j + 1] = 0.f;
             }
     }
     __device__ __forceinline__ float value(int i, int j) const { return 2.0f * csum_value(s[i][j]); }

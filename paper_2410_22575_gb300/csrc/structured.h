@@ -43,7 +43,7 @@ struct STile {
     int epl;    // Ackley: variables per lane
     // Fletcher-Powell: the (point, variable) pairs, the shape, the rows of this
     // part, and, with several parts, the tile's counter and first slot element
-    int pairs, nmax, mt, m0, m1, parts, part, done;
+    int pairs, nmax, mt, bufs, m0, m1, parts, part, done;
     long long slot;
 };
 

@@ -46,17 +46,23 @@ inline int ack_lanes(int n, long long batch, bool f64)
     return best;
 }
 
-// Rows of A and B per tile: all of them within 64 KiB (two or more CTAs per
-// SM hide the barriers between the passes), else even parts of the rows.
-template <typename T>
-inline FpShape fp_shape(int nmax, int rows, int P)
+// The shape of an FpTile: rows rows of A and B for P points, pairs pairs; f64:
+// FP64 arithmetic.  All rows in one buffer within 48 KiB, else even parts of
+// them in two buffers (two or more CTAs per SM).
+inline FpShape fp_shape(int nmax, int rows, int P, int pairs, bool f64)
 {
-    const size_t row = (size_t)fp_stride(nmax) * 2 * (sizeof(double) + (sizeof(T) == 4 ? sizeof(float) : 0));
-    const int most = std::max(1, (int)(64 * 1024 / row));
-    const int tiles = (rows + most - 1) / most;
+    const size_t row = (size_t)fp_stride(nmax) * (2 * sizeof(double) + (f64 ? 0 : 2 * sizeof(float)));
     FpShape s;
     s.nmax = nmax;
-    s.mt = (rows + tiles - 1) / tiles;
+    s.pairs = pairs;
+    s.bufs = 1;
+    s.mt = rows;
+    if ((size_t)rows * row > 48 * 1024) {
+        const int most = std::max(1, (int)(40 * 1024 / row));
+        const int tiles = (rows + most - 1) / most;
+        s.bufs = 2;
+        s.mt = (rows + tiles - 1) / tiles;
+    }
     // pass 1: enough lanes per (point, row) to occupy the CTA's threads
     s.lanes = 1;
     while (s.lanes < 32 && s.lanes < nmax && P * s.mt * s.lanes < kFpThreads) s.lanes <<= 1;
