@@ -18,6 +18,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "../../include/chessfad.h"
@@ -25,6 +26,7 @@
 
 struct chessfad_user_fn {
     cudaLibrary_t lib = nullptr;
+    cudaLibrary_t dir_lib = nullptr;     // the directional kernel's
     cudaKernel_t hvp = nullptr;          // plain (CHESS-VEC, Alg. 7)
     cudaKernel_t hessian = nullptr;      // plain (CHUNK-HESS, Alg. 5)
     cudaKernel_t sym_hvp = nullptr;      // symmetric (SC-HESS-VEC, Alg. 8)
@@ -124,6 +126,48 @@ struct UserArgs {  // the kernels' chessfad::user::UserArgs, field for field
     int acc;
 };
 
+// One NVRTC compilation: the cubin, or the error and its messages.
+struct Program {
+    bool ok = false;
+    std::string log;
+    std::vector<char> cubin;
+};
+
+void compile_program(const Nvrtc &rt, const std::string &text, const char *name, int csize, int prec, bool dir,
+                     Program &out)
+{
+    const char *headers[] = {kHdualSrc, kSymLayoutSrc, kUserNumSrc, kUserKernelSrc, ""};
+    const char *header_names[] = {"hdual.cuh", "sym_layout.cuh", "user_num.cuh", "user_kernel.cuh", "cuda_runtime.h"};
+    nvrtcProgram prog = nullptr;
+    if (rt.create(&prog, text.c_str(), "chessfad_user.cu", 5, headers, header_names) != NVRTC_SUCCESS) {
+        out.log = "nvrtcCreateProgram failed";
+        return;
+    }
+    const std::string def_t = std::string("-DCHESSFAD_USER_T=") + (prec == CHESSFAD_FP64 ? "double" : "float");
+    const std::string def_c = "-DCHESSFAD_USER_C=" + std::to_string(csize);
+    const std::string def_fn = std::string("-DCHESSFAD_USER_FN=") + name;
+    const std::string def_f32 = std::string("-DCHESSFAD_USER_F32=") + (prec == CHESSFAD_FP64 ? "0" : "1");
+    const std::string def_dir = std::string("-DCHESSFAD_USER_DIR=") + (dir ? "1" : "0");
+    const char *opts[] = {"--gpu-architecture=sm_103a", "--std=c++17", "-default-device",
+                          def_t.c_str(), def_c.c_str(), def_fn.c_str(), def_f32.c_str(), def_dir.c_str()};
+    const nvrtcResult cr = rt.compile(prog, (int)(sizeof(opts) / sizeof(opts[0])), opts);
+    size_t lsz = 0;
+    rt.log_size(prog, &lsz);
+    out.log.assign(lsz, '\0');
+    if (lsz > 0) rt.log(prog, &out.log[0]);
+    while (!out.log.empty() && out.log.back() == '\0') out.log.pop_back();
+    size_t csz = 0;
+    if (cr != NVRTC_SUCCESS) {
+        out.log = std::string(rt.error_string(cr)) + "\n" + out.log;
+    } else if (rt.cubin_size(prog, &csz) != NVRTC_SUCCESS || csz == 0 ||
+               (out.cubin.resize(csz), rt.cubin(prog, out.cubin.data())) != NVRTC_SUCCESS) {
+        out.log = "NVRTC produced no cubin";
+    } else {
+        out.ok = true;
+    }
+    rt.destroy(&prog);
+}
+
 long long hs_elems(int n, int C)  // staged chunk matrix of one point, symmetric HVP
 {
     const long long nch = (n + C - 1) / C;
@@ -214,12 +258,18 @@ int launch(chessfad_user_fn *fn, const chessfad_config *cfg, bool hvp, int n, lo
         smem = (size_t)args.maxpts * 2 * sizeof(double);
         k = hvp ? fn->hvp_n1 : fn->hessian_n1;
     } else if (hvp && !cfg) {
-        // the default: one thread per (point, chunk); CTAs of 128, so that
-        // small batches reach more SMs
+        // the default: one thread per (point, chunk), `lanes` points per CTA
+        // of 128 threads: a warp's worth while x and v of that many fit 48
+        // KiB, no more than the batch has
+        const size_t elem = fn->prec == CHESSFAD_FP64 ? sizeof(double) : sizeof(float);
         const long long nch = (n + fn->csize - 1) / fn->csize;
+        int lanes = 32;
+        while (lanes > 1 && ((size_t)(lanes + 1) * n * 2 * elem > 48 * 1024 || lanes >= 2 * batch)) lanes >>= 1;
         block = 128;
-        grid = (batch * nch + block - 1) / block;
-        smem = 0;
+        const long long slots = block / lanes;
+        args.maxpts = lanes;
+        grid = (batch + lanes - 1) / lanes * ((nch + slots - 1) / slots);
+        smem = (size_t)(lanes + 1) * n * 2 * elem;
         k = fn->dir_hvp;
     } else if (method == CHESSFAD_METHOD_SYMMETRIC) {
         grid = (batch + ppb - 1) / ppb;
@@ -275,56 +325,48 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     std::string text = "#include \"user_num.cuh\"\n#line 1 \"user_function\"\n";
     text += source;
     text += "\n#include \"user_kernel.cuh\"\n";
-    const char *headers[] = {kHdualSrc, kSymLayoutSrc, kUserNumSrc, kUserKernelSrc, ""};
-    const char *header_names[] = {"hdual.cuh", "sym_layout.cuh", "user_num.cuh", "user_kernel.cuh", "cuda_runtime.h"};
-    nvrtcProgram prog = nullptr;
-    if (rt.create(&prog, text.c_str(), "chessfad_user.cu", 5, headers, header_names) != NVRTC_SUCCESS) {
-        put_log(log, log_bytes, "nvrtcCreateProgram failed");
-        return CHESSFAD_ERR_JIT;
+    // The row methods and the directional kernel as two programs: compiled side
+    // by side they take about as long as the larger one.
+    Program prog[2];
+    std::thread second;
+    try {
+        second = std::thread([&] {
+            try {
+                compile_program(rt, text, name, csize, prec, true, prog[1]);
+            } catch (...) {
+                prog[1].ok = false;  // out of memory
+            }
+        });
+    } catch (...) {  // no thread: one after the other
     }
-    const std::string def_t = std::string("-DCHESSFAD_USER_T=") + (prec == CHESSFAD_FP64 ? "double" : "float");
-    const std::string def_c = "-DCHESSFAD_USER_C=" + std::to_string(csize);
-    const std::string def_fn = std::string("-DCHESSFAD_USER_FN=") + name;
-    const std::string def_f32 = std::string("-DCHESSFAD_USER_F32=") + (prec == CHESSFAD_FP64 ? "0" : "1");
-    const char *opts[] = {"--gpu-architecture=sm_103a", "--std=c++17", "-default-device",
-                          def_t.c_str(), def_c.c_str(), def_fn.c_str(), def_f32.c_str()};
-    const nvrtcResult cr = rt.compile(prog, (int)(sizeof(opts) / sizeof(opts[0])), opts);
-    size_t lsz = 0;
-    rt.log_size(prog, &lsz);
-    std::string ltext(lsz, '\0');
-    if (lsz > 0) rt.log(prog, &ltext[0]);
-    while (!ltext.empty() && ltext.back() == '\0') ltext.pop_back();
-    if (cr != NVRTC_SUCCESS) {
-        put_log(log, log_bytes, std::string(rt.error_string(cr)) + "\n" + ltext);
-        rt.destroy(&prog);
-        return CHESSFAD_ERR_JIT;
-    }
-    put_log(log, log_bytes, ltext);
-    size_t csz = 0;
-    rt.cubin_size(prog, &csz);
-    std::vector<char> cubin(csz);
-    if (csz == 0 || rt.cubin(prog, cubin.data()) != NVRTC_SUCCESS) {
-        rt.destroy(&prog);
-        put_log(log, log_bytes, "NVRTC produced no cubin");
-        return CHESSFAD_ERR_JIT;
-    }
-    rt.destroy(&prog);
+    compile_program(rt, text, name, csize, prec, false, prog[0]);
+    if (second.joinable()) second.join();
+    else compile_program(rt, text, name, csize, prec, true, prog[1]);
+    for (const Program &p : prog)
+        if (!p.ok) {
+            put_log(log, log_bytes, p.log);
+            return CHESSFAD_ERR_JIT;
+        }
+    put_log(log, log_bytes, prog[0].log);
 
     auto *fn = new chessfad_user_fn;
     fn->csize = csize;
     fn->prec = prec;
-    cudaError_t e = cudaLibraryLoadData(&fn->lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
+    cudaError_t e = cudaLibraryLoadData(&fn->lib, prog[0].cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
+    if (e == cudaSuccess)
+        e = cudaLibraryLoadData(&fn->dir_lib, prog[1].cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->hvp, fn->lib, "chessfad_user_hvp");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->hessian, fn->lib, "chessfad_user_hessian");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hvp, fn->lib, "chessfad_user_sym_hvp");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hessian, fn->lib, "chessfad_user_sym_hessian");
-    if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->dir_hvp, fn->lib, "chessfad_user_dir_hvp");
+    if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->dir_hvp, fn->dir_lib, "chessfad_user_dir_hvp");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP) e = cudaLibraryGetKernel(&fn->hvp_n1, fn->lib, "chessfad_user_hvp_n1");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP)
         e = cudaLibraryGetKernel(&fn->hessian_n1, fn->lib, "chessfad_user_hessian_n1");
     if (e != cudaSuccess) {
         cudaGetLastError();
         put_log(log, log_bytes, std::string("compiled; loading failed: ") + cudaGetErrorString(e));
+        if (fn->dir_lib) cudaLibraryUnload(fn->dir_lib);
         if (fn->lib) cudaLibraryUnload(fn->lib);
         delete fn;
         return CHESSFAD_ERR_CUDA;
@@ -336,7 +378,9 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
 CHESSFAD_API int chessfad_user_fn_destroy(chessfad_user_fn *fn)
 {
     if (!fn) return CHESSFAD_SUCCESS;
-    cudaError_t e = fn->lib ? cudaLibraryUnload(fn->lib) : cudaSuccess;
+    const cudaError_t d = fn->dir_lib ? cudaLibraryUnload(fn->dir_lib) : cudaSuccess;
+    const cudaError_t r = fn->lib ? cudaLibraryUnload(fn->lib) : cudaSuccess;
+    const cudaError_t e = d != cudaSuccess ? d : r;
     delete fn;
     return e == cudaSuccess ? CHESSFAD_SUCCESS : CHESSFAD_ERR_CUDA;
 }

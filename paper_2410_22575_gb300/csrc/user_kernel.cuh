@@ -6,6 +6,7 @@
 //   CHESSFAD_USER_FN   the name of the user's function template
 //                        template <class R, class X>
 //                        R name(const X &x, int n, const double *params);
+//   CHESSFAD_USER_DIR  1: the directional kernel only, 0: the others
 // Two decompositions:
 //  plain (CHESS-VEC / CHUNK-HESS, the paper's L2 over rows, Sec. VI): one
 //    thread per (point, row i), sweeping the row's ceil(n/C) chunks; a CTA
@@ -18,8 +19,10 @@
 //    sums whole rows, each off-diagonal-chunk entry serving both r_i and r_j;
 //  directional (HVP, the default): one thread per (point, chunk), a single
 //    evaluation with d1 seeded by v gives the chunk's rows of H v (ceil(n/C)
-//    evaluations per point instead of n ceil(n/C)); rows that are not finite,
-//    and points whose v is not, are evaluated again by the plain method.
+//    evaluations per point instead of n ceil(n/C)), on numbers that skip the
+//    zero components of what does not depend on the chunk; rows that are not
+//    finite, and points whose d1 or v is not, are evaluated again by the plain
+//    method.
 // FP32: the row-times-v products are summed as a Dot2 (TwoProd by FMA plus
 // TwoSum); the function's own arithmetic is plain FP32, as written by the
 // user, except at n = 1 (FP64 arithmetic, float I/O).  FP64: fused
@@ -257,43 +260,70 @@ __device__ __noinline__ void user_dense_rows(const T *xp, const T *vp, T *out, i
     }
 }
 
-// Bound by the arithmetic of f on 2C + 2 components (FP64 pipe or FMA issue);
-// x and v come from L1 (the lanes of a point read the same element).  The
-// extended-operator test function, n = 64, C = 8, FP64, 4096 points: symmetric
-// method 100.7 ms, here 2.83 ms.  Errors against the oracle (FP32, n = 19 and
-// 64, rms over the test functions): 1.0 to 1.24 times the symmetric method's,
-// below 1.7e-7.
+// A CTA holds a.maxpts points (a power of two <= 32, one per lane) and
+// blockDim / maxpts of their chunks; x and v of its points are staged in
+// shared memory point by point within each variable, so a warp's lanes read
+// different banks.  Lanes of a warp are on the same chunk (or on a few), so
+// the activity of their numbers agrees and its branches do not diverge.
+// Bound by the arithmetic of f: its functions of values, once per chunk, and the
+// active components.  The extended-operator test function, n = 64, C = 8, FP64,
+// 4096 points: symmetric method 100.7 ms; every component of every number 2.83
+// ms; active components 1.67 ms; one power instead of three per pow() 1.31 ms.
+// Errors against the oracle (FP32, n = 19 and 64, rms over the test functions):
+// 1.0 to 1.24 times the symmetric method's, below 1.7e-7.
 template <typename T, int C>
 __device__ __forceinline__ void user_directional(const UserArgs &a)
 {
-    const int n = a.n, nch = (n + C - 1) / C;
-    const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (item >= a.batch * nch) return;
-    const long long p = item / nch;
-    const int cstart = (int)(item - p * nch) * C;
-    const T *xp = static_cast<const T *>(a.x) + p * n, *vp = static_cast<const T *>(a.v) + p * n;
-    T *out = static_cast<T *>(a.out) + p * n;
-    const DirVars<T, C> x{xp, vp, cstart, seed_constants<T>()};
-    const Num<T, C> r = ::CHESSFAD_USER_FN<Num<T, C>, DirVars<T, C>>(x, n, a.params);
-    T zero = T(0);  // stays 0 while every value is finite
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n, nch = (n + C - 1) / C, L = a.maxpts, slots = blockDim.x / L;
+    const int groups = (nch + slots - 1) / slots;
+    const long long p0 = (long long)(blockIdx.x / groups) * L;
+    const int npts = (int)(a.batch - p0 < L ? a.batch - p0 : L);
+    const int S = L + 1;  // odd: the transposing stores hit different banks
+    T *xs = reinterpret_cast<T *>(smem_raw), *vs = xs + (size_t)n * S;
+    const T *xg = static_cast<const T *>(a.x) + p0 * n, *vg = static_cast<const T *>(a.v) + p0 * n;
+    for (int e = threadIdx.x; e < npts * n; e += blockDim.x) {
+        const int q = e / n, k = e - q * n;
+        xs[k * S + q] = xg[e];
+        vs[k * S + q] = vg[e];
+    }
+    __syncthreads();
+    const int q = threadIdx.x & (L - 1);
+    const int cn = (int)(blockIdx.x % groups) * slots + threadIdx.x / L, cstart = cn * C;
+    if (q >= npts || cn >= nch) return;
+    using N = Num<T, C, true>;
+    const DirVars<T, C> x{xs + q, vs + q, S, cstart, seed_constants<T>()};
+    const N r = ::CHESSFAD_USER_FN<N, DirVars<T, C>>(x, n, a.params);
+    T *out = static_cast<T *>(a.out) + (p0 + q) * n;
+    // stays 0 while the chunk's rows, d1 (which every skipped product's
+    // factors reach) and v are finite
+    T zero = r.a.d1 * T(0);
 #pragma unroll
     for (int l = 0; l < C; ++l) {
         if (cstart + l < n) {
-            out[cstart + l] = r.a.h[l];
-            zero += r.a.h[l] * T(0);
+            const T h = r.act ? r.a.h[l] : T(0);
+            out[cstart + l] = h;
+            zero += h * T(0);
         }
     }
-    for (int k = 0; k < n; ++k) zero += vp[k] * T(0);
-    if (!(zero == T(0))) user_dense_rows<T, C>(xp, vp, out, n, cstart, a.params);
+    for (int k = 0; k < n; ++k) zero += vs[k * S + q] * T(0);
+    if (!(zero == T(0)))
+        user_dense_rows<T, C>(xg + (size_t)q * n, vg + (size_t)q * n, out, n, cstart, a.params);
 }
 
 }  // namespace user
 }  // namespace chessfad
 
+// CHESSFAD_USER_DIR: the directional kernel, else the row methods; the two are
+// compiled as two programs at the same time.
+#if CHESSFAD_USER_DIR
+
 extern "C" __global__ void __launch_bounds__(256) chessfad_user_dir_hvp(chessfad::user::UserArgs a)
 {
     chessfad::user::user_directional<CHESSFAD_USER_T, CHESSFAD_USER_C>(a);
 }
+
+#else
 
 extern "C" __global__ void __launch_bounds__(256) chessfad_user_sym_hvp(chessfad::user::UserArgs a)
 {
@@ -328,4 +358,6 @@ extern "C" __global__ void __launch_bounds__(256) chessfad_user_hessian_n1(chess
 {
     chessfad::user::user_sweep<double, float, 1, false>(a);
 }
+#endif
+
 #endif

@@ -26,10 +26,8 @@ namespace user {
 
 // Scalar math by precision (distinct names, so the Num overloads below never
 // hide the scalar ones inside this namespace).
-__device__ __forceinline__ float m_sin(float x) { return sinf(x); }
-__device__ __forceinline__ double m_sin(double x) { return sin(x); }
-__device__ __forceinline__ float m_cos(float x) { return cosf(x); }
-__device__ __forceinline__ double m_cos(double x) { return cos(x); }
+__device__ __forceinline__ void m_sincos(float x, float &s, float &c) { sincosf(x, &s, &c); }
+__device__ __forceinline__ void m_sincos(double x, double &s, double &c) { sincos(x, &s, &c); }
 __device__ __forceinline__ float m_tan(float x) { return tanf(x); }
 __device__ __forceinline__ double m_tan(double x) { return tan(x); }
 __device__ __forceinline__ float m_tanh(float x) { return tanhf(x); }
@@ -43,154 +41,278 @@ __device__ __forceinline__ double m_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float m_pow(float x, float p) { return powf(x, p); }
 __device__ __forceinline__ double m_pow(double x, double p) { return pow(x, p); }
 
-template <typename T, int C>
+// A: whether the number tracks activity.  In one evaluation a variable outside
+// the chunk has zero g and h components, and so has everything computed from
+// such variables alone; with A the zeros are neither stored nor multiplied
+// (act is false), only the value and d1 are.  A skipped product would be an
+// exact zero unless its other factor is Inf or NaN.  Such a factor makes d1
+// not finite, at the latest through the phi''(u) * 0 that the unary rule adds,
+// and d1 stays so in whatever is computed from it; callers look at the
+// result's d1.
+template <typename T, int C, bool A = false>
 struct Num {
     HD<T, C> a;
+    bool act;
 
-    __device__ __forceinline__ Num() : a(hzero<T, C>()) {}
+    __device__ __forceinline__ Num() : a(hzero<T, C>()), act(!A) {}
     // A constant: value s, every derivative component zero.
-    __device__ __forceinline__ Num(double s) : a(hzero<T, C>()) { a.v = T(s); }
-    __device__ __forceinline__ explicit Num(const HD<T, C> &h) : a(h) {}
+    __device__ __forceinline__ Num(double s) : a(hzero<T, C>()), act(!A) { a.v = T(s); }
+    __device__ __forceinline__ explicit Num(const HD<T, C> &h, bool on = true) : a(h), act(!A || on) {}
 
     __device__ __forceinline__ T value() const { return a.v; }
 
-    __device__ __forceinline__ Num &operator+=(const Num &w) { a = hadd(a, w.a); return *this; }
-    __device__ __forceinline__ Num &operator-=(const Num &w) { a = hsub(a, w.a); return *this; }
-    __device__ __forceinline__ Num &operator*=(const Num &w) { a = hmul(a, w.a); return *this; }
+    __device__ __forceinline__ Num &operator+=(const Num &w) { return *this = *this + w; }
+    __device__ __forceinline__ Num &operator-=(const Num &w) { return *this = *this - w; }
+    __device__ __forceinline__ Num &operator*=(const Num &w) { return *this = *this * w; }
     __device__ __forceinline__ Num &operator+=(double s) { a.v += T(s); return *this; }
     __device__ __forceinline__ Num &operator-=(double s) { a.v -= T(s); return *this; }
-    __device__ __forceinline__ Num &operator*=(double s) { a = smul(T(s), a); return *this; }
+    __device__ __forceinline__ Num &operator*=(double s) { return *this = *this * s; }
     __device__ __forceinline__ Num &operator/=(const Num &w);
     __device__ __forceinline__ Num &operator/=(double s);
 };
 
-template <typename T, int C>
-__device__ __forceinline__ T value(const Num<T, C> &u) { return u.a.v; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ T value(const Num<T, C, A> &u) { return u.a.v; }
 
 // ---- arithmetic (Fig. 1)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u, const Num<T, C, A> &w)
+{
+    if constexpr (!A) return Num<T, C, A>(hadd(u.a, w.a));
+    Num<T, C, A> r = u;
+    r.a.v = u.a.v + w.a.v;
+    r.a.d1 = u.a.d1 + w.a.d1;
+    if (w.act) {
+        if (u.act) {
+            vadd(u.a.g, w.a.g, r.a.g);
+            vadd(u.a.h, w.a.h, r.a.h);
+        } else {
+#pragma unroll
+            for (int l = 0; l < C; ++l) {
+                r.a.g[l] = w.a.g[l];
+                r.a.h[l] = w.a.h[l];
+            }
+            r.act = true;
+        }
+    }
+    return r;
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u, const Num<T, C, A> &w)
+{
+    if constexpr (!A) return Num<T, C, A>(hsub(u.a, w.a));
+    Num<T, C, A> r = u;
+    r.a.v = u.a.v - w.a.v;
+    r.a.d1 = u.a.d1 - w.a.d1;
+    if (w.act) {
+#pragma unroll
+        for (int l = 0; l < C; ++l) {
+            r.a.g[l] = u.act ? u.a.g[l] - w.a.g[l] : -w.a.g[l];
+            r.a.h[l] = u.act ? u.a.h[l] - w.a.h[l] : -w.a.h[l];
+        }
+        r.act = true;
+    }
+    return r;
+}
+// u * w with w inactive: the rule's terms without the zeros of w
 template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator+(const Num<T, C> &u, const Num<T, C> &w) { return Num<T, C>(hadd(u.a, w.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator-(const Num<T, C> &u, const Num<T, C> &w) { return Num<T, C>(hsub(u.a, w.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator*(const Num<T, C> &u, const Num<T, C> &w) { return Num<T, C>(hmul(u.a, w.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator-(const Num<T, C> &u) { return Num<T, C>(rsub(T(0), u.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator+(const Num<T, C> &u) { return u; }
+__device__ __forceinline__ void hmul_by(const HD<T, C> &u, const HD<T, C> &w, HD<T, C> &r)
+{
+    vmul(w.v, u.g, r.g);
+    vmul(w.d1, u.g, r.h);
+    vfma(w.v, u.h, r.h);
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, const Num<T, C, A> &w)
+{
+    if constexpr (!A) return Num<T, C, A>(hmul(u.a, w.a));
+    Num<T, C, A> r;
+    if (u.act) {
+        if (w.act) {
+            r.a = hmul(u.a, w.a);
+            r.act = true;
+            return r;
+        }
+        hmul_by(u.a, w.a, r.a);
+    } else if (w.act) {
+        hmul_by(w.a, u.a, r.a);
+    }
+    r.act = u.act || w.act;
+    r.a.v = u.a.v * w.a.v;
+    r.a.d1 = fma_(w.a.v, u.a.d1, u.a.v * w.a.d1);
+    return r;
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u)
+{
+    if constexpr (!A) return Num<T, C, A>(rsub(T(0), u.a));
+    Num<T, C, A> r = u;
+    r.a.v = T(0) - u.a.v;
+    r.a.d1 = -u.a.d1;
+    if (u.act) {
+#pragma unroll
+        for (int l = 0; l < C; ++l) {
+            r.a.g[l] = -u.a.g[l];
+            r.a.h[l] = -u.a.h[l];
+        }
+    }
+    return r;
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u) { return u; }
 
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator+(const Num<T, C> &u, double s) { Num<T, C> r = u; r.a.v += T(s); return r; }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator+(double s, const Num<T, C> &u) { Num<T, C> r = u; r.a.v = T(s) + r.a.v; return r; }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator-(const Num<T, C> &u, double s) { Num<T, C> r = u; r.a.v -= T(s); return r; }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator-(double s, const Num<T, C> &u) { return Num<T, C>(rsub(T(s), u.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator*(const Num<T, C> &u, double s) { return Num<T, C>(smul(T(s), u.a)); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator*(double s, const Num<T, C> &u) { return Num<T, C>(smul(T(s), u.a)); }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u, double s) { Num<T, C, A> r = u; r.a.v += T(s); return r; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator+(double s, const Num<T, C, A> &u) { Num<T, C, A> r = u; r.a.v = T(s) + r.a.v; return r; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u, double s) { Num<T, C, A> r = u; r.a.v -= T(s); return r; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator-(double s, const Num<T, C, A> &u)
+{
+    Num<T, C, A> r = -u;
+    r.a.v = T(s) - u.a.v;
+    return r;
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, double s)
+{
+    if constexpr (!A) return Num<T, C, A>(smul(T(s), u.a));
+    Num<T, C, A> r = u;
+    r.a.v = T(s) * u.a.v;
+    r.a.d1 = T(s) * u.a.d1;
+    if (u.act) {
+        vmul(T(s), u.a.g, r.a.g);
+        vmul(T(s), u.a.h, r.a.h);
+    }
+    return r;
+}
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator*(double s, const Num<T, C, A> &u) { return u * s; }
 
 // phi(u) from phi, phi', phi'' at the value.
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> apply(const Num<T, C> &u, T phi, T d1, T d2) { return Num<T, C>(unary(u.a, phi, d1, d2)); }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> apply(const Num<T, C, A> &u, T phi, T d1, T d2)
+{
+    if constexpr (!A) return Num<T, C, A>(unary(u.a, phi, d1, d2));
+    Num<T, C, A> r;
+    if (u.act) {
+        r.a = unary(u.a, phi, d1, d2);
+    } else {
+        r.a.v = phi;
+        r.a.d1 = fma_(d2, T(0), d1 * u.a.d1);
+    }
+    r.act = u.act;
+    return r;
+}
 
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> recip(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> recip(const Num<T, C, A> &u)
 {
     const T r = T(1) / u.a.v;
     return apply(u, r, -r * r, T(2) * r * r * r);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator/(const Num<T, C> &u, const Num<T, C> &w) { return u * recip(w); }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator/(double s, const Num<T, C> &w) { return s * recip(w); }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator/(const Num<T, C, A> &u, const Num<T, C, A> &w) { return u * recip(w); }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator/(double s, const Num<T, C, A> &w) { return s * recip(w); }
 // u / s divides every component (correctly rounded per component).
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> operator/(const Num<T, C> &u, double s)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> operator/(const Num<T, C, A> &u, double s)
 {
     const T d = T(s);
-    Num<T, C> r = u;
+    Num<T, C, A> r = u;
     r.a.v /= d;
     r.a.d1 /= d;
+    if (!A || u.act) {
 #pragma unroll
-    for (int l = 0; l < C; ++l) {
-        r.a.g[l] /= d;
-        r.a.h[l] /= d;
+        for (int l = 0; l < C; ++l) {
+            r.a.g[l] /= d;
+            r.a.h[l] /= d;
+        }
     }
     return r;
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> &Num<T, C>::operator/=(const Num<T, C> &w) { *this = *this / w; return *this; }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> &Num<T, C>::operator/=(double s) { *this = *this / s; return *this; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> &Num<T, C, A>::operator/=(const Num<T, C, A> &w) { *this = *this / w; return *this; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> &Num<T, C, A>::operator/=(double s) { *this = *this / s; return *this; }
 
 // ---- elementary functions
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> sin(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> sin(const Num<T, C, A> &u)
 {
-    const T s = m_sin(u.a.v), c = m_cos(u.a.v);
+    T s, c;
+    m_sincos(u.a.v, s, c);
     return apply(u, s, c, -s);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> cos(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> cos(const Num<T, C, A> &u)
 {
-    const T s = m_sin(u.a.v), c = m_cos(u.a.v);
+    T s, c;
+    m_sincos(u.a.v, s, c);
     return apply(u, c, -s, -c);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> tan(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> tan(const Num<T, C, A> &u)
 {
     const T t = m_tan(u.a.v), d = T(1) + t * t;
     return apply(u, t, d, T(2) * t * d);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> tanh(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> tanh(const Num<T, C, A> &u)
 {
     const T t = m_tanh(u.a.v), d = T(1) - t * t;
     return apply(u, t, d, T(-2) * t * d);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> exp(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> exp(const Num<T, C, A> &u)
 {
     const T e = m_exp(u.a.v);
     return apply(u, e, e, e);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> log(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> log(const Num<T, C, A> &u)
 {
     const T r = T(1) / u.a.v;
     return apply(u, m_log(u.a.v), r, -r * r);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> sqrt(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> sqrt(const Num<T, C, A> &u)
 {
     const T s = m_sqrt(u.a.v), d = T(0.5) / s;
     return apply(u, s, d, -d / (T(2) * u.a.v));
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> pow(const Num<T, C> &u, double p)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> pow(const Num<T, C, A> &u, double p)
 {
-    const T q = T(p);
-    return apply(u, m_pow(u.a.v, q), q * m_pow(u.a.v, q - T(1)), q * (q - T(1)) * m_pow(u.a.v, q - T(2)));
+    // One power and two products (each correctly rounded) where u and the
+    // power are positive and far from the ends of the range; the three powers
+    // themselves elsewhere (zero, negative, overflow, underflow, NaN).
+    const T q = T(p), x = u.a.v, w = m_pow(x, q - T(2)), big = sizeof(T) == 8 ? T(1e75) : T(1e9);
+    T w1 = w * x, w0 = w1 * x;
+    if (!(x > T(1) / big && x < big && w > T(1) / big && w < big)) {
+        w1 = m_pow(x, q - T(1));
+        w0 = m_pow(x, q);
+    }
+    return apply(u, w0, q * w1, q * (q - T(1)) * w);
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> abs(const Num<T, C> &u)
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> abs(const Num<T, C, A> &u)
 {
     return u.a.v < T(0) ? -u : u;
 }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> fabs(const Num<T, C> &u) { return abs(u); }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> fabs(const Num<T, C, A> &u) { return abs(u); }
 
 // ---- comparisons on values
 #define CHESSFAD_USER_CMP(op)                                                                               \
-    template <typename T, int C>                                                                           \
-    __device__ __forceinline__ bool operator op(const Num<T, C> &u, const Num<T, C> &w) { return u.a.v op w.a.v; } \
-    template <typename T, int C>                                                                           \
-    __device__ __forceinline__ bool operator op(const Num<T, C> &u, double s) { return u.a.v op T(s); }    \
-    template <typename T, int C>                                                                           \
-    __device__ __forceinline__ bool operator op(double s, const Num<T, C> &u) { return T(s) op u.a.v; }
+    template <typename T, int C, bool A>                                                                           \
+    __device__ __forceinline__ bool operator op(const Num<T, C, A> &u, const Num<T, C, A> &w) { return u.a.v op w.a.v; } \
+    template <typename T, int C, bool A>                                                                           \
+    __device__ __forceinline__ bool operator op(const Num<T, C, A> &u, double s) { return u.a.v op T(s); }    \
+    template <typename T, int C, bool A>                                                                           \
+    __device__ __forceinline__ bool operator op(double s, const Num<T, C, A> &u) { return T(s) op u.a.v; }
 CHESSFAD_USER_CMP(<)
 CHESSFAD_USER_CMP(<=)
 CHESSFAD_USER_CMP(>)
@@ -199,10 +321,10 @@ CHESSFAD_USER_CMP(==)
 CHESSFAD_USER_CMP(!=)
 #undef CHESSFAD_USER_CMP
 
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> fmin(const Num<T, C> &u, const Num<T, C> &w) { return w.a.v < u.a.v ? w : u; }
-template <typename T, int C>
-__device__ __forceinline__ Num<T, C> fmax(const Num<T, C> &u, const Num<T, C> &w) { return w.a.v > u.a.v ? w : u; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> fmin(const Num<T, C, A> &u, const Num<T, C, A> &w) { return w.a.v < u.a.v ? w : u; }
+template <typename T, int C, bool A>
+__device__ __forceinline__ Num<T, C, A> fmax(const Num<T, C, A> &u, const Num<T, C, A> &w) { return w.a.v > u.a.v ? w : u; }
 
 // The variables x_0 .. x_{n-1} of one evaluation: x[k] is the CHUNK-INIT
 // seed of variable k (Alg. 4) for Hessian row i and the chunk starting at
@@ -221,13 +343,24 @@ struct Vars {
 template <typename T, int C>
 struct DirVars {
     const T *x, *v;
-    int cstart;
+    int stride, cstart;
     SeedK<T> z;
-    __device__ __forceinline__ Num<T, C> operator[](int k) const
+    __device__ __forceinline__ Num<T, C, true> operator[](int k) const
     {
-        HD<T, C> y = seed<T, C>(x[k], k, -1, cstart, z);
-        y.d1 = v[k];
-        return Num<T, C>(y);
+        // x, v: this point's variables, `stride` elements apart
+        HD<T, C> y;
+        y.v = x[k * stride];
+        y.d1 = v[k * stride];
+        const int d = k - cstart;
+        const bool in = d >= 0 && d < C;
+        if (in) {
+#pragma unroll
+            for (int l = 0; l < C; ++l) {
+                y.g[l] = (d == l) ? z.one : z.z;
+                y.h[l] = z.z;
+            }
+        }
+        return Num<T, C, true>(y, in);
     }
 };
 
