@@ -66,6 +66,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Load the CUDA library (building it first if it is absent or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -146,11 +148,18 @@ def _addr(t) -> int | None:
     raise TypeError(f"expected a device tensor or an address, got {type(t)}")
 
 
+def _current_stream() -> int:
+    """The handle of the current device's current stream, without the Stream
+    object around it."""
+    import torch
+
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
+
+
 def _stream(s) -> int | None:
     if s is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream
@@ -184,6 +193,12 @@ def _require_cuda(**tensors):
             raise ValueError(f"{name}: expected a tensor on {first or 'a CUDA device'}, got {t.device}")
         if first is None:
             first = t.device
+
+
+def _fits(t, dtype, shape, device) -> bool:
+    """Whether t passes _require and _require_cuda beside tensors of `device`
+    (their checks in the order that is cheapest when all hold)."""
+    return t.dtype is dtype and t.shape == shape and t.is_contiguous() and t.device == device
 
 
 def _points(x, name="x"):
@@ -361,14 +376,21 @@ def hvp(fn, x, v, csize=0, params=None, prec=None, stream=None, out=None, cfg=No
     import torch
 
     batch, n = _points(x)
+    dtype = x.dtype
     if prec is None:
-        prec = FP64 if x.dtype == torch.float64 else FP32_COMP
-    _require(x, "x", _dtype(prec), (batch, n))
-    _require(v, "v", _dtype(prec), (batch, n))
-    if out is not None:
-        _require(out, "out", _dtype(prec), (batch, n))
-    _require_fp_extent(fn, n, params)
-    _require_cuda(x=x, v=v, out=out)
+        prec = FP64 if dtype == torch.float64 else FP32_COMP
+    want, shape, device = _dtype(prec), x.shape, x.device
+    if not (isinstance(v, torch.Tensor) and (out is None or isinstance(out, torch.Tensor)) and device.type == "cuda"
+            and _fits(x, want, shape, device) and _fits(v, want, shape, device)
+            and (out is None or _fits(out, want, shape, device))):
+        _require(x, "x", want, (batch, n))
+        _require(v, "v", want, (batch, n))
+        if out is not None:
+            _require(out, "out", want, (batch, n))
+        _require_fp_extent(fn, n, params)
+        _require_cuda(x=x, v=v, out=out)
+    if params is not None:
+        _require_fp_extent(fn, n, params)
     if out is None:
         out = torch.empty_like(x)
     if cfg is not None:
