@@ -27,7 +27,8 @@
  *    a function's terms use error-free transformations (TwoProd by FMA,
  *    TwoSum), and the sums whose cancellation matters -- the Fletcher-Powell
  *    residuals E_m - sum_j(...) and the Ackley sums under sqrt and exp -- are
- *    computed in FP64 once per point.  Fletcher-Powell A, B, E are always
+ *    computed in FP64 once per point (the Ackley sums of the structured H v as
+ *    Dot2 and Sum2, twice FP32's precision, in about the same bits).  Fletcher-Powell A, B, E are always
  *    double.
  *  - csize (the chunk size) must be one of 1, 2, 4, 8, 16, 32, or 0 for
  *    "choose for me".  A call that names neither a chunk size nor a method

@@ -3,7 +3,7 @@
 //
 // H v through the default call, GB300, dense symmetric method -> here:
 //   Ackley n = 64, FP64, 65536 points            102.2 ms -> 0.256 ms
-//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.197 ms
+//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.143 ms
 //   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.086 ms
 //   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.115 ms
 // Hessians:

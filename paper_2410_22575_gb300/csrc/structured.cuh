@@ -298,11 +298,12 @@ __device__ __forceinline__ AckTail<double> ack_tail(double S, double C, const Ac
     k.q2 = n.k[3] * e2;
     return k;
 }
-__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const AckConst &n, bool, float)
+// In compensated FP32, from a0 = S/n and c = C/n.
+__device__ __forceinline__ AckTail<float> ack_tail_f(float a0, float c, const AckConst &n)
 {
     AckTail<float> k;
-    const float a0 = narrow<float>(S * n.inv_n), sq = sqrtf(a0);
-    const float e1 = expf(-0.2f * sq), e2 = expf(narrow<float>(C * n.inv_n));
+    const float sq = sqrtf(a0);
+    const float e1 = expf(-0.2f * sq), e2 = expf(c);
     const float d1 = 1.0f / sq, d2 = -1.0f / (sq * a0);
     auto times = [&](int i, float y) { return __fmaf_rn(n.hi[i], y, n.lo[i] * y); };
     k.r1 = times(0, d1);
@@ -312,6 +313,10 @@ __device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const Ack
     k.q1 = times(2, e2);
     k.q2 = times(3, e2);
     return k;
+}
+__device__ __forceinline__ AckTail<float> ack_tail(double S, double C, const AckConst &n, bool, float)
+{
+    return ack_tail_f(narrow<float>(S * n.inv_n), narrow<float>(C * n.inv_n), n);
 }
 
 // One variable's h component of the whole tail: S/2 carries (d1 = sd, g = x,
@@ -377,6 +382,100 @@ __device__ __noinline__ void ack_dense_hvp(const IO *x, const IO *v, IO *out, in
         out[s] = (IO)dense_row<T>(v, n, s, wide, [&](int i, int j) { return d.entry(i, j); });
 }
 
+// The four sums of one point: S = sum x^2, C = sum cos 2 pi x and the
+// direction's sum x v and sum sin(2 pi x) v, over a lane's variables, then
+// over the G lanes of its group.
+template <typename T>
+struct AckSums;
+template <>
+struct AckSums<double> {
+    double S = 0.0, C = 0.0, X = 0.0, Y = 0.0;
+    __device__ __forceinline__ void add(double x, double v, double s, double c)
+    {
+        S = fma(x, x, S);
+        C += c;
+        X = fma(x, v, X);
+        Y = fma(s, v, Y);
+    }
+    __device__ __forceinline__ void merge(int G)
+    {
+        for (int off = G >> 1; off > 0; off >>= 1) {
+            S += __shfl_xor_sync(0xffffffffu, S, off);
+            C += __shfl_xor_sync(0xffffffffu, C, off);
+            X += __shfl_xor_sync(0xffffffffu, X, off);
+            Y += __shfl_xor_sync(0xffffffffu, Y, off);
+        }
+    }
+    __device__ __forceinline__ AckTail<double> tail(const AckConst &n, bool pair) const
+    {
+        return ack_tail(S, C, n, pair, 0.0);
+    }
+    __device__ __forceinline__ double x() const { return X; }
+    __device__ __forceinline__ double y() const { return Y; }
+    __device__ __forceinline__ bool small() const { return false; }
+};
+// Compensated FP32: Dot2 and Sum2 (the error term catches the rounding of
+// every product and addition, so a sum is as accurate as one formed in twice
+// FP32's precision), the sums two by two in packed instructions: (S, X) of
+// x * (x, v), (Y, C) of (s, c) * (v, 1).  FP64 sums of the same values took
+// 60 % of the kernel's time, on a pipe with 1/64 of the FP32 rate, for bits
+// that the rounding of S/n and C/n to FP32 discards.
+template <>
+struct AckSums<float> {
+    float2 p, pe, q, qe;  // (S, X), (Y, C) and their errors
+    __device__ __forceinline__ AckSums()
+    {
+        p = pe = q = qe = make_float2(0.f, 0.f);
+    }
+    // (s, e) += a * b by TwoProd and TwoSum
+    __device__ __forceinline__ static void dot2(float2 &s, float2 &e, float2 a, float2 b)
+    {
+        const float2 m1 = make_float2(-1.f, -1.f);
+        const float2 w = __fmul2_rn(a, b), we = __ffma2_rn(a, b, make_float2(-w.x, -w.y));
+        const float2 t = __fadd2_rn(s, w), bb = __ffma2_rn(m1, s, t);
+        const float2 u = __ffma2_rn(m1, __ffma2_rn(m1, bb, t), s), z = __ffma2_rn(m1, bb, w);
+        e = __fadd2_rn(e, __fadd2_rn(__fadd2_rn(u, z), we));
+        s = t;
+    }
+    __device__ __forceinline__ void add(float x, float v, float s, float c)
+    {
+        dot2(p, pe, make_float2(x, x), make_float2(x, v));
+        dot2(q, qe, make_float2(s, c), make_float2(v, 1.0f));
+    }
+    __device__ __forceinline__ static void merge1(float &s, float &e, int off)
+    {
+        CSum o;
+        o.s = __shfl_xor_sync(0xffffffffu, s, off);
+        o.e = __shfl_xor_sync(0xffffffffu, e, off);
+        o = csum_merge(CSum{s, e}, o);
+        s = o.s;
+        e = o.e;
+    }
+    __device__ __forceinline__ void merge(int G)
+    {
+        for (int off = G >> 1; off > 0; off >>= 1) {
+            merge1(p.x, pe.x, off);
+            merge1(p.y, pe.y, off);
+            merge1(q.x, qe.x, off);
+            merge1(q.y, qe.y, off);
+        }
+    }
+    // (s + e) / n, rounded once but for the last bits of the small terms
+    __device__ __forceinline__ static float over_n(float s, float e, const AckConst &n)
+    {
+        return __fmaf_rn(n.hi[0], s, __fmaf_rn(n.hi[0], e, n.lo[0] * s));
+    }
+    __device__ __forceinline__ AckTail<float> tail(const AckConst &n, bool) const
+    {
+        return ack_tail_f(over_n(p.x, pe.x, n), over_n(q.y, qe.y, n), n);
+    }
+    __device__ __forceinline__ float x() const { return __fadd_rn(p.y, pe.y); }
+    __device__ __forceinline__ float y() const { return __fadd_rn(q.x, qe.x); }
+    // squares whose TwoProd error underflows: the point goes the dense way
+    // (FP64 sums)
+    __device__ __forceinline__ bool small() const { return p.x < 1e-30f; }
+};
+
 // H v of one point by the G lanes of an aligned group of its warp, EPL
 // variables per lane (variable t + G j), n <= G EPL.
 template <typename T, typename IO, int EPL>
@@ -387,8 +486,7 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
     const int m = active ? n : 0;
     const Turn<T> turn;
     T xs[EPL], vs[EPL], sn[EPL], cs[EPL];
-    double S = 0.0, C = 0.0;
-    RowSum<T> xv, sv;
+    AckSums<T> sum;
 #pragma unroll
     for (int j = 0; j < EPL; ++j) {
         const int k = t + G * j;
@@ -403,26 +501,15 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
     for (int j = 0; j < EPL; ++j) {
         if (G * j < n) {  // uniform in the group
             turn(xs[j], sn[j], cs[j]);
-            if (t + G * j < m) {
-                const double xd = widen(xs[j]);
-                S = fma(xd, xd, S);
-                C += widen(cs[j]);
-                xv.add(xs[j], vs[j]);
-                sv.add(sn[j], vs[j]);
-            }
+            if (t + G * j < m) sum.add(xs[j], vs[j], sn[j], cs[j]);
         }
     }
-    for (int off = G >> 1; off > 0; off >>= 1) {
-        S += __shfl_xor_sync(0xffffffffu, S, off);
-        C += __shfl_xor_sync(0xffffffffu, C, off);
-        xv.merge_xor(off);
-        sv.merge_xor(off);
-    }
-    bool bad = false;
-    const AckTail<T> k = ack_tail(S, C, nc, G > 1, T(0));
+    sum.merge(G);
+    const AckTail<T> k = sum.tail(nc, G > 1);
+    bool bad = active && sum.small();
     if (active) {
         // f1 h + (f2 d1) g of S/2 plus q1 h + (q2 d1) g of C
-        const T f1 = k.f1(), fx = k.f2() * xv.value(), qs = k.q2 * sv.value();
+        const T f1 = k.f1(), fx = k.f2() * sum.x(), qs = k.q2 * sum.y();
 #pragma unroll
         for (int j = 0; j < EPL; ++j) {
             if (t + G * j < n) {
