@@ -27,8 +27,8 @@
  *    a function's terms use error-free transformations (TwoProd by FMA,
  *    TwoSum), and the sums whose cancellation matters -- the Fletcher-Powell
  *    residuals E_m - sum_j(...) and the Ackley sums under sqrt and exp -- are
- *    computed in FP64 once per point (the Ackley sums of the structured H v as
- *    Dot2 and Sum2, twice FP32's precision, in about the same bits).  Fletcher-Powell A, B, E are always
+ *    computed in FP64 once per point (the structured H v forms the Ackley sums
+ *    as Dot2 and Sum2, as accurate as sums in twice FP32's precision).  Fletcher-Powell A, B, E are always
  *    double.
  *  - csize (the chunk size) must be one of 1, 2, 4, 8, 16, 32, or 0 for
  *    "choose for me".  A call that names neither a chunk size nor a method
@@ -191,7 +191,8 @@ CHESSFAD_API int chessfad_hessian_config(int fn, int n, long long batch, const c
                             void *H, const chessfad_fp_params *params, int prec, chessfad_stream_t stream);
 
 /* chessfad_hvp for x, v and out in HOST memory, end to end: the batch is cut
- * into `slices` contiguous parts (0 = 8; at most 64; at most batch); part k's
+ * into `slices` contiguous parts (0 = 8, or with csize
+ * 0 one per 8 MiB of x and v up to 8; at most 64; at most batch); part k's
  * x and v are copied host -> device, its HVPs computed (as chessfad_hvp with
  * csize) and its out copied device -> host, with part k's sweep overlapping
  * the copies of its neighbours (internal copy and compute streams of the
