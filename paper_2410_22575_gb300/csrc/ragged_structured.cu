@@ -24,7 +24,9 @@ namespace {
 constexpr int kThreads = kFpThreads;
 
 // 4000 requests, n log-uniform in 2 .. 512, compensated FP32: dense 308 ms, here
-// 0.437 ms, bound by the FP64 residuals of the large Fletcher-Powell requests.
+// 0.270 ms.  The FP64 FMAs of the residuals, nearly all of them in the
+// Fletcher-Powell requests of n >= 128, need 0.106 ms; the rest is the latency
+// of the large requests' parts (one part alone takes 55 us, 16 of them FP64).
 
 // The tile functions are calls, so that each has registers of its own: inlined
 // into one kernel, the FP64 and many-variable variants made all of them spill.
@@ -57,7 +59,7 @@ __device__ __noinline__ void lanes_tile(const SRaggedArgs &a, const STile &t)
     }
 }
 
-template <typename T, typename IO>
+template <typename T, typename IO, bool kWide>
 __device__ __noinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile &t, unsigned char *smem)
 {
     __shared__ int s_last;
@@ -78,7 +80,7 @@ __device__ __noinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile &t
     }
     __syncthreads();
     FpSums<T, 2> sums[kFpNpt];
-    tile.run(t.m0, t.m1, sums);
+    tile.template run<kWide>(t.m0, t.m1, sums);
     if (t.parts > 1) {
         double *slot = a.slots + t.slot + (long long)t.part * 4 * t.pairs;
 #pragma unroll
@@ -101,14 +103,19 @@ __device__ __noinline__ void fp_ragged_tile(const SRaggedArgs &a, const STile &t
         const int u = threadIdx.x + i * kThreads;
         if (u >= t.pairs) break;
         T f[4];
-        for (int k = 0; k < 4; ++k) {
-            if (t.parts > 1) {
-                double s = 0.0;
-                for (int p = 0; p < t.parts; ++p) s += __ldcg(&a.slots[t.slot + ((long long)p * 4 + k) * t.pairs + u]);
-                f[k] = (T)s;
-            } else {
-                f[k] = sums[i].value(k);
-            }
+        if (t.parts > 1) {
+            // every part's four sums, the loads of four parts in flight
+            const double *slot = a.slots + t.slot + u;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+            for (int p = 0; p < t.parts; ++p)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s[k] += __ldcg(slot + ((long long)p * 4 + k) * t.pairs);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) f[k] = (T)s[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) f[k] = sums[i].value(k);
         }
         const T o = tile.combine(u, f[0], f[1], f[2], f[3]);
         bad |= not_finite(o);
@@ -130,10 +137,11 @@ __global__ void __launch_bounds__(kThreads, 2) structured_ragged_kernel(const __
         if (s_tile >= a.ntiles) break;
         const STile t = a.tiles[s_tile];
         if (IsComp<T>::value && t.f64) {
-            if (t.fn == FN_FP) fp_ragged_tile<double, T>(a, t, smem_raw);
+            if (t.fn == FN_FP) fp_ragged_tile<double, T, false>(a, t, smem_raw);
             else lanes_tile<double, T>(a, t);
         } else {
-            if (t.fn == FN_FP) fp_ragged_tile<T, T>(a, t, smem_raw);
+            if (t.fn == FN_FP && t.bufs == 0) fp_ragged_tile<T, T, true>(a, t, smem_raw);
+            else if (t.fn == FN_FP) fp_ragged_tile<T, T, false>(a, t, smem_raw);
             else lanes_tile<T, T>(a, t);
         }
     }

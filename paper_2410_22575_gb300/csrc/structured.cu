@@ -3,7 +3,7 @@
 //
 // H v through the default call, GB300, dense symmetric method -> here:
 //   Ackley n = 64, FP64, 65536 points            102.2 ms -> 0.256 ms
-//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.143 ms
+//   Ackley n = 64, FP32-comp, 524288 points       15.9 ms -> 0.119 ms
 //   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.086 ms
 //   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.115 ms
 // Hessians:
@@ -17,6 +17,7 @@
 // words, coefficients come from registers (fp64_sincos.cuh).
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "structured.cuh"
 #include "structured.h"
@@ -26,6 +27,7 @@ namespace chessfad {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kAckThreads = 128;  // small CTAs: the last round of CTAs is short
 constexpr long long kMaxBlocks = 0x7fffffffLL;
 
 template <typename T, typename IO>
@@ -39,18 +41,18 @@ __global__ void __launch_bounds__(kThreads) ros_hvp_kernel(const StructArgs a, i
                      a.n, t, G, active, a.wide);
 }
 
-template <typename T, typename IO, int EPL>
-__global__ void __launch_bounds__(kThreads) ack_hvp_kernel(const StructArgs a, int G, const AckConst nc)
+template <typename T, typename IO, int EPL, bool kVec = false>
+__global__ void __launch_bounds__(kAckThreads) ack_hvp_kernel(const StructArgs a, int G, const AckConst nc)
 {
-    const long long p = ((long long)blockIdx.x * kThreads + threadIdx.x) / G;
+    const long long p = ((long long)blockIdx.x * kAckThreads + threadIdx.x) / G;
     const int t = threadIdx.x & (G - 1);
     const bool active = p < a.batch;
     const size_t o = active ? (size_t)p * a.n : 0;
-    ack_point<T, IO, EPL>(static_cast<const IO *>(a.x) + o, static_cast<const IO *>(a.v) + o,
+    ack_point<T, IO, EPL, kVec>(static_cast<const IO *>(a.x) + o, static_cast<const IO *>(a.v) + o,
                           static_cast<IO *>(a.out) + o, a.n, t, G, active, a.wide, nc);
 }
 
-template <typename T, typename IO>
+template <typename T, typename IO, bool kWide>
 __global__ void __launch_bounds__(kFpThreads) fp_hvp_kernel(const StructArgs a, const FpShape sh, int ppb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(kFpThreads) fp_hvp_kernel(const StructArgs a, 
     }
     __syncthreads();
     FpSums<T, 2> sums[kFpNpt];
-    tile.run(0, n, sums);
+    tile.template run<kWide>(0, n, sums);
     bool bad = false;
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
@@ -240,7 +242,7 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
 // cos again would take that launch as long as its products.
 constexpr int kGramSmall = 64;
 __device__ __forceinline__ int beside(int l, int k, int n) { return l + k < n ? l + k : l + k - n; }
-template <typename T, typename IO>
+template <typename T, typename IO, bool kWide>
 __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructArgs a, const FpShape sh, int ppb)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructAr
     }
     __syncthreads();
     FpSums<T, 1> sums[kFpNpt];
-    tile.run(0, n, sums);
+    tile.template run<kWide>(0, n, sums);
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
@@ -465,11 +467,23 @@ cudaError_t ack_launch(const StructArgs &a, int G, unsigned blocks, cudaStream_t
 {
     const int it = (a.n + G - 1) / G;
     const AckConst nc = ack_const(a.n);
-    if (it <= 1) ack_hvp_kernel<T, IO, 1><<<blocks, kThreads, 0, s>>>(a, G, nc);
-    else if (it <= 2) ack_hvp_kernel<T, IO, 2><<<blocks, kThreads, 0, s>>>(a, G, nc);
-    else if (it <= 4) ack_hvp_kernel<T, IO, 4><<<blocks, kThreads, 0, s>>>(a, G, nc);
-    else if (it <= 8) ack_hvp_kernel<T, IO, 8><<<blocks, kThreads, 0, s>>>(a, G, nc);
-    else ack_hvp_kernel<T, IO, 16><<<blocks, kThreads, 0, s>>>(a, G, nc);
+    if constexpr (std::is_same<T, float>::value) {
+        // whole 16-byte pieces per lane (a quarter of the load, store and
+        // predicate instructions of a kernel bound by instruction issue:
+        // n = 64, 524288 points, 143 -> 119 us with AckSums' halved merges)
+        const size_t bits = (size_t)a.x | (size_t)a.v | (size_t)a.out;
+        if (it > 2 && a.n % 4 == 0 && bits % 16 == 0) {
+            if (it <= 4) ack_hvp_kernel<T, IO, 4, true><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+            else if (it <= 8) ack_hvp_kernel<T, IO, 8, true><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+            else ack_hvp_kernel<T, IO, 16, true><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+            return cudaGetLastError();
+        }
+    }
+    if (it <= 1) ack_hvp_kernel<T, IO, 1><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+    else if (it <= 2) ack_hvp_kernel<T, IO, 2><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+    else if (it <= 4) ack_hvp_kernel<T, IO, 4><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+    else if (it <= 8) ack_hvp_kernel<T, IO, 8><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
+    else ack_hvp_kernel<T, IO, 16><<<blocks, kAckThreads, 0, s>>>(a, G, nc);
     return cudaGetLastError();
 }
 
@@ -496,15 +510,15 @@ int fp_points(int n, long long batch, int fmas)
     return best;
 }
 
-template <typename T, typename IO, bool kHvp>
-cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
+template <typename T, typename IO, bool kHvp, bool kWide>
+cudaError_t fp_launch_as(const StructArgs &a, cudaStream_t s)
 {
     const int ppb = fp_points(a.n, a.batch, sizeof(T) == 8 ? (kHvp ? 8 : 4) : 2);
     const FpShape sh = fp_shape(a.n, a.n, ppb, ppb * a.n, sizeof(T) == 8);
     const size_t bytes = fp_smem<T>(sh).total;
     const long long blocks = (a.batch + ppb - 1) / ppb;
     if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
-    auto kern = kHvp ? fp_hvp_kernel<T, IO> : fp_curvature_kernel<T, IO>;
+    auto kern = kHvp ? fp_hvp_kernel<T, IO, kWide> : fp_curvature_kernel<T, IO, kWide>;
     static std::atomic<int> configured[64];
     const cudaError_t e = opt_in_smem(kern, bytes, configured);
     if (e != cudaSuccess) return e;
@@ -512,12 +526,18 @@ cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <typename T, typename IO, bool kHvp>
+cudaError_t fp_launch(const StructArgs &a, cudaStream_t s)
+{
+    return a.n >= kFpWide ? fp_launch_as<T, IO, kHvp, true>(a, s) : fp_launch_as<T, IO, kHvp, false>(a, s);
+}
+
 template <typename T, typename IO>
 cudaError_t hvp(int fn, const StructArgs &a, cudaStream_t s)
 {
     if (fn == FN_FP) return fp_launch<T, IO, true>(a, s);
     const int G = fn == FN_ROSENBROCK ? ros_lanes(a.n) : ack_lanes(a.n, a.batch, sizeof(T) == 8);
-    const long long ppb = kThreads / G, blocks = (a.batch + ppb - 1) / ppb;
+    const long long ppb = (fn == FN_ACKLEY ? kAckThreads : kThreads) / G, blocks = (a.batch + ppb - 1) / ppb;
     if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
     if (fn == FN_ACKLEY) return ack_launch<T, IO>(a, G, (unsigned)blocks, s);
     ros_hvp_kernel<T, IO><<<(unsigned)blocks, kThreads, 0, s>>>(a, G);

@@ -451,14 +451,43 @@ struct AckSums<float> {
         s = o.s;
         e = o.e;
     }
+    // From 4 lanes on, each lane keeps two of the four sums at the first
+    // distance and one at the second, and fetches the others at the end: 3 +
+    // log2(G / 4) merges instead of 4 log2(G).
     __device__ __forceinline__ void merge(int G)
     {
-        for (int off = G >> 1; off > 0; off >>= 1) {
-            merge1(p.x, pe.x, off);
-            merge1(p.y, pe.y, off);
-            merge1(q.x, qe.x, off);
-            merge1(q.y, qe.y, off);
+        if (G < 4) {
+            for (int off = G >> 1; off > 0; off >>= 1) {
+                merge1(p.x, pe.x, off);
+                merge1(p.y, pe.y, off);
+                merge1(q.x, qe.x, off);
+                merge1(q.y, qe.y, off);
+            }
+            return;
         }
+        const int lane = threadIdx.x & 31, a = G >> 1, b = G >> 2;
+        const bool ha = lane & a, hb = lane & b;
+        CSum k0 = half(ha, CSum{p.x, pe.x}, CSum{q.x, qe.x}, a), k1 = half(ha, CSum{p.y, pe.y}, CSum{q.y, qe.y}, a);
+        k0 = half(hb, k0, k1, b);
+        for (int off = b >> 1; off > 0; off >>= 1) merge1(k0.s, k0.e, off);
+        const int at = lane & ~(G - 1);
+        p.x = __shfl_sync(0xffffffffu, k0.s, at);
+        pe.x = __shfl_sync(0xffffffffu, k0.e, at);
+        p.y = __shfl_sync(0xffffffffu, k0.s, at + b);
+        pe.y = __shfl_sync(0xffffffffu, k0.e, at + b);
+        q.x = __shfl_sync(0xffffffffu, k0.s, at + a);
+        qe.x = __shfl_sync(0xffffffffu, k0.e, at + a);
+        q.y = __shfl_sync(0xffffffffu, k0.s, at + a + b);
+        qe.y = __shfl_sync(0xffffffffu, k0.e, at + a + b);
+    }
+    // x (high: y) merged with the partner's
+    __device__ __forceinline__ static CSum half(bool high, const CSum &x, const CSum &y, int off)
+    {
+        const CSum keep = high ? y : x, give = high ? x : y;
+        CSum o;
+        o.s = __shfl_xor_sync(0xffffffffu, give.s, off);
+        o.e = __shfl_xor_sync(0xffffffffu, give.e, off);
+        return csum_merge(keep, o);
     }
     // (s + e) / n, rounded once but for the last bits of the small terms
     __device__ __forceinline__ static float over_n(float s, float e, const AckConst &n)
@@ -476,32 +505,73 @@ struct AckSums<float> {
     __device__ __forceinline__ bool small() const { return p.x < 1e-30f; }
 };
 
+// A load the compiler may not replace by the value of an earlier one.
+__device__ __forceinline__ double load_again(const double *p)
+{
+    double r;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(r) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ float load_again(const float *p)
+{
+    float r;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(r) : "l"(p));
+    return r;
+}
+
 // H v of one point by the G lanes of an aligned group of its warp, EPL
-// variables per lane (variable t + G j), n <= G EPL.
-template <typename T, typename IO, int EPL>
+// variables per lane, n <= G EPL: variable t + G j, or, kVec (float, n a
+// multiple of 4, 16-byte aligned x, v, out), four neighbours at a time.
+template <typename T, typename IO, int EPL, bool kVec = false>
 __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__restrict__ v, IO *__restrict__ out,
                                           int n, int t, int G, bool active, bool wide,
                                           const AckConst &nc)
 {
     const int m = active ? n : 0;
     const Turn<T> turn;
-    T xs[EPL], vs[EPL], sn[EPL], cs[EPL];
+    constexpr int V = kVec ? 4 : 1;
+    auto var = [&](int j) { return V == 1 ? t + G * j : 4 * (t + G * (j / 4)) + j % 4; };
+    // FP64 with many variables per lane: x and v are read again (from L1) for
+    // the tail instead of held in 4 EPL registers, so that twice the warps
+    // keep the FP64 pipe filled.
+    constexpr bool kReload = sizeof(T) == 8 && EPL >= 8;
+    constexpr int kHeld = kReload ? 1 : EPL;
+    T xs[kHeld], vs[kHeld], sn[EPL], cs[EPL];
     AckSums<T> sum;
+    if constexpr (kVec) {
 #pragma unroll
-    for (int j = 0; j < EPL; ++j) {
-        const int k = t + G * j;
-        xs[j] = T(0);
-        vs[j] = T(0);
-        if (k < m) {
-            xs[j] = (T)x[k];
-            vs[j] = (T)v[k];
+        for (int j = 0; j < EPL; j += 4) {
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (var(j) < m) {
+                a = *reinterpret_cast<const float4 *>(x + var(j));
+                b = *reinterpret_cast<const float4 *>(v + var(j));
+            }
+            xs[j] = a.x, xs[j + 1] = a.y, xs[j + 2] = a.z, xs[j + 3] = a.w;
+            vs[j] = b.x, vs[j + 1] = b.y, vs[j + 2] = b.z, vs[j + 3] = b.w;
+        }
+    } else if constexpr (!kReload) {
+#pragma unroll
+        for (int j = 0; j < EPL; ++j) {
+            const int k = var(j);
+            xs[j] = T(0);
+            vs[j] = T(0);
+            if (k < m) {
+                xs[j] = (T)x[k];
+                vs[j] = (T)v[k];
+            }
         }
     }
 #pragma unroll
     for (int j = 0; j < EPL; ++j) {
-        if (G * j < n) {  // uniform in the group
-            turn(xs[j], sn[j], cs[j]);
-            if (t + G * j < m) sum.add(xs[j], vs[j], sn[j], cs[j]);
+        if (V * G * (j / V) < n) {  // uniform in the group
+            const bool on = var(j) < m;
+            if constexpr (kReload) {
+                xs[0] = on ? (T)x[t + G * j] : T(0);
+                vs[0] = on ? (T)v[t + G * j] : T(0);
+            }
+            const T xj = xs[kReload ? 0 : j], vj = vs[kReload ? 0 : j];
+            turn(xj, sn[j], cs[j]);
+            if (on) sum.add(xj, vj, sn[j], cs[j]);
         }
     }
     sum.merge(G);
@@ -510,14 +580,26 @@ __device__ __forceinline__ void ack_point(const IO *__restrict__ x, const IO *__
     if (active) {
         // f1 h + (f2 d1) g of S/2 plus q1 h + (q2 d1) g of C
         const T f1 = k.f1(), fx = k.f2() * sum.x(), qs = k.q2 * sum.y();
+        T o4[V];
 #pragma unroll
         for (int j = 0; j < EPL; ++j) {
-            if (t + G * j < n) {
-                T o = fma_(fx, xs[j], f1 * vs[j]);
+            if (var(j) < n) {
+                T xj, vj;
+                if constexpr (kReload) {
+                    xj = (T)load_again(x + t + G * j);
+                    vj = (T)load_again(v + t + G * j);
+                } else {
+                    xj = xs[j];
+                    vj = vs[j];
+                }
+                T o = fma_(fx, xj, f1 * vj);
                 o = fma_(qs, sn[j], o);
-                o = fma_(k.q1, cs[j] * vs[j], o);
+                o = fma_(k.q1, cs[j] * vj, o);
                 bad |= not_finite(o);
-                out[t + G * j] = (IO)o;
+                o4[j % V] = o;
+                if constexpr (!kVec) out[var(j)] = (IO)o;
+                else if (j % 4 == 3)
+                    *reinterpret_cast<float4 *>(out + var(j - 3)) = make_float4(o4[0], o4[1], o4[2], o4[3]);
             }
         }
     }
@@ -549,9 +631,10 @@ constexpr int kFpMaxPts = 128;
 struct FpShape {
     int nmax;   // largest n of the tile's points
     int mt;     // rows of A, B per shared-memory tile
-    int bufs;   // tile buffers: 2 when the rows take several tiles
+    int bufs;   // tile buffers: 2 when the rows take several tiles; 0: wide rows
     int pairs;  // (point, variable) pairs the shared arrays hold
-    int lanes;  // lanes per (point, row) in pass 1, a power of two <= 32
+    int lanes;  // lanes per (point, row) in pass 1, a power of two <= 32; wide
+                // rows: (point, row) items per warp, 2 or 4
 };
 
 // Two values read and multiplied together: (A, B) of one (m, j), (sin, cos)
@@ -588,7 +671,8 @@ __host__ __device__ inline FpSmem<T> fp_smem(const FpShape &sh)
     s.t = take(np * sizeof(Two<T>));
     s.rd = take(np * sizeof(Two<T>));
     s.ab = take(tile * sizeof(Two<double>));
-    s.fab = sizeof(T) == 4 ? take(tile * sizeof(Two<T>)) : s.ab;
+    s.fab = s.ab;
+    if (sizeof(T) == 4) s.fab = take((sh.bufs ? tile : (size_t)sh.mt * fp_stride(sh.nmax)) * sizeof(Two<T>));
     s.n = take(kFpMaxPts * sizeof(int));
     s.base = take((kFpMaxPts + 1) * sizeof(int));
     s.q = take(np);
@@ -828,11 +912,183 @@ struct FpTile {
         }
     }
 
+    // Wide rows (few points per CTA): A and B come straight from L2.  A warp
+    // takes S (point, row) items at a time, its lanes the columns; after a
+    // barrier the threads add the items' rows to their columns, in compensated
+    // FP32 from the rounded rows that pass 1 left in shared memory.
+    template <int S>
+    __device__ __forceinline__ void run_wide(int m0, int m1, FpSums<T, NS> (&sums)[kFpNpt])
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = fp_stride(sh.nmax), chunk = sh.mt;
+        for (int mb = m0; mb < m1; mb += chunk) {
+            const int mend = min(mb + chunk, m1), items = (mend - mb) * P;
+            __syncthreads();  // sin and cos are staged; the last chunk's rows are read
+            double s[S], s2[S];
+            FpSums<T, 1> d[S];
+            int z0[S], n[S], row[S];
+            const double *Ar[S], *Br[S];
+            bool put[S];
+#pragma unroll
+            for (int v = 0; v < S; ++v) {
+                // a row's points on neighbouring slots; its first point leaves
+                // the rounded row (the points are ordered by size)
+                const int idx = warp * S + v, q = idx < items ? idx % P : 0, m = mb + (idx < items ? idx / P : 0);
+                z0[v] = base[q];
+                n[v] = idx < items && m < ns[q] ? ns[q] : 0;
+                put[v] = sizeof(T) == 4 && idx < items && q == 0;
+                row[v] = (m - mb) * w;
+                Ar[v] = a.A + (size_t)m * a.ld;
+                Br[v] = a.B + (size_t)m * a.ld;
+                s[v] = s2[v] = 0.0;
+                d[v].init();
+            }
+            int blk = 0;
+            // 64 columns at a time, the next ones' loads under this one's sums
+            double av[2][S], bv[2][S], an[2][S], bn[2][S];
+            auto fetch = [&](int j0, double (&x)[2][S], double (&y)[2][S]) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int v = 0; v < S; ++v) {
+                        const int j = j0 + 32 * h;
+                        x[h][v] = y[h][v] = 0.0;
+                        if (j < (put[v] ? sh.nmax : n[v])) {
+                            x[h][v] = __ldg(Ar[v] + j);
+                            y[h][v] = __ldg(Br[v] + j);
+                        }
+                    }
+            };
+            constexpr bool kAhead = S == 2;  // four items have loads enough, and registers for no more
+            if (kAhead) fetch(lane, an, bn);
+            for (int j0 = lane; j0 < sh.nmax; j0 += 64) {
+                if constexpr (kAhead) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int v = 0; v < S; ++v) {
+                            av[h][v] = an[h][v];
+                            bv[h][v] = bn[h][v];
+                        }
+                    fetch(j0 + 64, an, bn);
+                } else {
+                    fetch(j0, av, bv);
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int v = 0; v < S; ++v) {
+                        const int j = j0 + 32 * h;
+                        const Two<T> g{narrow<T>(av[h][v]), narrow<T>(bv[h][v])};
+                        if (put[v] && j < sh.nmax) fab[row[v] + j] = g;
+                        if (j < n[v]) {
+                            const Two<double> zz = z[z0[v] + j];
+                            s[v] = fma(av[h][v], zz.x, s[v]);
+                            s2[v] = fma(bv[h][v], zz.y, s2[v]);
+                            if constexpr (kDir) {
+                                const Two<T> tt = t[z0[v] + j];
+                                d[v].add(0, g, tt.x, tt.y);
+                            }
+                        }
+                    }
+                blk += 2;
+                if (kDir && blk == kSumBlock) {
+                    blk = 0;
+#pragma unroll
+                    for (int v = 0; v < S; ++v) d[v].flush();
+                }
+            }
+            // Across the lanes: halve the slots a lane holds at distances 16
+            // and, with four, 8 (6 additions for four sums, 5 for two).
+            RowSum<T> e[S];
+#pragma unroll
+            for (int v = 0; v < S; ++v) {
+                s[v] += s2[v];
+                if constexpr (kDir) d[v].flush();
+                e[v] = d[v].both();
+            }
+            const bool h16 = lane & 16, h8 = lane & 8;
+#pragma unroll
+            for (int v = 0; v < S / 2; ++v) {
+                fold(s[v], s[v + S / 2], h16, 16);
+                if constexpr (kDir) fold_row(e[v], e[v + S / 2], h16, 16);
+            }
+            if constexpr (S == 4) {
+                fold(s[0], s[1], h8, 8);
+                if constexpr (kDir) fold_row(e[0], e[1], h8, 8);
+            }
+            for (int off = S == 4 ? 4 : 8; off > 0; off >>= 1) {
+                s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
+                if constexpr (kDir) e[0].merge_xor(off);
+            }
+            const int idx = warp * S + (S == 4 ? (h16 ? 2 : 0) + (h8 ? 1 : 0) : (h16 ? 1 : 0));
+            if ((lane & (S == 4 ? 7 : 15)) == 0 && idx < items) {
+                const int q = idx % P, m = mb + idx / P;
+                if (m < ns[q])
+                    rd[base[q] + m] = Two<T>{narrow<T>(a.E[eoff[q] + m] - s[0]), kDir ? -e[0].value() : T(0)};
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < kFpNpt; ++i) {
+                const int u = threadIdx.x + i * kFpThreads;
+                if (u >= npairs) break;
+                const int q = qs[u], l = u - base[q], end = min(mend, ns[q]);
+                const Two<T> *f = rd + base[q], *g = fab + l;
+                const double *Al = a.A + l, *Bl = a.B + l;
+                auto term = [&](int m) {
+                    const Two<T> ff = f[m];
+                    Two<T> gg;
+                    if constexpr (sizeof(T) == 4) {
+                        gg = g[(m - mb) * w];
+                    } else {
+                        gg.x = __ldg(Al + (size_t)m * a.ld);
+                        gg.y = __ldg(Bl + (size_t)m * a.ld);
+                    }
+                    sums[i].add(0, gg, ff.x, ff.x);
+                    if constexpr (kDir) sums[i].add(1, gg, ff.y, ff.y);
+                };
+                int m = mb;
+                for (; m + kSumBlock <= end; m += kSumBlock) {
+#pragma unroll
+                    for (int k = 0; k < kSumBlock; ++k) term(m + k);
+                    sums[i].flush();
+                }
+                for (; m < end; ++m) term(m);
+                sums[i].flush();
+            }
+        }
+        __syncthreads();
+    }
+    // lanes with `high` keep b, the others a, each adding its partner's part
+    __device__ __forceinline__ static void fold(double &x, double &y, bool high, int off)
+    {
+        const double keep = high ? y : x, give = high ? x : y;
+        x = keep + __shfl_xor_sync(0xffffffffu, give, off);
+    }
+    __device__ __forceinline__ static void fold_row(RowSum<double> &x, RowSum<double> &y, bool high, int off)
+    {
+        fold(x.s, y.s, high, off);
+    }
+    __device__ __forceinline__ static void fold_row(RowSum<float> &x, RowSum<float> &y, bool high, int off)
+    {
+        const CSum keep = high ? y.s : x.s, give = high ? x.s : y.s;
+        CSum o;
+        o.s = __shfl_xor_sync(0xffffffffu, give.s, off);
+        o.e = __shfl_xor_sync(0xffffffffu, give.e, off);
+        x.s = csum_merge(keep, o);
+    }
+
     // Rows m0 <= m < m1.  The next tile's copy runs under this tile's passes.
+    template <bool kWide>
     __device__ __forceinline__ void run(int m0, int m1, FpSums<T, NS> (&sums)[kFpNpt])
     {
 #pragma unroll
         for (int i = 0; i < kFpNpt; ++i) sums[i].init();
+        if constexpr (kWide) {
+            stage();
+            if (sh.lanes == 4) run_wide<4>(m0, m1, sums);
+            else run_wide<2>(m0, m1, sums);
+            return;
+        }
         load_tile(0, m0, min(m0 + sh.mt, m1));
         stage();
         int buf = 0;

@@ -46,6 +46,12 @@ inline int ack_lanes(int n, long long batch, bool f64)
     return best;
 }
 
+// From this n on (at most 4 points per CTA) the rows of A and B are read from
+// L2 instead of through a shared-memory tile: the tile would hold a few rows
+// only, too few items for the CTA's warps between two barriers (4000 uneven
+// requests up to n = 512: 426 us with tiles, 270 so).
+constexpr int kFpWide = 128;
+
 // The shape of an FpTile: rows rows of A and B for P points, pairs pairs; f64:
 // FP64 arithmetic.  All rows in one buffer within 48 KiB, else even parts of
 // them in two buffers (two or more CTAs per SM).
@@ -57,6 +63,14 @@ inline FpShape fp_shape(int nmax, int rows, int P, int pairs, bool f64)
     s.pairs = pairs;
     s.bufs = 1;
     s.mt = rows;
+    if (nmax >= kFpWide) {
+        // rows per barrier: the CTA's warps' items, 4 per warp (fewer FP64
+        // additions across lanes) while the rounded rows fit 64 KiB
+        s.bufs = 0;
+        s.lanes = nmax <= 256 ? 4 : 2;
+        s.mt = kFpThreads / 32 * s.lanes / P;
+        return s;
+    }
     if ((size_t)rows * row > 48 * 1024) {
         const int most = std::max(1, (int)(40 * 1024 / row));
         const int tiles = (rows + most - 1) / most;
