@@ -160,6 +160,43 @@ def load_counts() -> dict:
     return {k: v for k, v in tj.get("kernels", {}).items() if tj.get("source_hash") == h}
 
 
+# The structured evaluation (the default call): its kernels, the counts file of
+# its own capture, and the key of a workload's entry.
+STRUCTURED_SOURCES = ("structured.cuh", "fp64_sincos.cuh", "structured.cu", "structured_tune.h", "hdual.cuh")
+STRUCTURED_COUNTS_FILE = os.path.join(ROOT, "profiles", "counts_structured.json")
+STRUCTURED_KERNELS = {0: ("ros_hvp_kernel", "ros_hessian_kernel"), 1: ("ack_hvp_kernel", "ack_hessian_kernel"),
+                      2: ("fp_hvp_kernel", "fp_gram_kernel")}
+
+
+def structured_source_hash() -> str:
+    h = hashlib.sha256()
+    csrc = os.path.join(ROOT, "paper_2410_22575_gb300", "csrc")
+    for name in STRUCTURED_SOURCES:
+        h.update(code_tokens(open(os.path.join(csrc, name)).read()).encode())
+    return h.hexdigest()[:16]
+
+
+def load_structured_counts() -> dict:
+    """Executed FP operations and DRAM bytes per point of the default call's
+    kernels (ncu), dropped when their sources have changed since."""
+    if not os.path.exists(STRUCTURED_COUNTS_FILE):
+        return {}
+    tj = json.load(open(STRUCTURED_COUNTS_FILE))
+    return tj.get("kernels", {}) if tj.get("source_hash") == structured_source_hash() else {}
+
+
+def structured_key(workload: str, prec: int, kind: str) -> str:
+    return f"{workload}/{PREC_NAME[prec]}/{kind}/structured"
+
+
+def structured_model_flops(fn: int, n: int, kind: str) -> float:
+    """Operations of the structured evaluation's rules (FMA = 2), sin and cos
+    at 40, without the per-point scalar functions."""
+    if kind == "hessian":
+        return {0: 16.0 * n, 1: 4.0 * n * n + 50.0 * n, 2: float(n) ** 3 + 12.0 * n * n}[fn]
+    return {0: 20.0 * n, 1: 56.0 * n, 2: 16.0 * n * n + 60.0 * n}[fn]
+
+
 def count_key(workload: str, prec: int, kind: str, method: str, c: int) -> str:
     return f"{workload}/{PREC_NAME[prec]}/{kind}/{method}/c{c}"
 
@@ -351,8 +388,10 @@ def _checked(st, what):
 
 
 def headline_arm(cf, b, prec, args, world, dev, stream, flush, peaks, counts):
-    """The named workload in one precision: autotuned HVP config, K timed
-    steps (clocks sampled), then the same through host buffers (e2e)."""
+    """The named workload in one precision: the default call (structured
+    evaluation), K timed steps (clocks sampled), the dense evaluation in its
+    autotuned configuration beside it, then the default call through host
+    buffers (e2e)."""
     import torch
 
     dt = torch.float64 if prec == cf.FP64 else torch.float32
@@ -374,14 +413,25 @@ def headline_arm(cf, b, prec, args, world, dev, stream, flush, peaks, counts):
     barrier(world)
     tot = max_over_ranks(world, sum(ms), dev)
     per = tot / len(ms)
-    cd = cfg.as_dict()
-    sym = cd["method"] == "symmetric"
-    key = count_key(WORKLOAD, prec, "hvp", cd["method"], cfg.csize)
-    roof = roofline_entry(counts, key, batch, sum(ms) / len(ms), prec, peaks, n, "hvp",
-                          model_flops_hvp(fn, n, cfg.csize, sym), kernel_name(cd["method"], prec, cfg.csize, fn, "hvp"))
+    roof = roofline_entry(load_structured_counts(), structured_key(WORKLOAD, prec, "hvp"), batch, sum(ms) / len(ms),
+                          prec, peaks, n, "hvp", structured_model_flops(fn, n, "hvp"), STRUCTURED_KERNELS[fn][0])
     res = {"value": world * batch / (per * 1e-3), "unit": "HVP/s", "steps": len(ms), "ms_per_step": per,
-           "config": cd, "roofline": roof, "clocks": clocks, "_out": out.double().cpu().numpy(),
-           "_x": x.double().cpu().numpy(), "_v": v.double().cpu().numpy()}
+           "config": {"evaluation": "structured (csize 0, the default call)"}, "roofline": roof, "clocks": clocks,
+           "_out": out.double().cpu().numpy(), "_x": x.double().cpu().numpy(), "_v": v.double().cpu().numpy()}
+
+    # the dense chunked evaluation, in the configuration the autotuner picks
+    def dense_step():
+        _checked(cf.chessfad_hvp_config(fn, n, batch, cfg, x, v, out, None, prec, stream), "chessfad_hvp_config")
+
+    k = max(1, min(5, args.steps))
+    m = timed_steps(dense_step, k, 1, stream, flush)
+    t = max_over_ranks(world, sum(m), dev) / k
+    cd = cfg.as_dict()
+    res["dense"] = {"hvp_per_s": world * batch / (t * 1e-3), "ms": t, "launch": cd, "steps": k,
+                    "roofline": roofline_entry(counts, count_key(WORKLOAD, prec, "hvp", cd["method"], cfg.csize), batch,
+                                               sum(m) / k, prec, peaks, n, "hvp",
+                                               model_flops_hvp(fn, n, cfg.csize, cd["method"] == "symmetric"),
+                                               kernel_name(cd["method"], prec, cfg.csize, fn, "hvp"))}
 
     # chunk-size sweep (shorter), same precision, both methods
     sweep = {}
@@ -449,6 +499,8 @@ def headline_arm(cf, b, prec, args, world, dev, stream, flush, peaks, counts):
 # n=16) is quoted in FP64 with c=4 by the plain method, HVP and Hessian; C3
 # (Fletcher-Powell n=32) in FP64 and in compensated FP32 (FP64 residuals);
 # C4 (Rosenbrock n=256) HVP and Hessian, autotuned, in both precisions.
+# Both are dense configurations; each tuned row carries the default call (the
+# structured evaluation) beside it.
 WORKLOAD_ROWS = (
     ("rosenbrock_n16", "hvp", "stated", 0),
     ("rosenbrock_n16", "hessian", "stated", 0),
@@ -519,6 +571,23 @@ def workloads_arm(cf, args, world, dev, stream, flush, peaks, counts):
                ("hvp_per_s" if kind == "hvp" else "hessians_per_s"): rate, "ms": per, "steps": len(ms),
                "roofline": roof}
         row["_out"] = out.double().cpu().numpy() if kind == "hvp" else out.cpu().numpy()
+        if how == "tuned":
+            def default_step():
+                if kind == "hvp":
+                    st = cf.chessfad_hvp(b.fn, b.n, b.batch, 0, x, v, out, params, prec, stream)
+                else:
+                    st = cf.chessfad_hessian(b.fn, b.n, b.batch, 0, x, out, params, prec, stream)
+                _checked(st, "default call")
+
+            ms = timed_steps(default_step, k, 2, stream, flush)
+            per = max_over_ranks(world, sum(ms), dev) / len(ms)
+            row["default_call"] = {
+                ("hvp_per_s" if kind == "hvp" else "hessians_per_s"): world * b.batch / (per * 1e-3), "ms": per,
+                "roofline": roofline_entry(load_structured_counts(), structured_key(name, prec, kind), b.batch,
+                                           sum(ms) / len(ms), prec, peaks, b.n, kind,
+                                           structured_model_flops(b.fn, b.n, kind),
+                                           STRUCTURED_KERNELS[b.fn][0 if kind == "hvp" else 1])}
+            row["_out_default"] = out.double().cpu().numpy() if kind == "hvp" else out.cpu().numpy()
         row["_x"] = x.double().cpu().numpy()
         row["_v"] = v.double().cpu().numpy()
         row["_b"] = b
@@ -574,6 +643,7 @@ def gpu_arm(args):
         "data": "synthetic (seeded PCG64 draws of the workload's distributions)",
         "config": config,
         "launch": f64["config"],
+        "dense": f64["dense"],
         "roofline": f64["roofline"],
         "e2e": f64["e2e"],
         "gpu_launches": f64["steps"],
@@ -581,7 +651,7 @@ def gpu_arm(args):
         "fp32_comp": {"value": f32["value"], "unit": "HVP/s", "dtype": "f32",
                       "precision": "FP32 hDual arithmetic with compensated sums and dots, FP64 islands",
                       "steps": f32["steps"], "ms_per_step": f32["ms_per_step"], "launch": f32["config"],
-                      "roofline": f32["roofline"], "e2e": f32["e2e"], "clocks": f32["clocks"]},
+                      "dense": f32["dense"], "roofline": f32["roofline"], "e2e": f32["e2e"], "clocks": f32["clocks"]},
         "fp32_over_fp64": f32["value"] / f64["value"],
         "chunk_sweep": {"fp64": f64["chunk_sweep"], "fp32_comp": f32["chunk_sweep"]},
         "seed_sparse": {"fp64": f64["seed_sparse"], "fp32_comp": f32["seed_sparse"],
@@ -602,6 +672,9 @@ def gpu_arm(args):
         line["fp32_comp"]["error_vs_oracle"] = headline_error(f32, 1)
         for k, r in rows.items():
             line["workloads"][k]["error_vs_oracle"] = workload_error(r)
+            if "_out_default" in r:
+                line["workloads"][k]["default_call"]["error_vs_oracle"] = workload_error(
+                    {**r, "_out": r["_out_default"]})
         if ragged is not None:
             e, t_all = ragged_error_all(ragged)
             line["ragged_100k"]["error_vs_oracle"] = e
@@ -670,10 +743,9 @@ def model_flops_request(fn: int, n: int, c: int) -> float:
 
 def ragged_arm(args, world, dev, stream, flush):
     """The 100000-request uneven batch (three functions, n log-uniform in
-    [2, 512], seed 4) in compensated FP32: the library's uneven-batch
-    autotuner picks (chunk size, lanes per row) per (function, n range), then
-    one persistent launch per step, replayed from a captured CUDA graph.  The
-    default (untuned) plan is timed once beside it."""
+    [2, 512], seed 4) in compensated FP32: one persistent launch per step of a
+    plan without a chunk size (the structured evaluation), replayed from a
+    captured CUDA graph.  The dense plan is timed once beside it."""
     import numpy as np
     import torch
 
@@ -702,40 +774,28 @@ def ragged_arm(args, world, dev, stream, flush):
         barrier(world)
         return max_over_ranks(world, sum(ms), dev), len(ms)
 
-    default_plan = cf.RaggedPlan(reqs, cf.FP32_COMP, 16)
-    t_default, _ = (None, 0) if args.no_ragged_default else time_plan(default_plan, 1)
-    ws = default_plan.workspace
-    t0 = time.perf_counter()
-    ngroups = cf.chessfad_ragged_autotune(reqs, cf.FP32_COMP, x, v, out, params, ws, ws.numel())
-    t_tune = time.perf_counter() - t0
-    del default_plan, ws
     t0 = time.perf_counter()
     plan = cf.RaggedPlan(reqs, cf.FP32_COMP, 0)
     t_plan = time.perf_counter() - t0
     tot, steps = time_plan(plan, args.ragged_steps)
-    groups = {}
-    flops = 0.0
-    for f in (0, 1, 2):
-        for b in range(1, 9):
-            lo, hi = 1 << b, min(512, (2 << b) - 1) if b < 8 else 512
-            sel = (rg.fns == f) & (rg.ns >= lo) & (rg.ns <= hi)
-            if not sel.any():
-                continue
-            c, tpr, mt = cf.chessfad_ragged_plan_group_config(plan.handle, f, int(rg.ns[sel][0]))
-            groups[f"{W.FN_NAMES[f]}/n{lo}-{hi}"] = {"csize": c, "threads_per_row": tpr, "requests": int(sel.sum()),
-                                                    **({"ab_tile_rows_at_n": [int(rg.ns[sel][0]), mt]}
-                                                       if f == 2 else {})}
-            flops += sum(model_flops_request(f, int(n), c) for n in rg.ns[sel])
+    got = out.double().cpu().numpy()
+    # the dense evaluation of the same requests (chunk size 16), once
+    t_dense, dense_tflops = None, None
+    if not args.no_ragged_default:
+        dense_plan = cf.RaggedPlan(reqs, cf.FP32_COMP, 16)
+        t_dense, _ = time_plan(dense_plan, 1)
+        flops = sum(model_flops_request(int(f), int(n), 16) for f, n in zip(rg.fns, rg.ns))
+        dense_tflops = flops / (t_dense * 1e-3) / 1e12
     per = tot / steps
     return {"value": world * rg.nreq * steps / (tot * 1e-3), "unit": "HVP/s", "requests": rg.nreq,
             "steps": steps, "warmup": 1, "ms_per_step": per, "precision": "fp32_comp",
             "launch": "one persistent kernel per step, CUDA graph replay", "tiles": plan.info["ntiles"],
-            "method": "plain; symmetric (SC-HESS-VEC) for Fletcher-Powell n >= 128",
-            "tuned_groups": groups, "autotune_seconds": t_tune, "groups_tuned": ngroups,
-            "untuned_ms_per_step": t_default, "untuned_config": "csize 16, default lanes per row",
+            "method": "structured (plan without a chunk size)",
+            "untuned_ms_per_step": t_dense, "dense_model_tflops": dense_tflops,
+            "untuned_config": "dense evaluation, csize 16, default lanes per row; plain, symmetric (SC-HESS-VEC) "
+                              "for Fletcher-Powell n >= 128",
             "workspace_bytes": plan.info["workspace_bytes"], "plan_seconds": t_plan,
-            "model_tflops": flops / (per * 1e-3) / 1e12,
-            "_out": out.double().cpu().numpy(), "_x": x.double().cpu().numpy(), "_v": v.double().cpu().numpy(),
+            "_out": got, "_x": x.double().cpu().numpy(), "_v": v.double().cpu().numpy(),
             "_rg": rg, "_c": 16}  # the oracle's CHESS-VEC chunk size for the CPU baseline
 
 
@@ -1464,7 +1524,7 @@ def main():
     ap.add_argument("--block", type=int, default=128)
     ap.add_argument("--ref-budget", type=float, default=100.0,
                     help="reference arm: seconds of oracle work over all steps (bounded per step)")
-    ap.add_argument("--e2e-slices", type=int, default=16,
+    ap.add_argument("--e2e-slices", type=int, default=0,
                     help="slices of the end-to-end call (copies of one overlap the sweep of the next)")
     ap.add_argument("--method", choices=["plain", "symmetric", "symmetric_sparse"], default="plain")
     ap.add_argument("--tpp", type=int, default=64, help="kernel-only, symmetric: threads per point")

@@ -131,6 +131,42 @@ def test_points_are_independent(fn):
     assert np.array_equal(Hv.cpu().numpy(), d.hessian(), equal_nan=True)
 
 
+@pytest.mark.parametrize("prec", PRECS)
+def test_fletcher_powell_several_points_per_cta_with_wide_rows(prec):
+    """A batch that puts four points of n = 128 into a CTA (rows of A and B
+    read past shared memory) and leaves a CTA with fewer."""
+    d = Dev(W.make_batch(W.FLETCHER_POWELL, 128, 1215, seed=6), prec)
+    assert hvp_err(d, d.hvp()).max() <= BOUND[prec]
+
+
+@pytest.mark.parametrize("n", [12, 64, 128])
+def test_ackley_fp32_off_the_16_byte_grid(n):
+    """n a multiple of 4 with x, v and out 4 bytes off a 16-byte boundary, one
+    at a time: the loads go element by element."""
+    import torch
+
+    d = Dev(W.make_batch(W.ACKLEY, n, 100, seed=n), cf.FP32_COMP)
+    for which in range(3):
+        t = [torch.empty(100 * n + 4, dtype=torch.float32, device="cuda") for _ in range(3)]
+        x, v, out = [b[int(i == which):][:100 * n].view(100, n) for i, b in enumerate(t)]
+        x.copy_(d.x)
+        v.copy_(d.v)
+        cf.hvp(W.ACKLEY, x, v, out=out)
+        e = hvp_err(d, out.double().cpu().numpy())
+        assert e.max() <= BOUND[cf.FP32_COMP], (which, e.max())
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_fletcher_powell_arguments_beyond_the_reduction(prec):
+    """x on both sides of the range that sin and cos reduce themselves."""
+    b = W.make_batch(W.FLETCHER_POWELL, 17, 60, seed=12)
+    b.x[:30] *= 1e4
+    b.x[30:] *= 1e7
+    d = Dev(b, prec)
+    assert hvp_err(d, d.hvp()).max() <= BOUND[prec]
+    assert hessian_err(d, d.hessian()).max() <= BOUND[prec]
+
+
 class _Uneven:
     """An uneven batch of the given functions and sizes and its plan (csize 0)."""
 
