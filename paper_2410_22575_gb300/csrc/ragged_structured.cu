@@ -24,7 +24,7 @@ namespace {
 constexpr int kThreads = kFpThreads;
 
 // 4000 requests, n log-uniform in 2 .. 512, compensated FP32: dense 308 ms, here
-// 0.270 ms.  The FP64 FMAs of the residuals, nearly all of them in the
+// 0.257 ms.  The FP64 FMAs of the residuals, nearly all of them in the
 // Fletcher-Powell requests of n >= 128, need 0.106 ms; the rest is the latency
 // of the large requests' parts (one part alone takes 55 us, 16 of them FP64).
 
@@ -176,9 +176,12 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
     double total = 0.0;
     for (long long e = 0; e < nreq; ++e)
         total += reqs[order[e]].fn == CHESSFAD_FLETCHER_POWELL ? fp_cost(pl.n[e]) : (f64 ? 50.0 : 4.0) * pl.n[e];
-    // a tile larger than this is split: about an eighth of an SM's share of
-    // the batch, and at least 15 us of its FP64 pipe (2 FMAs a clock)
-    const double most = std::max(62000.0, total / (152.0 * 8.0));
+    // a tile larger than this is split: about a quarter of an SM's share of
+    // the batch, and at least 15 us of its FP64 pipe (2 FMAs a clock).  4000
+    // requests up to n = 512: a sixteenth 268 us, an eighth 268, a quarter 257;
+    // at least 7.5 us 258, 15 us 257, 30 us 256; one request of n = 505: 64, 65
+    // and 85 us.
+    const double most = std::max(62000.0, total / (152.0 * 4.0));
     std::vector<std::pair<double, STile>> work;
     for (long long e = 0; e < nreq;) {
         const int fn = reqs[order[e]].fn, g = group(order[e]), nmax = pl.n[e];
