@@ -7,9 +7,9 @@
 //   Fletcher-Powell n = 32, FP32-comp, 16384       1.83 ms -> 0.086 ms
 //   Fletcher-Powell n = 75, FP64, 1000            151.7 ms -> 0.115 ms
 // Hessians:
-//   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.082 ms (6.6 TB/s written)
+//   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.076 ms (7.0 TB/s written)
 //   Ackley n = 33, FP32-comp, 20000                0.178 ms -> 0.035 ms
-//   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.111 ms
+//   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.107 ms
 // The Rosenbrock kernels stream; the others are bound by the FP64 pipe (sin,
 // cos and the sums under sqrt and exp; the residuals), in compensated FP32 too.
 // It takes one warp instruction per 16 clocks and SM, so what is not FP64
@@ -132,7 +132,13 @@ __global__ void __launch_bounds__(kThreads) ros_hessian_kernel(const StructArgs 
         if ((unsigned)d <= 2u) v = d == 1 ? diag[r] : d == 2 ? up[r] : lo[r];
         return v;
     };
-    stream_rows(H, cnt, n, fd, val);
+    stream_rows(H, cnt, n, fd, val, [&](int r, int j, IO *q) {
+        const int d = j - ls[r];  // -1, 0, 1: the row's entries
+        const T a0 = lo[r], a1 = diag[r], a2 = up[r];
+#pragma unroll
+        for (int i = 0; i < 16 / (int)sizeof(IO); ++i)
+            q[i] = (IO)(d + i == -1 ? a0 : d + i == 0 ? a1 : d + i == 1 ? a2 : T(0));
+    });
 }
 
 // ppc whole points per CTA, or, split > 1, one of `split` parts of one
@@ -225,7 +231,19 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
         if (w == u) v += dg[u];
         return v;
     };
-    stream_rows(H, r1 - r0, n, fd, val);
+    stream_rows(H, r1 - r0, n, fd, val, [&](int r, int j, IO *q) {
+        const int u = r + r0, w = (split > 1 ? 0 : fd.div(u) * n) + j;
+        const Pair above = ab[u], below = xs[u];
+        const T d = dg[u];
+#pragma unroll
+        for (int i = 0; i < 16 / (int)sizeof(IO); ++i) {
+            const bool left = w + i < u;
+            const Pair e = (left ? ab : xs)[w + i], f = left ? below : above;
+            T v = fma_(f.x, e.x, f.s * e.s);
+            if (w + i == u) v += d;
+            q[i] = (IO)v;
+        }
+    });
     bool any = false;
     for (int q = tid; q < npts; q += kThreads) any |= flag[q] != 0;
     if (__syncthreads_or(any))
@@ -358,7 +376,19 @@ __global__ void __launch_bounds__(kThreads) fp_gram_small_kernel(const StructArg
             }
     }
     __syncthreads();
-    stream_rows(H, nv, n, fd, [&](int row, int j) { return J[(size_t)row * np + j]; });
+    stream_rows(
+        H, nv, n, fd, [&](int row, int j) { return J[(size_t)row * np + j]; },
+        [&](int row, int j, IO *q) {
+            constexpr int V = 16 / (int)sizeof(IO);
+            Two<T> p[V / 2];  // n even: np and j are too
+#pragma unroll
+            for (int i = 0; i < V / 2; ++i) p[i] = *reinterpret_cast<const Two<T> *>(J + (size_t)row * np + j + 2 * i);
+#pragma unroll
+            for (int i = 0; i < V / 2; ++i) {
+                q[2 * i] = (IO)p[i].x;
+                q[2 * i + 1] = (IO)p[i].y;
+            }
+        });
     if (__syncthreads_or(bad))
         for (int k = 0; k < npts; ++k) {
             bool b = false;

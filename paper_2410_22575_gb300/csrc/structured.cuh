@@ -1213,16 +1213,40 @@ struct FastDiv {
 };
 
 // The elements of `rows` consecutive Hessian rows of n, out[r n + j] =
-// val(r, j), with 16-byte streaming stores where the address allows.  Every
-// thread of the CTA calls it.
-template <typename IO, typename F>
-__device__ __forceinline__ void stream_rows(IO *out, int rows, int n, FastDiv fd, F &&val)
+// val(r, j), with 16-byte streaming stores where the address allows.  When
+// every store lies in one row (n a multiple of the store's values, out aligned)
+// vec(r, j, q) gives its values together, with what the row shares read once.
+// Every thread of the CTA calls it.
+template <typename IO, typename F, typename G>
+__device__ __forceinline__ void stream_rows(IO *out, int rows, int n, FastDiv fd, F &&val, G &&vec)
 {
     using Vec = typename std::conditional<sizeof(IO) == 8, double2, float4>::type;
     constexpr int V = 16 / (int)sizeof(IO);
     const int cnt = rows * n;
     const int mis = (int)(((16 - ((size_t)out & 15)) & 15) / sizeof(IO));
     const int head = mis < cnt ? mis : cnt, nvec = (cnt - head) / V;
+    auto put = [&](int e, const IO(&q)[V]) {
+        Vec o;
+        if constexpr (V == 2) {
+            o.x = q[0];
+            o.y = q[1];
+        } else {
+            o.x = q[0];
+            o.y = q[1];
+            o.z = q[2];
+            o.w = q[3];
+        }
+        __stcs(reinterpret_cast<Vec *>(out + e), o);
+    };
+    if (n % V == 0 && head == 0) {
+        for (int w = threadIdx.x; w < nvec; w += blockDim.x) {
+            const int e = w * V, r = fd.div(e);
+            IO q[V];
+            vec(r, e - r * n, q);
+            put(e, q);
+        }
+        return;
+    }
     auto one = [&](int e) {
         const int r = fd.div(e);
         out[e] = (IO)val(r, e - r * n);
@@ -1240,17 +1264,7 @@ __device__ __forceinline__ void stream_rows(IO *out, int rows, int n, FastDiv fd
                 ++r;
             }
         }
-        Vec o;
-        if constexpr (V == 2) {
-            o.x = q[0];
-            o.y = q[1];
-        } else {
-            o.x = q[0];
-            o.y = q[1];
-            o.z = q[2];
-            o.w = q[3];
-        }
-        __stcs(reinterpret_cast<Vec *>(out + e), o);
+        put(e, q);
     }
     for (int e = head + nvec * V + threadIdx.x; e < cnt; e += blockDim.x) one(e);
 }

@@ -156,6 +156,21 @@ def test_ackley_fp32_off_the_16_byte_grid(n):
         assert e.max() <= BOUND[cf.FP32_COMP], (which, e.max())
 
 
+@pytest.mark.parametrize("fn", FNS)
+@pytest.mark.parametrize("prec", PRECS)
+def test_hessian_stores_whole_rows_or_not(fn, prec):
+    """n a multiple of the values of a 16-byte store: an aligned output (a
+    store's values together) and one that starts one element later (one by
+    one) hold the same bits."""
+    import torch
+
+    for n in (4, 20, 64, 68):
+        d = Dev(W.make_batch(fn, n, 37, seed=n), prec)
+        flat = torch.empty(37 * n * n + 1, dtype=d.x.dtype, device="cuda")
+        H = cf.hessian(fn, d.x, params=d.params, prec=prec, out=flat[1:].view(37, n, n))
+        assert np.array_equal(H.double().cpu().numpy(), d.hessian())
+
+
 @pytest.mark.parametrize("prec", PRECS)
 def test_fletcher_powell_arguments_beyond_the_reduction(prec):
     """x on both sides of the range that sin and cos reduce themselves."""
