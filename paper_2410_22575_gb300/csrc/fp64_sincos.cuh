@@ -96,10 +96,11 @@ __device__ __forceinline__ void sincos_rad(const SinCosK &k, double x, double &s
     sincos_quadrant(__double2loint(m), __fma_rn(r * z, sincos_p(k, z), r), sincos_q(k, z), s, c);
 }
 
-// sin 2 pi x, cos 2 pi x
+// sin 2 pi x, cos 2 pi x.  4x + 1.5 * 2^52 rounds to an integer while it lies
+// between 2^52 and 2^53, that is for |4x| <= 2^51.
 __device__ __forceinline__ void sincos_turn(const SinCosK &k, double x, double &s, double &c)
 {
-    if (((unsigned)__double2hiint(x) & 0x7fffffffu) >= 0x43100000u) {  // |x| >= 2^50, Inf, NaN
+    if (((unsigned)__double2hiint(x) & 0x7fffffffu) >= 0x43000000u) {  // |x| >= 2^49, Inf, NaN
         sincospi(2.0 * x, &s, &c);
         return;
     }

@@ -1,0 +1,53 @@
+"""Inputs at the edges of what the structured evaluation's own arithmetic
+covers: the end of the range that its sine and cosine reduce themselves, one
+variable, values below the normal float range, parameters that are finite in
+FP64 only."""
+import math
+
+import numpy as np
+import pytest
+
+import paper_2410_22575_gb300 as cf
+from paper_2410_22575_gb300 import workloads as W
+
+from gpu_helpers import BOUND, Dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _ackley_far(x, v):
+    """H and H v of Ackley at points with a variable so large that
+    exp(-0.2 sqrt(S/n)) is 0: (4 pi^2/n) exp(C/n) (diag(cos) - sin sin^T / n),
+    the angles from the exact fractional parts."""
+    n = x.shape[1]
+    t = x - np.rint(x)
+    s, c = np.sin(2 * math.pi * t), np.cos(2 * math.pi * t)
+    k = 4 * math.pi ** 2 / n * np.exp(c.mean(1))
+    H = k[:, None, None] * (np.eye(n)[None] * c[:, None, :] - s[:, :, None] * s[:, None, :] / n)
+    return H, np.einsum("pij,pj->pi", H, v)
+
+
+@pytest.mark.parametrize("n", [1, 2, 5, 64, 130])
+def test_ackley_fp64_large_arguments(n):
+    """|x| on both sides of 2^49 and 2^50, beyond which 4x + 1.5 * 2^52 is no
+    longer rounded to an integer, and beyond which the units of x are whole
+    turns; H v, Hessian and uneven request."""
+    import torch
+
+    far = [2.0 ** 47 + 0.25, 2.0 ** 48, 2.0 ** 49 - 0.25, 2.0 ** 49, 2.0 ** 49 + 0.5, 9e14 + 1, 2.0 ** 50 - 0.5,
+           2.0 ** 50, 2.0 ** 51 + 1]
+    far = np.array(far + [-t for t in far])
+    b = W.make_batch(W.ACKLEY, n, len(far), seed=60 + n)
+    b.x[np.arange(len(far)), np.arange(len(far)) % n] = far
+    d = Dev(b, cf.FP64)
+    H, Hv = _ackley_far(d.xh, d.vh)
+    scale = np.sqrt((H * H).sum((1, 2)))
+    out = d.hvp()
+    assert np.all(np.linalg.norm(out - Hv, axis=1) <= BOUND[cf.FP64] * scale * np.linalg.norm(d.vh, axis=1))
+    assert np.all(np.sqrt(((d.hessian() - H) ** 2).sum((1, 2))) <= BOUND[cf.FP64] * scale)
+    plan = cf.RaggedPlan(cf.requests([W.ACKLEY] * len(far), [n] * len(far), np.arange(len(far)) * n), cf.FP64)
+    packed = torch.empty_like(d.x)
+    plan.run(d.x, d.v, packed)
+    torch.cuda.synchronize()
+    got = packed.cpu().numpy()
+    assert np.all(np.linalg.norm(got - Hv, axis=1) <= BOUND[cf.FP64] * scale * np.linalg.norm(d.vh, axis=1))
