@@ -269,7 +269,10 @@ __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs 
 // (FP64 residuals), written to the diagonal of H.  For 3 <= n <= kGramSmall it
 // also leaves sin x_l and cos x_l beside it, at columns l + 1 and l + 2 (mod
 // n), where the second launch reads them before it overwrites H: FP64 sin and
-// cos again would take that launch as long as its products.
+// cos again would take that launch as long as its products.  One variable in
+// compensated FP32 (T double, IO float): the whole entry 2 J^2 + curvature,
+// whose terms can cancel, is formed here in FP64, rounded once, and there is no
+// second launch.
 constexpr int kGramSmall = 64;
 __device__ __forceinline__ int beside(int l, int k, int n) { return l + k < n ? l + k : l + k - n; }
 template <typename T, typename IO, bool kWide>
@@ -292,6 +295,25 @@ __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructAr
     __syncthreads();
     FpSums<T, 1> sums[kFpNpt];
     tile.template run<kWide>(0, n, sums);
+    if constexpr (!std::is_same<T, IO>::value) {
+        IO *H = static_cast<IO *>(a.out) + p0;
+        bool bad = false;
+#pragma unroll
+        for (int i = 0; i < kFpNpt; ++i) {
+            const int u = threadIdx.x + i * kFpThreads;
+            if (u >= P) break;
+            const T j = fp_jacobian<T>(a.A[0], a.B[0], tile.z[u].x, tile.z[u].y);
+            const IO h = (IO)fma_(T(2) * j, j, tile.curvature(u, sums[i]));
+            bad |= not_finite(h);
+            H[u] = h;
+        }
+        if (__syncthreads_or(bad))
+            for (int q = 0; q < P; ++q)
+                if (not_finite(H[q]))
+                    fp_dense_hessian<T, IO>(FpArgs{a.A, a.B, a.E, a.ld}, static_cast<const IO *>(a.x) + p0 + q, H + q,
+                                            1, tile.z, tile.rd);
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
@@ -597,7 +619,7 @@ cudaError_t fp_hessian(const StructArgs &a, FastDiv fd, cudaStream_t s)
     const int nbk = (n + kGramTile - 1) / kGramTile, nt = nbk * (nbk + 1) / 2;
     if (n > kGramSmall && a.batch > kMaxBlocks / nt) return cudaErrorInvalidConfiguration;
     cudaError_t e = fp_launch<T, IO, false>(a, s);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !std::is_same<T, IO>::value) return e;  // one variable: the entry is whole
     static std::atomic<int> small_smem[64], gram_attr[64];
     if (n <= kGramSmall) {
         const int nb = (n + 3) / 4, np = 4 * nb, tiles = nb * (nb + 1) / 2;

@@ -51,3 +51,26 @@ def test_ackley_fp64_large_arguments(n):
     torch.cuda.synchronize()
     got = packed.cpu().numpy()
     assert np.all(np.linalg.norm(got - Hv, axis=1) <= BOUND[cf.FP64] * scale * np.linalg.norm(d.vh, axis=1))
+
+
+def test_fletcher_powell_one_variable_hessian_many_points():
+    """n = 1 in compensated FP32: the entry 2 J^2 + 2 r P, whose terms cancel at
+    some points, is formed in FP64 and rounded once, at each of 200000 points;
+    where a value is not finite it is what the dense method gives."""
+    b = W.make_batch(W.FLETCHER_POWELL, 1, 200000, seed=9)
+    b.x[5, 0], b.x[6, 0], b.x[7, 0] = np.nan, np.inf, -np.inf
+    d = Dev(b, cf.FP32_COMP)
+    H = d.hessian()[:, 0, 0]
+    A, B, E = float(b.fp.A[0, 0]), float(b.fp.B[0, 0]), float(b.fp.E[0])
+    x = d.xh[:, 0]
+    with np.errstate(invalid="ignore"):
+        s, c = np.sin(x), np.cos(x)
+    ref = 2 * (A * c - B * s) ** 2 + 2 * (E - A * s - B * c) * (A * s + B * c)
+    ok = np.isfinite(ref)
+    assert np.all(np.isnan(H[~ok]))
+    assert np.max(np.abs(H[ok] - ref[ok]) / np.abs(ref[ok])) <= BOUND[cf.FP32_COMP]
+    for which in range(3):
+        b = W.make_batch(W.FLETCHER_POWELL, 1, 300, seed=9)
+        (b.fp.A, b.fp.B, b.fp.E)[which].flat[0] = np.inf
+        d = Dev(b, cf.FP32_COMP)
+        assert np.array_equal(d.hessian(), d.hessian(cfg=cf.Config(1, 1, 256)), equal_nan=True)
