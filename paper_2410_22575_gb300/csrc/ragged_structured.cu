@@ -183,10 +183,11 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
     // and 85 us.
     const double most = std::max(62000.0, total / (152.0 * 4.0));
     std::vector<std::pair<double, STile>> work;
+    long long end = 0;  // of the current tile's group
     for (long long e = 0; e < nreq;) {
-        const int fn = reqs[order[e]].fn, g = group(order[e]), nmax = pl.n[e];
-        long long end = e;
-        while (end < nreq && group(order[end]) == g) ++end;  // the group
+        const int fn = reqs[order[e]].fn, nmax = pl.n[e];
+        if (e == end)
+            while (end < nreq && group(order[end]) == group(order[e])) ++end;
         STile t{};
         t.fn = fn;
         t.first = (int)e;
