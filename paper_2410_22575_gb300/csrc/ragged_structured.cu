@@ -155,11 +155,12 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
     // entries: by function, one-variable requests apart (in compensated FP32
     // they are computed in FP64), then by size, largest first
     std::vector<int> order(nreq);
-    std::iota(order.begin(), order.end(), 0);
     auto group = [&](int q) { return 2 * reqs[q].fn + (reqs[q].n == 1); };
-    std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
-        return group(p) != group(q) ? group(p) < group(q) : reqs[p].n > reqs[q].n;
-    });
+    auto key = [&](long long q) { return group((int)q) * (kMaxVars + 1) + kMaxVars - reqs[q].n; };
+    std::vector<long long> at(6 * (kMaxVars + 1) + 1, 0);  // counting sort: where each key starts
+    for (long long q = 0; q < nreq; ++q) ++at[key(q) + 1];
+    std::partial_sum(at.begin(), at.end(), at.begin());
+    for (long long q = 0; q < nreq; ++q) order[at[key(q)]++] = (int)q;
     pl.n.resize(nreq);
     pl.off.resize(nreq);
     pl.eoff.resize(nreq);
