@@ -268,7 +268,8 @@ __device__ __noinline__ void user_dense_rows(const T *xp, const T *vp, T *out, i
 // Bound by the arithmetic of f: its functions of values, once per chunk, and the
 // active components.  The extended-operator test function, n = 64, C = 8, FP64,
 // 4096 points: symmetric method 100.7 ms; every component of every number 2.83
-// ms; active components 1.67 ms; one power instead of three per pow() 1.31 ms.
+// ms; active components 1.67 ms; two powers instead of three in an inactive
+// pow() 1.34 ms.
 // Errors against the oracle (FP32, n = 19 and 64, rms over the test functions):
 // 1.0 to 1.24 times the symmetric method's, below 1.7e-7.
 template <typename T, int C>

@@ -286,15 +286,17 @@ __device__ __forceinline__ Num<T, C, A> sqrt(const Num<T, C, A> &u)
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> pow(const Num<T, C, A> &u, double p)
 {
-    // One power and two products (each correctly rounded) where u and the
-    // power are positive and far from the ends of the range; the three powers
-    // themselves elsewhere (zero, negative, overflow, underflow, NaN).
-    const T q = T(p), x = u.a.v, w = m_pow(x, q - T(2)), big = sizeof(T) == 8 ? T(1e75) : T(1e9);
-    T w1 = w * x, w0 = w1 * x;
-    if (!(x > T(1) / big && x < big && w > T(1) / big && w < big)) {
-        w1 = m_pow(x, q - T(1));
-        w0 = m_pow(x, q);
-    }
+    // Three powers, so that each has pow()'s own accuracy (u^0 is 1 and the
+    // derivative of u^1 is 1).  A number outside the chunk uses phi'' only to notice that it is
+    // not finite; where u^(p-2) = u^(p-1) / u and its factor are far inside the
+    // range, that power is left out (the extended-operator test function, FP64,
+    // n = 64, 4096 points: 1.67 ms with three powers everywhere, 1.34 ms so).
+    const T q = T(p), x = u.a.v, big = sizeof(T) == 8 ? T(1e75) : T(1e9);
+    const T w0 = m_pow(x, q), w1 = m_pow(x, q - T(1));
+    T w = T(0);
+    if (!A || u.act ||
+        !(x > T(1) / big && x < big && w1 < big && w1 > -big && q < big && q > -big))
+        w = m_pow(x, q - T(2));
     return apply(u, w0, q * w1, q * (q - T(1)) * w);
 }
 template <typename T, int C, bool A>

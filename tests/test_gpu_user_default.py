@@ -1,0 +1,70 @@
+"""The default H v of a user function where it could differ from the methods by
+rows."""
+import numpy as np
+import pytest
+
+import paper_2410_22575_gb300 as cf
+
+from test_gpu_user import PLAIN, SYM
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec", [cf.FP64, cf.FP32_COMP])
+def test_first_and_zeroth_powers_are_exact(prec):
+    """pow(u, 0) is 1, the derivative of pow(u, 1) is 1 and, in FP32, pow(u, 1) is
+    u (CUDA's double pow(x, 1.0) is not x at 4 % of x): every entry of this
+    Hessian is 0 or 1 and, with whole v, every product a whole number."""
+    import torch
+
+    src = """template <class R, class X> R powers(const X &x, int n, const double *p)
+    {
+        R f = 0.0;
+        for (int k = 0; k < n; ++k) {
+            R a = pow(x[k], 1.0);
+            if ((p[0] != 0.0 && a != x[k]) || pow(x[k], 0.0) != 1.0) f += 1e3 * x[k] * x[k];
+            f += pow(x[k], 0.0) * x[k];
+            if (k + 1 < n) f += a * x[k + 1];
+        }
+        return f;
+    }"""
+    f = cf.UserFunction(src, "powers", 8, prec)
+    rng = np.random.Generator(np.random.PCG64(5))
+    n = 30
+    dt = torch.float64 if prec == cf.FP64 else torch.float32
+    x = torch.tensor(rng.uniform(0.1, 5, (300, n)), dtype=dt, device="cuda")
+    v = torch.tensor(rng.integers(-50, 51, (300, n)), dtype=dt, device="cuda")
+    p = torch.tensor([float(prec == cf.FP32_COMP)], dtype=torch.float64, device="cuda")
+    H = np.eye(n, k=1) + np.eye(n, k=-1)
+    ref = v.double().cpu().numpy() @ H
+    for cfg in (None, PLAIN, SYM):
+        assert np.array_equal(f.hvp(x, v, p, cfg=cfg).double().cpu().numpy(), ref), cfg
+    assert np.array_equal(f.hessian(x, p).double().cpu().numpy(), np.broadcast_to(H, (300, n, n)))
+
+
+@pytest.mark.parametrize("prec", [cf.FP64, cf.FP32_COMP])
+def test_powers_that_are_not_finite(prec):
+    """Zero, negative, huge and tiny arguments of pow at whole and other
+    exponents: the default product has the NaN and Inf of the plain method."""
+    import torch
+
+    src = """template <class R, class X> R mixed_powers(const X &x, int n, const double *p)
+    { R f = 0.0; for (int k = 0; k < n; ++k) f += pow(x[k], p[k]) * (1.0 + x[0]); return f; }"""
+    f = cf.UserFunction(src, "mixed_powers", 4, prec)
+    dt = torch.float64 if prec == cf.FP64 else torch.float32
+    big = 1e200 if prec == cf.FP64 else 1e30
+    powers = [0.0, 1.0, 1.5, 2.0, 3.0, -1.0, 0.5, 40.0]
+    n = len(powers)
+    rng = np.random.Generator(np.random.PCG64(6))
+    x = rng.uniform(0.1, 5, (48, n))
+    for k, val in enumerate((0.0, -0.0, -2.0, big, 1 / big, np.inf)):
+        x[8 * k + np.arange(8), np.arange(8)] = val
+    x = torch.tensor(x, dtype=dt, device="cuda")
+    v = torch.tensor(rng.uniform(-1, 1, (48, n)), dtype=dt, device="cuda")
+    p = torch.tensor(powers, dtype=torch.float64, device="cuda")
+    got, ref = (f.hvp(x, v, p, cfg=c).double().cpu().numpy() for c in (None, PLAIN))
+    assert np.array_equal(np.isfinite(got), np.isfinite(ref))
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    ok = np.isfinite(ref)
+    scale = np.max(np.abs(np.where(ok, ref, 0)), axis=1, keepdims=True) * np.ones_like(ref)
+    assert np.all(np.abs(got - ref)[ok] <= (4e-12 if prec == cf.FP64 else 4e-5) * scale[ok])
