@@ -490,10 +490,10 @@ CHESSFAD_API int chessfad_version(void);
  * stands).  params is the caller's device pointer, passed through (may be
  * NULL).  The arithmetic of f runs in the handle's precision: FP64, or FP32
  * (CHESSFAD_FP32_COMP: the function's own sums are plain FP32 as written; the
- * plain and symmetric methods' row-times-v reduction is compensated, the
- * default HVP has none; at n = 1, where the Hessian
- * is one entry whose terms can cancel, the arithmetic is FP64 with float
- * inputs and outputs).
+ * sums over the direction are compensated, the row-times-v reduction of the
+ * plain and symmetric methods and d1 and h of the default HVP; at n = 1, where
+ * the Hessian is one entry whose terms can cancel, the arithmetic is FP64 with
+ * float inputs and outputs).
  *
  * The default HVP evaluates f once per chunk with d1 seeded by v, so that the
  * h components are the chunk's rows of H v.  Two decompositions by rows, as for

@@ -12,6 +12,7 @@
 #include <dlfcn.h>
 #include <nvrtc.h>
 
+#include <algorithm>
 #include <cctype>
 #include <cstdio>
 #include <cstdlib>
@@ -35,6 +36,7 @@ struct chessfad_user_fn {
     cudaKernel_t hvp_n1 = nullptr;       // FP32 handles, n = 1: FP64 arithmetic, float I/O
     cudaKernel_t hessian_n1 = nullptr;
     int csize = 0;
+    int dir_csize = 0;  // the directional kernel's
     int prec = 0;
     std::mutex mu;
     unsigned long long smem_opted = 0;  // bit d: the symmetric kernels' shared-memory limit raised on device d
@@ -262,7 +264,7 @@ int launch(chessfad_user_fn *fn, const chessfad_config *cfg, bool hvp, int n, lo
         // of 128 threads: a warp's worth while x and v of that many fit 48
         // KiB, no more than the batch has
         const size_t elem = fn->prec == CHESSFAD_FP64 ? sizeof(double) : sizeof(float);
-        const long long nch = (n + fn->csize - 1) / fn->csize;
+        const long long nch = (n + fn->dir_csize - 1) / fn->dir_csize;
         int lanes = 32;
         while (lanes > 1 && ((size_t)(lanes + 1) * n * 2 * elem > 48 * 1024 || lanes >= 2 * batch)) lanes >>= 1;
         block = 128;
@@ -326,13 +328,18 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     text += source;
     text += "\n#include \"user_kernel.cuh\"\n";
     // The row methods and the directional kernel as two programs: compiled side
-    // by side they take about as long as the larger one.
+    // by side they take about as long as the larger one.  The directional kernel's
+    // chunk size is not part of its result; in FP32 its numbers take two floats
+    // per component of d1 and h, and chunks larger than 8 spill (the extended-
+    // operator function at csize 16, n = 64, 4096 points: 337 us with chunks of
+    // 16, 143 with 8).
+    const int dir_csize = prec == CHESSFAD_FP32_COMP ? std::min(csize, 8) : csize;
     Program prog[2];
     std::thread second;
     try {
         second = std::thread([&] {
             try {
-                compile_program(rt, text, name, csize, prec, true, prog[1]);
+                compile_program(rt, text, name, dir_csize, prec, true, prog[1]);
             } catch (...) {
                 prog[1].ok = false;  // out of memory
             }
@@ -341,7 +348,7 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     }
     compile_program(rt, text, name, csize, prec, false, prog[0]);
     if (second.joinable()) second.join();
-    else compile_program(rt, text, name, csize, prec, true, prog[1]);
+    else compile_program(rt, text, name, dir_csize, prec, true, prog[1]);
     for (const Program &p : prog)
         if (!p.ok) {
             put_log(log, log_bytes, p.log);
@@ -351,6 +358,7 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
 
     auto *fn = new chessfad_user_fn;
     fn->csize = csize;
+    fn->dir_csize = dir_csize;
     fn->prec = prec;
     cudaError_t e = cudaLibraryLoadData(&fn->lib, prog[0].cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
     if (e == cudaSuccess)

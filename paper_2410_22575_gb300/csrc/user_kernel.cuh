@@ -24,7 +24,8 @@
 //    finite, and points whose d1 or v is not, are evaluated again by the plain
 //    method.
 // FP32: the row-times-v products are summed as a Dot2 (TwoProd by FMA plus
-// TwoSum); the function's own arithmetic is plain FP32, as written by the
+// TwoSum), the directional d1 and h carry their errors the same way (Dir); the
+// rest of the function's own arithmetic is plain FP32, as written by the
 // user, except at n = 1 (FP64 arithmetic, float I/O).  FP64: fused
 // multiply-add accumulation.
 #pragma once
@@ -269,9 +270,10 @@ __device__ __noinline__ void user_dense_rows(const T *xp, const T *vp, T *out, i
 // active components.  The extended-operator test function, n = 64, C = 8, FP64,
 // 4096 points: symmetric method 100.7 ms; every component of every number 2.83
 // ms; active components 1.67 ms; two powers instead of three in an inactive
-// pow() 1.34 ms.
-// Errors against the oracle (FP32, n = 19 and 64, rms over the test functions):
-// 1.0 to 1.24 times the symmetric method's, below 1.7e-7.
+// pow() 1.30 ms.
+// FP32, C = 8: 81 us with plain sums over v, whose rms error was up to 1.27 times
+// the symmetric method's and grew with n; 143 us with Dir's (0.6 to 1.0 times; the
+// symmetric method takes 1555 us).
 template <typename T, int C>
 __device__ __forceinline__ void user_directional(const UserArgs &a)
 {
@@ -298,11 +300,11 @@ __device__ __forceinline__ void user_directional(const UserArgs &a)
     T *out = static_cast<T *>(a.out) + (p0 + q) * n;
     // stays 0 while the chunk's rows, d1 (which every skipped product's
     // factors reach) and v are finite
-    T zero = r.a.d1 * T(0);
+    T zero = r.a.d1.value() * T(0);
 #pragma unroll
     for (int l = 0; l < C; ++l) {
         if (cstart + l < n) {
-            const T h = r.act ? r.a.h[l] : T(0);
+            const T h = r.act ? r.a.h[l].value() : T(0);
             out[cstart + l] = h;
             zero += h * T(0);
         }

@@ -41,35 +41,125 @@ __device__ __forceinline__ double m_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float m_pow(float x, float p) { return powf(x, p); }
 __device__ __forceinline__ double m_pow(double x, double p) { return pow(x, p); }
 
-// A: whether the number tracks activity.  In one evaluation a variable outside
-// the chunk has zero g and h components, and so has everything computed from
-// such variables alone; with A the zeros are neither stored nor multiplied
-// (act is false), only the value and d1 are.  A skipped product would be an
-// exact zero unless its other factor is Inf or NaN.  Such a factor makes d1
-// not finite, at the latest through the phi''(u) * 0 that the unary rule adds,
-// and d1 stays so in whatever is computed from it; callers look at the
-// result's d1.
+// A derivative along the direction v (see DirVars): a sum over the variables.
+// In FP32 it carries its rounding errors in e as Dot2 does (TwoProd, TwoSum), so
+// that the sums over v are as accurate as the compensated row-times-v sums of
+// the methods by rows; in FP64 it is one double.
+template <typename T>
+struct Dir;
+template <>
+struct Dir<double> {
+    double s;
+    __device__ __forceinline__ static Dir of(double x) { return Dir{x}; }
+    __device__ __forceinline__ double value() const { return s; }
+    __device__ __forceinline__ Dir operator+(const Dir &b) const { return Dir{s + b.s}; }
+    __device__ __forceinline__ Dir operator-(const Dir &b) const { return Dir{s - b.s}; }
+    __device__ __forceinline__ Dir operator-() const { return Dir{-s}; }
+    __device__ __forceinline__ Dir operator*(double x) const { return Dir{x * s}; }
+    __device__ __forceinline__ Dir operator/(double x) const { return Dir{s / x}; }
+    // acc + x * this
+    __device__ __forceinline__ Dir fma(double x, const Dir &acc) const { return Dir{__fma_rn(x, s, acc.s)}; }
+};
+template <>
+struct Dir<float> {
+    float s, e;
+    __device__ __forceinline__ static Dir of(float x) { return Dir{x, 0.f}; }
+    __device__ __forceinline__ float value() const { return __fadd_rn(s, e); }
+    __device__ __forceinline__ Dir operator+(const Dir &b) const
+    {
+        Dir r;
+        float t;
+        two_sum(s, b.s, r.s, t);
+        r.e = __fadd_rn(__fadd_rn(e, b.e), t);
+        return r;
+    }
+    __device__ __forceinline__ Dir operator-(const Dir &b) const { return *this + (-b); }
+    __device__ __forceinline__ Dir operator-() const { return Dir{-s, -e}; }
+    __device__ __forceinline__ Dir operator*(float x) const
+    {
+        Dir r;
+        float t;
+        two_prod(x, s, r.s, t);
+        r.e = __fmaf_rn(x, e, t);
+        return r;
+    }
+    __device__ __forceinline__ Dir operator/(float x) const
+    {
+        const float q = s / x;
+        return Dir{q, __fadd_rn(__fmaf_rn(-q, x, s), e) / x};
+    }
+    __device__ __forceinline__ Dir fma(float x, const Dir &acc) const
+    {
+        Dir r;
+        float p, pe, t;
+        two_prod(x, s, p, pe);
+        two_sum(acc.s, p, r.s, t);
+        r.e = __fadd_rn(acc.e, __fadd_rn(t, __fmaf_rn(x, e, pe)));
+        return r;
+    }
+};
+
+// The components of a number of the directional evaluation: as HD, with d1 and
+// h along v.
+template <typename T, int C>
+struct HDir {
+    T v;
+    Dir<T> d1;
+    T g[C];
+    Dir<T> h[C];
+};
+
+// A: whether the number is one of the directional evaluation, which tracks
+// activity.  In one evaluation a variable outside the chunk has zero g and h
+// components, and so has everything computed from such variables alone; with A
+// the zeros are neither stored nor multiplied (act is false), only the value
+// and d1 are.  A skipped product would be an exact zero unless its other factor
+// is Inf or NaN.  Such a factor makes d1 not finite, at the latest through the
+// phi''(u) * 0 that the unary rule adds, and d1 stays so in whatever is computed
+// from it; callers look at the result's d1.
 template <typename T, int C, bool A = false>
-struct Num {
+struct Num;
+
+// Members that both forms share.
+#define CHESSFAD_USER_MEMBERS                                                                  \
+    __device__ __forceinline__ T value() const { return a.v; }                                 \
+    __device__ __forceinline__ Num &operator+=(const Num &w) { return *this = *this + w; }     \
+    __device__ __forceinline__ Num &operator-=(const Num &w) { return *this = *this - w; }     \
+    __device__ __forceinline__ Num &operator*=(const Num &w) { return *this = *this * w; }     \
+    __device__ __forceinline__ Num &operator/=(const Num &w) { return *this = *this / w; }     \
+    __device__ __forceinline__ Num &operator+=(double s) { a.v += T(s); return *this; }        \
+    __device__ __forceinline__ Num &operator-=(double s) { a.v -= T(s); return *this; }        \
+    __device__ __forceinline__ Num &operator*=(double s) { return *this = *this * s; }         \
+    __device__ __forceinline__ Num &operator/=(double s) { return *this = *this / s; }
+template <typename T, int C>
+struct Num<T, C, false> {
     HD<T, C> a;
+
+    __device__ __forceinline__ Num() : a(hzero<T, C>()) {}
+    // A constant: value s, every derivative component zero.
+    __device__ __forceinline__ Num(double s) : a(hzero<T, C>()) { a.v = T(s); }
+    __device__ __forceinline__ explicit Num(const HD<T, C> &h) : a(h) {}
+    CHESSFAD_USER_MEMBERS
+};
+template <typename T, int C>
+struct Num<T, C, true> {
+    HDir<T, C> a;
     bool act;
 
-    __device__ __forceinline__ Num() : a(hzero<T, C>()), act(!A) {}
-    // A constant: value s, every derivative component zero.
-    __device__ __forceinline__ Num(double s) : a(hzero<T, C>()), act(!A) { a.v = T(s); }
-    __device__ __forceinline__ explicit Num(const HD<T, C> &h, bool on = true) : a(h), act(!A || on) {}
-
-    __device__ __forceinline__ T value() const { return a.v; }
-
-    __device__ __forceinline__ Num &operator+=(const Num &w) { return *this = *this + w; }
-    __device__ __forceinline__ Num &operator-=(const Num &w) { return *this = *this - w; }
-    __device__ __forceinline__ Num &operator*=(const Num &w) { return *this = *this * w; }
-    __device__ __forceinline__ Num &operator+=(double s) { a.v += T(s); return *this; }
-    __device__ __forceinline__ Num &operator-=(double s) { a.v -= T(s); return *this; }
-    __device__ __forceinline__ Num &operator*=(double s) { return *this = *this * s; }
-    __device__ __forceinline__ Num &operator/=(const Num &w);
-    __device__ __forceinline__ Num &operator/=(double s);
+    __device__ __forceinline__ Num() : Num(0.0) {}
+    __device__ __forceinline__ Num(double s) : act(false)
+    {
+        a.v = T(s);
+        a.d1 = Dir<T>::of(T(0));
+#pragma unroll
+        for (int l = 0; l < C; ++l) {
+            a.g[l] = T(0);
+            a.h[l] = Dir<T>::of(T(0));
+        }
+    }
+    CHESSFAD_USER_MEMBERS
 };
+#undef CHESSFAD_USER_MEMBERS
 
 template <typename T, int C, bool A>
 __device__ __forceinline__ T value(const Num<T, C, A> &u) { return u.a.v; }
@@ -78,85 +168,98 @@ __device__ __forceinline__ T value(const Num<T, C, A> &u) { return u.a.v; }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u, const Num<T, C, A> &w)
 {
-    if constexpr (!A) return Num<T, C, A>(hadd(u.a, w.a));
-    Num<T, C, A> r = u;
-    r.a.v = u.a.v + w.a.v;
-    r.a.d1 = u.a.d1 + w.a.d1;
-    if (w.act) {
-        if (u.act) {
-            vadd(u.a.g, w.a.g, r.a.g);
-            vadd(u.a.h, w.a.h, r.a.h);
-        } else {
+    if constexpr (!A) {
+        return Num<T, C, A>(hadd(u.a, w.a));
+    } else {
+        Num<T, C, A> r = u;
+        r.a.v = u.a.v + w.a.v;
+        r.a.d1 = u.a.d1 + w.a.d1;
+        if (w.act) {
+            if (u.act) vadd(u.a.g, w.a.g, r.a.g);
 #pragma unroll
             for (int l = 0; l < C; ++l) {
-                r.a.g[l] = w.a.g[l];
-                r.a.h[l] = w.a.h[l];
+                if (!u.act) r.a.g[l] = w.a.g[l];
+                r.a.h[l] = u.act ? u.a.h[l] + w.a.h[l] : w.a.h[l];
             }
             r.act = true;
         }
+        return r;
     }
-    return r;
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u, const Num<T, C, A> &w)
 {
-    if constexpr (!A) return Num<T, C, A>(hsub(u.a, w.a));
-    Num<T, C, A> r = u;
-    r.a.v = u.a.v - w.a.v;
-    r.a.d1 = u.a.d1 - w.a.d1;
-    if (w.act) {
+    if constexpr (!A) {
+        return Num<T, C, A>(hsub(u.a, w.a));
+    } else {
+        Num<T, C, A> r = u;
+        r.a.v = u.a.v - w.a.v;
+        r.a.d1 = u.a.d1 - w.a.d1;
+        if (w.act) {
 #pragma unroll
-        for (int l = 0; l < C; ++l) {
-            r.a.g[l] = u.act ? u.a.g[l] - w.a.g[l] : -w.a.g[l];
-            r.a.h[l] = u.act ? u.a.h[l] - w.a.h[l] : -w.a.h[l];
+            for (int l = 0; l < C; ++l) {
+                r.a.g[l] = u.act ? u.a.g[l] - w.a.g[l] : -w.a.g[l];
+                r.a.h[l] = u.act ? u.a.h[l] - w.a.h[l] : -w.a.h[l];
+            }
+            r.act = true;
         }
-        r.act = true;
+        return r;
     }
-    return r;
 }
 // u * w with w inactive: the rule's terms without the zeros of w
 template <typename T, int C>
-__device__ __forceinline__ void hmul_by(const HD<T, C> &u, const HD<T, C> &w, HD<T, C> &r)
+__device__ __forceinline__ void hmul_by(const HDir<T, C> &u, const HDir<T, C> &w, HDir<T, C> &r)
 {
     vmul(w.v, u.g, r.g);
-    vmul(w.d1, u.g, r.h);
-    vfma(w.v, u.h, r.h);
+#pragma unroll
+    for (int l = 0; l < C; ++l) r.h[l] = u.h[l].fma(w.v, w.d1 * u.g[l]);
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, const Num<T, C, A> &w)
 {
-    if constexpr (!A) return Num<T, C, A>(hmul(u.a, w.a));
-    Num<T, C, A> r;
-    if (u.act) {
-        if (w.act) {
-            r.a = hmul(u.a, w.a);
-            r.act = true;
-            return r;
+    if constexpr (!A) {
+        return Num<T, C, A>(hmul(u.a, w.a));
+    } else {
+        Num<T, C, A> r;
+        if (u.act && w.act) {
+            vmul(u.a.v, w.a.g, r.a.g);
+            vfma(w.a.v, u.a.g, r.a.g);
+#pragma unroll
+            for (int l = 0; l < C; ++l) {
+                Dir<T> h = w.a.h[l] * u.a.v;
+                h = u.a.d1.fma(w.a.g[l], h);
+                h = w.a.d1.fma(u.a.g[l], h);
+                r.a.h[l] = u.a.h[l].fma(w.a.v, h);
+            }
+        } else if (u.act) {
+            hmul_by(u.a, w.a, r.a);
+        } else if (w.act) {
+            hmul_by(w.a, u.a, r.a);
         }
-        hmul_by(u.a, w.a, r.a);
-    } else if (w.act) {
-        hmul_by(w.a, u.a, r.a);
+        r.act = u.act || w.act;
+        r.a.v = u.a.v * w.a.v;
+        r.a.d1 = u.a.d1.fma(w.a.v, w.a.d1 * u.a.v);
+        return r;
     }
-    r.act = u.act || w.act;
-    r.a.v = u.a.v * w.a.v;
-    r.a.d1 = fma_(w.a.v, u.a.d1, u.a.v * w.a.d1);
-    return r;
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u)
 {
-    if constexpr (!A) return Num<T, C, A>(rsub(T(0), u.a));
-    Num<T, C, A> r = u;
-    r.a.v = T(0) - u.a.v;
-    r.a.d1 = -u.a.d1;
-    if (u.act) {
+    if constexpr (!A) {
+        return Num<T, C, A>(rsub(T(0), u.a));
+    } else {
+        Num<T, C, A> r = u;
+        r.a.v = T(0) - u.a.v;
+        r.a.d1 = -u.a.d1;
+        if (u.act) {
 #pragma unroll
-        for (int l = 0; l < C; ++l) {
-            r.a.g[l] = -u.a.g[l];
-            r.a.h[l] = -u.a.h[l];
+            for (int l = 0; l < C; ++l) {
+                r.a.g[l] = -u.a.g[l];
+                r.a.h[l] = -u.a.h[l];
+            }
         }
+        return r;
     }
-    return r;
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u) { return u; }
@@ -177,15 +280,19 @@ __device__ __forceinline__ Num<T, C, A> operator-(double s, const Num<T, C, A> &
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, double s)
 {
-    if constexpr (!A) return Num<T, C, A>(smul(T(s), u.a));
-    Num<T, C, A> r = u;
-    r.a.v = T(s) * u.a.v;
-    r.a.d1 = T(s) * u.a.d1;
-    if (u.act) {
-        vmul(T(s), u.a.g, r.a.g);
-        vmul(T(s), u.a.h, r.a.h);
+    if constexpr (!A) {
+        return Num<T, C, A>(smul(T(s), u.a));
+    } else {
+        Num<T, C, A> r = u;
+        r.a.v = T(s) * u.a.v;
+        r.a.d1 = u.a.d1 * T(s);
+        if (u.act) {
+            vmul(T(s), u.a.g, r.a.g);
+#pragma unroll
+            for (int l = 0; l < C; ++l) r.a.h[l] = u.a.h[l] * T(s);
+        }
+        return r;
     }
-    return r;
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator*(double s, const Num<T, C, A> &u) { return u * s; }
@@ -194,16 +301,23 @@ __device__ __forceinline__ Num<T, C, A> operator*(double s, const Num<T, C, A> &
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> apply(const Num<T, C, A> &u, T phi, T d1, T d2)
 {
-    if constexpr (!A) return Num<T, C, A>(unary(u.a, phi, d1, d2));
-    Num<T, C, A> r;
-    if (u.act) {
-        r.a = unary(u.a, phi, d1, d2);
+    if constexpr (!A) {
+        return Num<T, C, A>(unary(u.a, phi, d1, d2));
     } else {
+        Num<T, C, A> r;
         r.a.v = phi;
-        r.a.d1 = fma_(d2, T(0), d1 * u.a.d1);
+        r.a.d1 = u.a.d1 * d1;
+        if (u.act) {
+            const Dir<T> q = u.a.d1 * d2;
+            vmul(d1, u.a.g, r.a.g);
+#pragma unroll
+            for (int l = 0; l < C; ++l) r.a.h[l] = q.fma(u.a.g[l], u.a.h[l] * d1);
+        } else {
+            r.a.d1.s = fma_(d2, T(0), r.a.d1.s);
+        }
+        r.act = u.act;
+        return r;
     }
-    r.act = u.act;
-    return r;
 }
 
 template <typename T, int C, bool A>
@@ -222,21 +336,19 @@ __device__ __forceinline__ Num<T, C, A> operator/(const Num<T, C, A> &u, double 
 {
     const T d = T(s);
     Num<T, C, A> r = u;
-    r.a.v /= d;
-    r.a.d1 /= d;
-    if (!A || u.act) {
+    bool act = true;
+    if constexpr (A) act = u.act;
+    r.a.v = u.a.v / d;
+    r.a.d1 = u.a.d1 / d;
+    if (act) {
 #pragma unroll
         for (int l = 0; l < C; ++l) {
-            r.a.g[l] /= d;
-            r.a.h[l] /= d;
+            r.a.g[l] = u.a.g[l] / d;
+            r.a.h[l] = u.a.h[l] / d;
         }
     }
     return r;
 }
-template <typename T, int C, bool A>
-__device__ __forceinline__ Num<T, C, A> &Num<T, C, A>::operator/=(const Num<T, C, A> &w) { *this = *this / w; return *this; }
-template <typename T, int C, bool A>
-__device__ __forceinline__ Num<T, C, A> &Num<T, C, A>::operator/=(double s) { *this = *this / s; return *this; }
 
 // ---- elementary functions
 template <typename T, int C, bool A>
@@ -290,13 +402,13 @@ __device__ __forceinline__ Num<T, C, A> pow(const Num<T, C, A> &u, double p)
     // derivative of u^1 is 1).  A number outside the chunk uses phi'' only to notice that it is
     // not finite; where u^(p-2) = u^(p-1) / u and its factor are far inside the
     // range, that power is left out (the extended-operator test function, FP64,
-    // n = 64, 4096 points: 1.67 ms with three powers everywhere, 1.34 ms so).
+    // n = 64, 4096 points: 1.67 ms with three powers everywhere, 1.30 so).
     const T q = T(p), x = u.a.v, big = sizeof(T) == 8 ? T(1e75) : T(1e9);
     const T w0 = m_pow(x, q), w1 = m_pow(x, q - T(1));
-    T w = T(0);
-    if (!A || u.act ||
-        !(x > T(1) / big && x < big && w1 < big && w1 > -big && q < big && q > -big))
-        w = m_pow(x, q - T(2));
+    bool needed = !(x > T(1) / big && x < big && w1 < big && q < big && q > -big);
+    if constexpr (A) needed |= u.act;
+    else needed = true;
+    const T w = needed ? m_pow(x, q - T(2)) : T(0);
     return apply(u, w0, q * w1, q * (q - T(1)) * w);
 }
 template <typename T, int C, bool A>
@@ -350,19 +462,19 @@ struct DirVars {
     __device__ __forceinline__ Num<T, C, true> operator[](int k) const
     {
         // x, v: this point's variables, `stride` elements apart
-        HD<T, C> y;
-        y.v = x[k * stride];
-        y.d1 = v[k * stride];
+        Num<T, C, true> y;
+        y.a.v = x[k * stride];
+        y.a.d1 = Dir<T>::of(v[k * stride]);
         const int d = k - cstart;
-        const bool in = d >= 0 && d < C;
-        if (in) {
+        y.act = d >= 0 && d < C;
+        if (y.act) {
 #pragma unroll
             for (int l = 0; l < C; ++l) {
-                y.g[l] = (d == l) ? z.one : z.z;
-                y.h[l] = z.z;
+                y.a.g[l] = (d == l) ? z.one : z.z;
+                y.a.h[l] = Dir<T>::of(z.z);
             }
         }
-        return Num<T, C, true>(y, in);
+        return y;
     }
 };
 

@@ -4,8 +4,9 @@ import numpy as np
 import pytest
 
 import paper_2410_22575_gb300 as cf
+from paper_2410_22575_gb300 import workloads as W
 
-from test_gpu_user import PLAIN, SYM
+from test_gpu_user import PLAIN, SYM, Case, user_fn
 
 pytestmark = pytest.mark.gpu
 
@@ -68,3 +69,32 @@ def test_powers_that_are_not_finite(prec):
     ok = np.isfinite(ref)
     scale = np.max(np.abs(np.where(ok, ref, 0)), axis=1, keepdims=True) * np.ones_like(ref)
     assert np.all(np.abs(got - ref)[ok] <= (4e-12 if prec == cf.FP64 else 4e-5) * scale[ok])
+
+
+def test_fp32_sums_over_the_direction_are_compensated():
+    """f = (sum x)^2 / 2, every entry of H is 1: each row of H v is sum v as a
+    compensated sum gives it, |error| <= 2u |sum v| + n^2 u^2 sum |v|."""
+    import torch
+
+    src = """template <class R, class X> R square_sum(const X &x, int n, const double *p)
+    { R s = 0.0; for (int k = 0; k < n; ++k) s += x[k]; return 0.5 * s * s; }"""
+    f = cf.UserFunction(src, "square_sum", 8, cf.FP32_COMP)
+    u = 2.0 ** -24
+    rng = np.random.Generator(np.random.PCG64(3))
+    for n in (3, 64, 130, 512):
+        x = torch.tensor(rng.uniform(-1, 1, (200, n)), dtype=torch.float32, device="cuda")
+        v = torch.tensor(rng.uniform(-1, 1, (200, n)), dtype=torch.float32, device="cuda")
+        vd = v.double().cpu().numpy()
+        ref = vd.sum(1)
+        err = np.abs(f.hvp(x, v).double().cpu().numpy() - ref[:, None]).max(1)
+        assert np.all(err <= 2 * u * np.abs(ref) + n * n * u * u * np.abs(vd).sum(1)), n
+
+
+@pytest.mark.parametrize("fn", [W.ROSENBROCK, W.ACKLEY, W.FLETCHER_POWELL, W.MIX])
+@pytest.mark.parametrize("n,batch", [(5, 400), (19, 200), (64, 64), (200, 12)])
+def test_fp32_default_is_as_accurate_as_the_symmetric_method(fn, n, batch):
+    """Root mean square error over the batch, normalised by |H|_F |v|_2; 1.1
+    allows for the different order of the sums."""
+    f, k = user_fn(fn, 8, cf.FP32_COMP), Case(fn, n, batch, 300 + n, cf.FP32_COMP)
+    rms = [np.sqrt(np.mean(k.hvp_err(f.hvp(k.x, k.v, k.params, cfg=c)) ** 2)) for c in (None, SYM)]
+    assert rms[0] <= 1.1 * rms[1], rms
