@@ -32,7 +32,8 @@ struct chessfad_user_fn {
     cudaKernel_t hessian = nullptr;      // plain (CHUNK-HESS, Alg. 5)
     cudaKernel_t sym_hvp = nullptr;      // symmetric (SC-HESS-VEC, Alg. 8)
     cudaKernel_t sym_hessian = nullptr;  // symmetric (SCHUNK-HESS, Alg. 6)
-    cudaKernel_t dir_hvp = nullptr;      // directional (the default HVP)
+    cudaKernel_t dir_hvp = nullptr;      // directional (the default HVP); null where the source does
+                                         // not compile for its numbers: symmetric then
     cudaKernel_t hvp_n1 = nullptr;       // FP32 handles, n = 1: FP64 arithmetic, float I/O
     cudaKernel_t hessian_n1 = nullptr;
     int csize = 0;
@@ -259,7 +260,7 @@ int launch(chessfad_user_fn *fn, const chessfad_config *cfg, bool hvp, int n, lo
         block = (unsigned)b;
         smem = (size_t)args.maxpts * 2 * sizeof(double);
         k = hvp ? fn->hvp_n1 : fn->hessian_n1;
-    } else if (hvp && !cfg) {
+    } else if (hvp && !cfg && fn->dir_hvp) {
         // the default: one thread per (point, chunk), `lanes` points per CTA
         // of 128 threads: a warp's worth while x and v of that many fit 48
         // KiB, no more than the batch has
@@ -328,7 +329,8 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     text += source;
     text += "\n#include \"user_kernel.cuh\"\n";
     // The row methods and the directional kernel as two programs: compiled side
-    // by side they take about as long as the larger one.  The directional kernel's
+    // by side they take about as long as the larger one.  A source that names the
+    // rows' number type Num<T, C> may compile for the row methods only.  The directional kernel's
     // chunk size is not part of its result; in FP32 its numbers take two floats
     // per component of d1 and h, and chunks larger than 8 spill (the extended-
     // operator function at csize 16, n = 64, 4096 points: 337 us with chunks of
@@ -349,11 +351,10 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     compile_program(rt, text, name, csize, prec, false, prog[0]);
     if (second.joinable()) second.join();
     else compile_program(rt, text, name, dir_csize, prec, true, prog[1]);
-    for (const Program &p : prog)
-        if (!p.ok) {
-            put_log(log, log_bytes, p.log);
-            return CHESSFAD_ERR_JIT;
-        }
+    if (!prog[0].ok) {
+        put_log(log, log_bytes, prog[0].log);
+        return CHESSFAD_ERR_JIT;
+    }
     put_log(log, log_bytes, prog[0].log);
 
     auto *fn = new chessfad_user_fn;
@@ -361,13 +362,13 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     fn->dir_csize = dir_csize;
     fn->prec = prec;
     cudaError_t e = cudaLibraryLoadData(&fn->lib, prog[0].cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && prog[1].ok)
         e = cudaLibraryLoadData(&fn->dir_lib, prog[1].cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->hvp, fn->lib, "chessfad_user_hvp");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->hessian, fn->lib, "chessfad_user_hessian");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hvp, fn->lib, "chessfad_user_sym_hvp");
     if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->sym_hessian, fn->lib, "chessfad_user_sym_hessian");
-    if (e == cudaSuccess) e = cudaLibraryGetKernel(&fn->dir_hvp, fn->dir_lib, "chessfad_user_dir_hvp");
+    if (e == cudaSuccess && prog[1].ok) e = cudaLibraryGetKernel(&fn->dir_hvp, fn->dir_lib, "chessfad_user_dir_hvp");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP) e = cudaLibraryGetKernel(&fn->hvp_n1, fn->lib, "chessfad_user_hvp_n1");
     if (e == cudaSuccess && prec == CHESSFAD_FP32_COMP)
         e = cudaLibraryGetKernel(&fn->hessian_n1, fn->lib, "chessfad_user_hessian_n1");

@@ -98,3 +98,25 @@ def test_fp32_default_is_as_accurate_as_the_symmetric_method(fn, n, batch):
     f, k = user_fn(fn, 8, cf.FP32_COMP), Case(fn, n, batch, 300 + n, cf.FP32_COMP)
     rms = [np.sqrt(np.mean(k.hvp_err(f.hvp(k.x, k.v, k.params, cfg=c)) ** 2)) for c in (None, SYM)]
     assert rms[0] <= 1.1 * rms[1], rms
+
+
+@pytest.mark.parametrize("prec", [cf.FP64, cf.FP32_COMP])
+def test_source_that_names_the_number_type(prec):
+    """A helper on chessfad::user::Num<T, C>, which takes the rows' numbers only:
+    the handle is created and its default product is the symmetric method's."""
+    src = """template <class T, int C> __device__ chessfad::user::Num<T, C> cube(const chessfad::user::Num<T, C> &u)
+    { return u * u * u; }
+    template <class R, class X> R cubes(const X &x, int n, const double *p)
+    { R f = 0.0; for (int k = 0; k < n; ++k) f += cube(x[k]) * x[0]; return f; }"""
+    f, k = cf.UserFunction(src, "cubes", 4, prec), Case(W.ROSENBROCK, 11, 50, 3, prec)
+    out = f.hvp(k.x, k.v).double().cpu().numpy()
+    assert np.array_equal(out, f.hvp(k.x, k.v, cfg=cf.Config(0, 0, 0, cf.SYMMETRIC, 32)).double().cpu().numpy())
+    x, v = k.xh, k.vh
+    H = np.zeros((50, 11, 11))
+    i = np.arange(11)
+    H[:, i, i] += 6 * x * x[:, :1]
+    H[:, 0, :] += 3 * x ** 2
+    H[:, :, 0] += 3 * x ** 2
+    ref = np.einsum("pij,pj->pi", H, v)
+    scale = np.sqrt((H * H).sum((1, 2))) * np.linalg.norm(v, axis=1)
+    assert np.max(np.linalg.norm(out - ref, axis=1) / scale) <= (1e-12 if prec == cf.FP64 else 1e-5)
