@@ -314,17 +314,28 @@ __global__ void __launch_bounds__(kFpThreads) fp_curvature_kernel(const StructAr
                                             1, tile.z, tile.rd);
         return;
     }
+    bool bad[kFpNpt] = {};
 #pragma unroll
     for (int i = 0; i < kFpNpt; ++i) {
         const int u = threadIdx.x + i * kFpThreads;
         if (u >= P * n) break;
         const int l = u - tile.base[tile.qs[u]];
         IO *row = static_cast<IO *>(a.out) + ((size_t)p0 * n + u) * n;
-        row[l] = (IO)tile.curvature(u, sums[i]);
+        const T h = tile.curvature(u, sums[i]);
+        bad[i] = not_finite(h);
+        row[l] = (IO)h;
         if (n >= 3 && n <= kGramSmall) {
             row[beside(l, 1, n)] = (IO)narrow<T>(tile.z[u].x);
             row[beside(l, 2, n)] = (IO)narrow<T>(tile.z[u].y);
         }
+    }
+    // n > kGramSmall: the third launch looks at a point's first entry
+    if (n > kGramSmall && __syncthreads_or(bad[0] || bad[1])) {
+#pragma unroll
+        for (int i = 0; i < kFpNpt; ++i)
+            if (bad[i])
+                static_cast<IO *>(a.out)[(size_t)(p0 + tile.qs[threadIdx.x + i * kFpThreads]) * n * n] =
+                    nan_of(IO(0));
     }
 }
 
@@ -507,8 +518,8 @@ __global__ void __launch_bounds__(kThreads) fp_gram_kernel(const StructArgs a, i
     }
 }
 
-// Third launch, n > kGramSmall: points whose residuals are not finite (their
-// whole diagonal is not) by the dense propagation.
+// Third launch, n > kGramSmall: points with a curvature that is not finite (the
+// first launch made their first entry NaN) by the dense propagation.
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kThreads) fp_hessian_fix_kernel(const StructArgs a)
 {

@@ -74,3 +74,19 @@ def test_fletcher_powell_one_variable_hessian_many_points():
         (b.fp.A, b.fp.B, b.fp.E)[which].flat[0] = np.inf
         d = Dev(b, cf.FP32_COMP)
         assert np.array_equal(d.hessian(), d.hessian(cfg=cf.Config(1, 1, 256)), equal_nan=True)
+
+
+@pytest.mark.parametrize("n", [3, 13, 64, 70, 140])
+@pytest.mark.parametrize("which", [0, 1])
+def test_fletcher_powell_fp32_parameters_beyond_float(n, which):
+    """An entry of A (B) finite in FP64 and infinite in FP32, in a column whose
+    sin (cos) hides it from the residuals at one point: every entry is NaN
+    there, as the dense method has it, whatever the column."""
+    for j in (0, n // 2, n - 1):
+        b = W.make_batch(W.FLETCHER_POWELL, n, 6, seed=80 + n)
+        (b.fp.A, b.fp.B)[which][1, j] = 1e39
+        b.x[2:4, j] = 0.0 if which == 0 else math.pi / 2
+        d = Dev(b, cf.FP32_COMP)
+        cfg = cf.Config(0, 0, 0, cf.SYMMETRIC, 0) if n >= 4 else cf.Config(2, 1, 256)
+        for got, dense in ((d.hessian(), d.hessian(cfg=cfg)), (d.hvp(), d.hvp(cfg=cfg))):
+            assert np.array_equal(np.isnan(got), np.isnan(dense)), j
