@@ -90,3 +90,21 @@ def test_fletcher_powell_fp32_parameters_beyond_float(n, which):
         cfg = cf.Config(0, 0, 0, cf.SYMMETRIC, 0) if n >= 4 else cf.Config(2, 1, 256)
         for got, dense in ((d.hessian(), d.hessian(cfg=cfg)), (d.hvp(), d.hvp(cfg=cfg))):
             assert np.array_equal(np.isnan(got), np.isnan(dense)), j
+
+
+@pytest.mark.parametrize("n", [5, 40, 140])
+def test_fletcher_powell_fp32_subnormal_parameters(n):
+    """A column of A and B whose floats are subnormal (rounded to 2^-149, a
+    relative 2e-5 of 1e-40): its row of H v and its diagonal entry keep three
+    digits."""
+    j = n // 2
+    b = W.make_batch(W.FLETCHER_POWELL, n, 20, seed=70 + n)
+    b.fp.A[:, j] *= 1e-42  # |A|, |B| up to 100
+    b.fp.B[:, j] *= 1e-42
+    d = Dev(b, cf.FP32_COMP)
+    Hv, _ = d.ref_hvp()
+    H = d.ref_hessian()
+    row, diag = d.hvp()[:, j], d.hessian()[:, j, j]
+    assert np.max(np.abs(Hv[:, j])) > 0
+    assert np.max(np.abs(row - Hv[:, j])) <= 1e-3 * np.max(np.abs(Hv[:, j]))
+    assert np.max(np.abs(diag - H[:, j, j])) <= 1e-3 * np.max(np.abs(H[:, j, j]))
