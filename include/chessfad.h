@@ -352,6 +352,14 @@ typedef struct chessfad_ragged_plan_s *chessfad_ragged_plan;
  * CHESSFAD_ERR_PLAN for a negative offset.  Launches nothing. */
 CHESSFAD_API int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, int prec, int csize,
                                              chessfad_ragged_plan *plan);
+
+/* As chessfad_ragged_plan_create, for the dense chunked evaluation in the
+ * configuration that chessfad_ragged_autotune found: each (function, n range)
+ * group of requests with the chunk size, lanes per row and Fletcher-Powell
+ * tile that it stored, groups it did not tune with the defaults
+ * (chessfad_ragged_plan_group_config says which). */
+CHESSFAD_API int chessfad_ragged_plan_create_tuned(const chessfad_request *reqs, long long nreq, int prec,
+                                                   chessfad_ragged_plan *plan);
 CHESSFAD_API int chessfad_ragged_plan_destroy(chessfad_ragged_plan plan);
 
 /* Device workspace bytes the plan needs (tile table, request list, offsets,
@@ -387,7 +395,7 @@ CHESSFAD_API int chessfad_ragged_plan_group_config(chessfad_ragged_plan plan, in
  * measuring the SM cycles its tiles take, summed over the CTAs (the group's
  * throughput inside a large mixed run, free of the small sample's own tail),
  * and store the cheapest per (prec, function, n range) in the process-wide
- * table that chessfad_ragged_plan_group_config reports from.  xpack, vpack,
+ * table that chessfad_ragged_plan_create_tuned builds from.  xpack, vpack,
  * outpack, params as for chessfad_hvp_ragged (outpack of the sampled requests
  * is overwritten); workspace: device scratch of workspace_bytes (candidates
  * whose trial plan needs more, plus 256 bytes for the cycle counter, are

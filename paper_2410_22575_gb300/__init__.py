@@ -95,6 +95,7 @@ def load(build_if_missing: bool = True):
         lib.chessfad_compensated_rows.argtypes = [P, P, L, I, I, I, P, P]
         lib.chessfad_compensated_rows.restype = I
         lib.chessfad_ragged_plan_create.argtypes = [P, L, I, I, ctypes.POINTER(P)]
+        lib.chessfad_ragged_plan_create_tuned.argtypes = [P, L, I, ctypes.POINTER(P)]
         lib.chessfad_ragged_plan_destroy.argtypes = [P]
         lib.chessfad_ragged_plan_info.argtypes = [P, ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(L),
                                                   ctypes.POINTER(ctypes.c_size_t)]
@@ -130,6 +131,7 @@ def load(build_if_missing: bool = True):
                      "chessfad_autotune_hessian", "chessfad_peak_flops",
                      "chessfad_peak_info", "chessfad_peak_operand_rates",
                      "chessfad_kernel_info", "chessfad_version", "chessfad_ragged_plan_create",
+                     "chessfad_ragged_plan_create_tuned",
                      "chessfad_ragged_plan_destroy", "chessfad_ragged_plan_info", "chessfad_ragged_plan_upload",
                      "chessfad_hvp_ragged", "chessfad_ragged_plan_group_config", "chessfad_ragged_autotune",
                      "chessfad_ragged_tuned_config"):
@@ -455,6 +457,18 @@ def chessfad_ragged_plan_create(reqs, prec=FP32_COMP, csize=0):
     return h.value
 
 
+def chessfad_ragged_plan_create_tuned(reqs, prec=FP32_COMP):
+    """Plan handle (int) of the dense evaluation as chessfad_ragged_autotune
+    tuned it."""
+    import numpy as np
+
+    reqs = np.ascontiguousarray(reqs, dtype=request_dtype())
+    h = ctypes.c_void_p()
+    _check(load().chessfad_ragged_plan_create_tuned(reqs.ctypes.data if len(reqs) else None, len(reqs), prec,
+                                                    ctypes.byref(h)), "chessfad_ragged_plan_create_tuned")
+    return h.value
+
+
 def chessfad_ragged_plan_destroy(plan) -> int:
     return load().chessfad_ragged_plan_destroy(plan)
 
@@ -514,13 +528,19 @@ def chessfad_hvp_ragged_noalloc(plan, xpack, vpack, outpack, params=None, stream
 
 
 class RaggedPlan:
-    """Owns a plan and its device workspace (a torch uint8 tensor)."""
+    """Owns a plan and its device workspace (a torch uint8 tensor).  tuned: the
+    dense evaluation as chessfad_ragged_autotune tuned it (csize 0)."""
 
-    def __init__(self, reqs, prec=FP32_COMP, csize=0, device="cuda", stream=None):
+    handle = None
+
+    def __init__(self, reqs, prec=FP32_COMP, csize=0, device="cuda", stream=None, tuned=False):
         import torch
 
+        if tuned and csize:
+            raise ValueError("tuned: the chunk sizes are the tuned ones, csize must be 0")
         self.prec = prec
-        self.handle = chessfad_ragged_plan_create(reqs, prec, csize)
+        self.handle = (chessfad_ragged_plan_create_tuned(reqs, prec) if tuned
+                       else chessfad_ragged_plan_create(reqs, prec, csize))
         info = chessfad_ragged_plan_info(self.handle)
         self.info = info
         self.workspace = torch.empty(max(256, info["workspace_bytes"]), dtype=torch.uint8, device=device)

@@ -10,9 +10,9 @@
 // (function, n range): from the table chessfad_ragged_autotune fills, else by
 // default.  The tables (tiles, request list, offsets) live in a
 // caller-provided device workspace together with a queue counter.  That is
-// the dense chunked evaluation, of a plan built with a chunk size; a plan
-// built without one is evaluated structurally (ragged_structured.cu), with
-// the same workspace, counter and launch scheme.
+// the dense chunked evaluation, of a plan built with a chunk size or with the
+// tuned ones; any other plan is evaluated structurally (ragged_structured.cu),
+// with the same workspace, counter and launch scheme.
 //
 // Device side: a persistent kernel, a few CTAs per SM, whose CTAs take tile
 // after tile from the counter with atomicAdd and run the tile's sweeps.  No
@@ -408,6 +408,7 @@ int sym_tpr(int tpr, int n)
 
 struct PlanOptions {
     int csize = 0;                               // fixed chunk size for every group (0: per group)
+    bool tuned = false;                          // csize 0: the dense evaluation with the tuned table
     const std::map<std::pair<int, int>, GroupCfg> *force = nullptr;  // (fn, bucket) -> forced config
 };
 
@@ -459,7 +460,7 @@ int build_plan(const chessfad_request *reqs, long long nreq, int prec, const Pla
     }
     std::vector<std::pair<double, RTile>> work;
     size_t smem = 0;
-    pl->structured = opt.csize == 0 && !opt.force;
+    pl->structured = opt.csize == 0 && !opt.tuned && !opt.force;
     for (auto &g : groups) {
         const int fn = g.first.first, n = g.first.second;
         GroupCfg gc;
@@ -730,8 +731,8 @@ int check_run(const chessfad_ragged_plan_s *plan, const void *xpack, const void 
 
 extern "C" {
 
-int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, int prec, int csize,
-                                chessfad_ragged_plan *plan_out)
+static int create_plan(const chessfad_request *reqs, long long nreq, int prec, int csize, bool tuned,
+                       chessfad_ragged_plan *plan_out)
 {
     if (!plan_out) return CHESSFAD_ERR_NULL;
     *plan_out = nullptr;
@@ -743,6 +744,7 @@ int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, in
     if (!pl) return CHESSFAD_ERR_PLAN;
     PlanOptions opt;
     opt.csize = csize;
+    opt.tuned = tuned;
     st = build_plan(reqs, nreq, prec, opt, pl);
     if (st) {
         delete pl;
@@ -750,6 +752,18 @@ int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, in
     }
     *plan_out = pl;
     return CHESSFAD_SUCCESS;
+}
+
+int chessfad_ragged_plan_create(const chessfad_request *reqs, long long nreq, int prec, int csize,
+                                chessfad_ragged_plan *plan_out)
+{
+    return create_plan(reqs, nreq, prec, csize, false, plan_out);
+}
+
+int chessfad_ragged_plan_create_tuned(const chessfad_request *reqs, long long nreq, int prec,
+                                      chessfad_ragged_plan *plan_out)
+{
+    return create_plan(reqs, nreq, prec, 0, true, plan_out);
 }
 
 int chessfad_ragged_plan_destroy(chessfad_ragged_plan plan)
