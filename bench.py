@@ -11,6 +11,8 @@ beside it as a complete block (``fp32_comp``: rate, roofline, end-to-end rate,
 error), so "FP32-comp vs FP64" is one line.  ``workloads`` holds the other
 named workloads (Rosenbrock n=16 and n=256 with Hessians, Fletcher-Powell
 n=32) in both precisions, ``ragged_100k`` the 100000-request uneven batch.
+The full record is printed on stderr; stdout has one JSON line with its
+headline fields and a summary of the rest.
 
 Roofline: the sweep kernels are bound by CUDA-core arithmetic (FP64 DFMA or
 FP32 FFMA pipe).  ``achieved`` = FP instructions the kernel executes per launch
@@ -683,7 +685,29 @@ def gpu_arm(args):
         line["summary"] = compact_summary(line)
     except Exception as exc:  # the summary repeats figures; it must never cost the line
         line["summary"] = {"error": repr(exc)}
-    print(json.dumps(line))
+    print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line)), flush=True)
+
+
+# The printed line's keys; everything else is in the full record on stderr.
+SHORT_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "launch", "roofline", "e2e", "gpu_launches", "clocks",
+              "fp32_over_fp64", "error_vs_oracle")
+
+
+def short_line(line: dict) -> dict:
+    """The line printed on stdout: the headline fields and the summary, under
+    4 KB, so that whoever keeps only the end of the output still has all of it
+    (the full record, about 40 KB, goes to stderr)."""
+    out = {k: line[k] for k in SHORT_KEYS if k in line}
+    f32 = line.get("fp32_comp")
+    if f32:
+        out["fp32_comp"] = {k: f32[k] for k in ("value", "unit", "dtype", "ms_per_step", "e2e") if k in f32}
+    cb = line.get("cpu_baseline")
+    if cb:
+        out["cpu_baseline"] = {k: cb[k] for k in ("value", "unit", "cores", "kind") if k in cb}
+    out["summary"] = line.get("summary")
+    return out
 
 
 def _sig(x, digits: int = 3):
