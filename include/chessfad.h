@@ -35,7 +35,10 @@
  *    (csize 0, no configuration or one of zeros) gets the structured
  *    evaluation: the same hDual rules on the components the seeds make
  *    nonzero, with the dense method's results for finite and non-finite
- *    inputs (to rounding).  Naming a chunk size or a method runs the dense
+ *    inputs (to rounding).  How many lanes share a point follows the batch
+ *    size, so the last bits of a point's result may differ between batches of
+ *    different sizes (one call and its slices, say); the same call gives the
+ *    same bits.  Naming a chunk size or a method runs the dense
  *    chunked algorithm with it.  csize need not divide n: the last chunk is
  *    ragged and its positions beyond n are never seeded.
  *  - 1 <= n <= CHESSFAD_MAX_N.  batch == 0 is a valid no-op; batch < 0 is an

@@ -182,7 +182,7 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
     // requests up to n = 512: a sixteenth 268 us, an eighth 268, a quarter 257;
     // at least 7.5 us 258, 15 us 257, 30 us 256; one request of n = 505: 64, 65
     // and 85 us.
-    const double most = std::max(62000.0, total / (152.0 * 4.0));
+    const double most = std::max(62000.0, total / (kSms * 4.0));
     std::vector<std::pair<double, STile>> work;
     long long end = 0;  // of the current tile's group
     for (long long e = 0; e < nreq;) {
@@ -228,7 +228,7 @@ void structured_plan(const chessfad_request *reqs, long long nreq, int prec, SPl
         t.epl = it <= 1 ? 1 : it <= 4 ? 4 : it <= 8 ? 8 : 16;
         // rounds of the CTA's lane groups: fewer when the batch is small
         const int groups = kThreads / t.lanes;
-        const long long rounds = std::max<long long>(1, std::min<long long>(4, (end - e) / (608LL * groups)));
+        const long long rounds = std::max<long long>(1, std::min<long long>(4, (end - e) / (4LL * kSms * groups)));
         double elems = 0.0;
         while (e < end && t.count < groups * rounds && 2 * pl.n[e] >= nmax) {
             elems += pl.n[e];

@@ -10,11 +10,13 @@
 //   Rosenbrock n = 256, FP64, 1024                 86.1 ms -> 0.076 ms (7.0 TB/s written)
 //   Ackley n = 33, FP32-comp, 20000                0.178 ms -> 0.035 ms
 //   Fletcher-Powell n = 48, FP32-comp, 4096        2.23 ms -> 0.107 ms
-// The Rosenbrock kernels stream; the others are bound by the FP64 pipe (sin,
-// cos and the sums under sqrt and exp; the residuals), in compensated FP32 too.
-// It takes one warp instruction per 16 clocks and SM, so what is not FP64
-// arithmetic stays off it: conversions and tests of FP64 values run on 32-bit
-// words, coefficients come from registers (fp64_sincos.cuh).
+// The Rosenbrock kernels stream.  In FP64 the others are bound by the FP64 pipe
+// (sin, cos and the sums under sqrt and exp; the residuals), and so are the
+// Fletcher-Powell ones in compensated FP32; Ackley's H v there is bound by
+// instruction issue and its Hessian by shared-memory loads.  The FP64 pipe takes
+// one warp instruction per 16 clocks and SM, so what is not FP64 arithmetic stays
+// off it: conversions and tests of FP64 values run on 32-bit words, coefficients
+// come from registers (fp64_sincos.cuh).
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -156,8 +158,8 @@ __global__ void __launch_bounds__(kThreads) ros_hessian_kernel(const StructArgs 
 // ppc whole points per CTA, or, split > 1, one of `split` parts of one
 // point's rows.  Entry (i, j) is (K x_i) x_j + (G s_i) s_j, K = p1 r2 + p2 r1^2
 // and G = q2 the second derivatives of the tail in its two sums, s = sin 2 pi x;
-// the diagonal adds p1 r1 + q1 cos 2 pi x.  Bound by the stores and the
-// products that feed them.
+// the diagonal adds p1 r1 + q1 cos 2 pi x.  Bound by the shared-memory loads
+// per element (n = 33, FP32-comp: 76 % busy, issue 60 %, 2.5 TB/s written).
 template <typename T, typename IO>
 __global__ void __launch_bounds__(kThreads) ack_hessian_kernel(const StructArgs a, int ppc, int split, FastDiv fd,
                                                                const AckConst nc)
@@ -575,7 +577,7 @@ int fp_points(int n, long long batch, int fmas)
     int best = most;
     double best_cost = 1e300;
     for (int p = std::min(most, (127 + n) / n); p <= most; ++p) {
-        const long long ctas = (batch + p - 1) / p, rounds = (ctas + 151) / 152;
+        const long long ctas = (batch + p - 1) / p, rounds = (ctas + kSms - 1) / kSms;
         const double cost = (double)rounds * (std::min<long long>(p, batch) * point + cta);
         if (cost <= best_cost) {
             best_cost = cost;
@@ -637,7 +639,7 @@ cudaError_t fp_hessian(const StructArgs &a, FastDiv fd, cudaStream_t s)
         // points per CTA: one 4 x 4 block per thread, at most 64 KiB of J
         const size_t per = (size_t)n * (np + 3) * sizeof(T);
         int ppc = std::max(1, std::min(kThreads / tiles, (int)(64 * 1024 / per)));
-        ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 303) / 304));
+        ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 2 * kSms - 1) / (2 * kSms)));
         const size_t bytes = align_up((size_t)n * (sizeof(Two<double>) + sizeof(Two<T>)), 16) + ppc * per;
         const long long blocks = (a.batch + ppc - 1) / ppc;
         if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
@@ -666,7 +668,7 @@ cudaError_t hessian(int fn, const StructArgs &a, cudaStream_t s)
     if (fn == FN_ROSENBROCK) {
         const long long total = a.batch * n;
         int rows = std::max(1, std::min(1024, kHessElems / n));
-        rows = (int)std::min<long long>(rows, std::max<long long>(8, total / 304));
+        rows = (int)std::min<long long>(rows, std::max<long long>(8, total / (2 * kSms)));
         const long long blocks = (total + rows - 1) / rows;
         if (blocks > kMaxBlocks) return cudaErrorInvalidConfiguration;
         const size_t bytes = (size_t)rows * (3 * sizeof(T) + sizeof(short));
@@ -675,7 +677,7 @@ cudaError_t hessian(int fn, const StructArgs &a, cudaStream_t s)
     }
     const int split = std::max(1, (n * n + kHessElems - 1) / kHessElems);
     int ppc = split > 1 ? 1 : std::max(1, std::min(512 / n, kHessElems / (n * n)));
-    ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 303) / 304));
+    ppc = (int)std::min<long long>(ppc, std::max<long long>(1, (a.batch + 2 * kSms - 1) / (2 * kSms)));
     const long long ctas = (a.batch + ppc - 1) / ppc;
     if (ctas > kMaxBlocks / split) return cudaErrorInvalidConfiguration;
     const size_t bytes = align_up((size_t)ppc * n * 5 * sizeof(T), 16) + ppc * (2 * sizeof(double) + 4 * sizeof(T)) +

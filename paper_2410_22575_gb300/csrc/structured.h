@@ -12,6 +12,9 @@
 namespace chessfad {
 
 constexpr int kMaxVars = 512;  // CHESSFAD_MAX_N
+// SMs of GB300, for the rules that share work out; plans are built on hosts
+// without a device too, so it is a constant.  Results are right for any count.
+constexpr int kSms = 152;
 
 struct StructArgs {
     const void *x;

@@ -6,6 +6,7 @@
 #include <algorithm>
 
 #include "structured.cuh"
+#include "structured.h"
 
 namespace chessfad {
 
@@ -36,7 +37,7 @@ inline int ack_lanes(int n, long long batch, bool f64)
     for (int g = 1; g <= 32; g <<= 1) {
         const int it = (n + g - 1) / g;
         if (it > 16 || (g > 1 && g >= 2 * n) || (!f64 && g < 8 && it > 1)) continue;
-        const double waves = std::max(1.0, (double)batch * g / (152.0 * 512.0));
+        const double waves = std::max(1.0, (double)batch * g / (kSms * 512.0));
         const double cost = (it + over) * waves;
         if (cost < best_cost) {
             best_cost = cost;
@@ -48,8 +49,13 @@ inline int ack_lanes(int n, long long batch, bool f64)
 
 // From this n on (at most 4 points per CTA) the rows of A and B are read from
 // L2 instead of through a shared-memory tile: the tile would hold a few rows
-// only, too few items for the CTA's warps between two barriers (4000 uneven
-// requests up to n = 512: 426 us with tiles, 270 so).
+// only, too few items for the CTA's warps between two barriers.  Time from L2
+// over time with tiles, FP64 / FP32-comp: H v of 1000 points, n = 64 1.55/1.62,
+// 96 1.21/1.49, 112 1.16/1.21, 127 1.00/0.91, 128 0.76/0.53, 160 0.77/0.49, 256
+// 0.68/0.51, 512 0.79/0.41; of 16 points, 96 1.07/1.12, 127 0.79/0.65, 160
+// 0.75/0.48; Hessians (curvature) between 0.97 and 1.16 up to n = 257, 0.98/0.73
+// at 512; 200 uneven requests of sizes about n, 112 1.13/1.33, 128 1.02/1.05, 160
+// 1.12/1.11, 200 0.97/1.10, 256 0.78/0.72, 512 0.74/0.44.
 constexpr int kFpWide = 128;
 
 // The shape of an FpTile: rows rows of A and B for P points, pairs pairs; f64:
