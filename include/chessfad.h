@@ -543,7 +543,8 @@ CHESSFAD_API int chessfad_user_fn_info(const chessfad_user_fn *fn, int hvp, int 
  * precision (double, or float for CHESSFAD_FP32_COMP): one evaluation of f
  * per chunk with d1 seeded by v (rows that are not finite, and points whose v
  * is not, by the plain method; a source written for the number type of the
- * methods by rows only, by the symmetric method).  Asynchronous on `stream`; allocates nothing.
+ * methods by rows only, by the symmetric method, and chessfad_user_fn_create's
+ * log says so).  Asynchronous on `stream`; allocates nothing.
  * The first symmetric launch on a device that needs more than 48 KiB of shared memory raises the
  * kernel's limit (a host call; make it before capturing a CUDA graph). */
 CHESSFAD_API int chessfad_user_hvp(chessfad_user_fn *fn, int n, long long batch, const void *x, const void *v,

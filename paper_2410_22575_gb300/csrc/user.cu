@@ -330,12 +330,14 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
     text += "\n#include \"user_kernel.cuh\"\n";
     // The row methods and the directional kernel as two programs: compiled side
     // by side they take about as long as the larger one.  A source that names the
-    // rows' number type Num<T, C> may compile for the row methods only.  The directional kernel's
-    // chunk size is not part of its result; in FP32 its numbers take two floats
-    // per component of d1 and h, and chunks larger than 8 spill (the extended-
-    // operator function at csize 16, n = 64, 4096 points: 337 us with chunks of
-    // 16, 143 with 8).
-    const int dir_csize = prec == CHESSFAD_FP32_COMP ? std::min(csize, 8) : csize;
+    // rows' number type Num<T, C> may compile for the row methods only.
+    // The directional kernel's chunk size is not part of its result.  In FP32 its
+    // numbers take two floats per component of d1 and h, and the components' sums
+    // cost more than f's values again for every chunk: chunks of 16 spill (337 us
+    // for the extended-operator function, n = 64, 4096 points), and of 8 and 4 take
+    // 203 and 145 us at n = 20 (40000 points), 130 and 130 at 64, 185 and 160 at
+    // 128 (512 points).
+    const int dir_csize = prec == CHESSFAD_FP32_COMP ? std::min(csize, 4) : csize;
     Program prog[2];
     std::thread second;
     try {
@@ -355,7 +357,11 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
         put_log(log, log_bytes, prog[0].log);
         return CHESSFAD_ERR_JIT;
     }
-    put_log(log, log_bytes, prog[0].log);
+    std::string messages = prog[0].log;
+    if (!prog[1].ok)
+        messages += "\nthe default H v is the symmetric method's: not compiled for one evaluation per chunk\n" +
+                    prog[1].log;
+    put_log(log, log_bytes, messages);
 
     auto *fn = new chessfad_user_fn;
     fn->csize = csize;
@@ -374,7 +380,7 @@ CHESSFAD_API int chessfad_user_fn_create(const char *source, const char *name, i
         e = cudaLibraryGetKernel(&fn->hessian_n1, fn->lib, "chessfad_user_hessian_n1");
     if (e != cudaSuccess) {
         cudaGetLastError();
-        put_log(log, log_bytes, std::string("compiled; loading failed: ") + cudaGetErrorString(e));
+        put_log(log, log_bytes, std::string("compiled; loading failed: ") + cudaGetErrorString(e) + "\n" + messages);
         if (fn->dir_lib) cudaLibraryUnload(fn->dir_lib);
         if (fn->lib) cudaLibraryUnload(fn->lib);
         delete fn;

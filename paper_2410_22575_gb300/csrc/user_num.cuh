@@ -99,6 +99,49 @@ struct Dir<float> {
     }
 };
 
+// Two of them, the operations packed (Dir<float>'s roundings: TwoProd's error is
+// formed with the sign reversed, a - b as the exact fma(-1, b, a)).
+struct Dir2 {
+    float2 s, e;
+    __device__ __forceinline__ static Dir2 both(const Dir<float> &d)
+    {
+        return Dir2{make_float2(d.s, d.s), make_float2(d.e, d.e)};
+    }
+    __device__ __forceinline__ static float2 sub(float2 a, float2 b)
+    {
+        return __ffma2_rn(make_float2(-1.f, -1.f), b, a);
+    }
+    __device__ __forceinline__ static void sum(float2 a, float2 b, float2 &s, float2 &t)
+    {
+        s = __fadd2_rn(a, b);
+        const float2 bb = sub(s, a);
+        t = __fadd2_rn(sub(a, sub(s, bb)), sub(b, bb));
+    }
+    __device__ __forceinline__ Dir2 operator+(const Dir2 &b) const
+    {
+        Dir2 r;
+        float2 t;
+        sum(s, b.s, r.s, t);
+        r.e = __fadd2_rn(__fadd2_rn(e, b.e), t);
+        return r;
+    }
+    __device__ __forceinline__ Dir2 operator*(float2 x) const
+    {
+        const float2 m = make_float2(-x.x, -x.y), p = __fmul2_rn(x, s), q = __ffma2_rn(m, s, p);
+        return Dir2{p, __ffma2_rn(x, e, make_float2(-q.x, -q.y))};
+    }
+    __device__ __forceinline__ Dir2 fma(float2 x, const Dir2 &acc) const
+    {
+        const float2 m = make_float2(-x.x, -x.y), p = __fmul2_rn(x, s);
+        const float2 q = __ffma2_rn(m, e, __ffma2_rn(m, s, p));
+        Dir2 r;
+        float2 t;
+        sum(acc.s, p, r.s, t);
+        r.e = __fadd2_rn(acc.e, sub(t, q));
+        return r;
+    }
+};
+
 // The components of a number of the directional evaluation: as HD, with d1 and
 // h along v.
 template <typename T, int C>
@@ -108,6 +151,49 @@ struct HDir {
     T g[C];
     Dir<T> h[C];
 };
+
+// f(l, ...) for every component l of h: f takes its arguments for one component,
+// or in FP32 with an even C for two neighbours at a time.  at(): components l,
+// l + 1 of h or g; all(): a scalar's or a derivative's value for both.
+template <typename T>
+struct One {
+    template <int C>
+    __device__ __forceinline__ static Dir<T> at(const Dir<T> (&h)[C], int l) { return h[l]; }
+    template <int C>
+    __device__ __forceinline__ static T at(const T (&g)[C], int l) { return g[l]; }
+    __device__ __forceinline__ static T all(T x) { return x; }
+    __device__ __forceinline__ static Dir<T> all(const Dir<T> &d) { return d; }
+    template <int C>
+    __device__ __forceinline__ static void put(Dir<T> (&h)[C], int l, const Dir<T> &d) { h[l] = d; }
+};
+struct Pair {
+    template <int C>
+    __device__ __forceinline__ static Dir2 at(const Dir<float> (&h)[C], int l)
+    {
+        return Dir2{make_float2(h[l].s, h[l + 1].s), make_float2(h[l].e, h[l + 1].e)};
+    }
+    template <int C>
+    __device__ __forceinline__ static float2 at(const float (&g)[C], int l) { return make_float2(g[l], g[l + 1]); }
+    __device__ __forceinline__ static float2 all(float x) { return make_float2(x, x); }
+    __device__ __forceinline__ static Dir2 all(const Dir<float> &d) { return Dir2::both(d); }
+    template <int C>
+    __device__ __forceinline__ static void put(Dir<float> (&h)[C], int l, const Dir2 &d)
+    {
+        h[l] = Dir<float>{d.s.x, d.e.x};
+        h[l + 1] = Dir<float>{d.s.y, d.e.y};
+    }
+};
+template <typename T, int C, typename F>
+__device__ __forceinline__ void components(Dir<T> (&h)[C], F &&f)
+{
+    if constexpr (sizeof(T) == 4 && C % 2 == 0) {
+#pragma unroll
+        for (int l = 0; l < C; l += 2) Pair::put(h, l, f(Pair(), l));
+    } else {
+#pragma unroll
+        for (int l = 0; l < C; ++l) One<T>::put(h, l, f(One<T>(), l));
+    }
+}
 
 // A: whether the number is one of the directional evaluation, which tracks
 // activity.  In one evaluation a variable outside the chunk has zero g and h
@@ -175,11 +261,15 @@ __device__ __forceinline__ Num<T, C, A> operator+(const Num<T, C, A> &u, const N
         r.a.v = u.a.v + w.a.v;
         r.a.d1 = u.a.d1 + w.a.d1;
         if (w.act) {
-            if (u.act) vadd(u.a.g, w.a.g, r.a.g);
+            if (u.act) {
+                vadd(u.a.g, w.a.g, r.a.g);
+                components(r.a.h, [&](auto k, int l) { return k.at(u.a.h, l) + k.at(w.a.h, l); });
+            } else {
 #pragma unroll
-            for (int l = 0; l < C; ++l) {
-                if (!u.act) r.a.g[l] = w.a.g[l];
-                r.a.h[l] = u.act ? u.a.h[l] + w.a.h[l] : w.a.h[l];
+                for (int l = 0; l < C; ++l) {
+                    r.a.g[l] = w.a.g[l];
+                    r.a.h[l] = w.a.h[l];
+                }
             }
             r.act = true;
         }
@@ -192,17 +282,8 @@ __device__ __forceinline__ Num<T, C, A> operator-(const Num<T, C, A> &u, const N
     if constexpr (!A) {
         return Num<T, C, A>(hsub(u.a, w.a));
     } else {
-        Num<T, C, A> r = u;
+        Num<T, C, A> r = u + (-w);
         r.a.v = u.a.v - w.a.v;
-        r.a.d1 = u.a.d1 - w.a.d1;
-        if (w.act) {
-#pragma unroll
-            for (int l = 0; l < C; ++l) {
-                r.a.g[l] = u.act ? u.a.g[l] - w.a.g[l] : -w.a.g[l];
-                r.a.h[l] = u.act ? u.a.h[l] - w.a.h[l] : -w.a.h[l];
-            }
-            r.act = true;
-        }
         return r;
     }
 }
@@ -211,8 +292,7 @@ template <typename T, int C>
 __device__ __forceinline__ void hmul_by(const HDir<T, C> &u, const HDir<T, C> &w, HDir<T, C> &r)
 {
     vmul(w.v, u.g, r.g);
-#pragma unroll
-    for (int l = 0; l < C; ++l) r.h[l] = u.h[l].fma(w.v, w.d1 * u.g[l]);
+    components(r.h, [&](auto k, int l) { return k.at(u.h, l).fma(k.all(w.v), k.all(w.d1) * k.at(u.g, l)); });
 }
 template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, const Num<T, C, A> &w)
@@ -224,13 +304,12 @@ __device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, const N
         if (u.act && w.act) {
             vmul(u.a.v, w.a.g, r.a.g);
             vfma(w.a.v, u.a.g, r.a.g);
-#pragma unroll
-            for (int l = 0; l < C; ++l) {
-                Dir<T> h = w.a.h[l] * u.a.v;
-                h = u.a.d1.fma(w.a.g[l], h);
-                h = w.a.d1.fma(u.a.g[l], h);
-                r.a.h[l] = u.a.h[l].fma(w.a.v, h);
-            }
+            components(r.a.h, [&](auto k, int l) {
+                auto h = k.at(w.a.h, l) * k.all(u.a.v);
+                h = k.all(u.a.d1).fma(k.at(w.a.g, l), h);
+                h = k.all(w.a.d1).fma(k.at(u.a.g, l), h);
+                return k.at(u.a.h, l).fma(k.all(w.a.v), h);
+            });
         } else if (u.act) {
             hmul_by(u.a, w.a, r.a);
         } else if (w.act) {
@@ -288,8 +367,7 @@ __device__ __forceinline__ Num<T, C, A> operator*(const Num<T, C, A> &u, double 
         r.a.d1 = u.a.d1 * T(s);
         if (u.act) {
             vmul(T(s), u.a.g, r.a.g);
-#pragma unroll
-            for (int l = 0; l < C; ++l) r.a.h[l] = u.a.h[l] * T(s);
+            components(r.a.h, [&](auto k, int l) { return k.at(u.a.h, l) * k.all(T(s)); });
         }
         return r;
     }
@@ -310,8 +388,8 @@ __device__ __forceinline__ Num<T, C, A> apply(const Num<T, C, A> &u, T phi, T d1
         if (u.act) {
             const Dir<T> q = u.a.d1 * d2;
             vmul(d1, u.a.g, r.a.g);
-#pragma unroll
-            for (int l = 0; l < C; ++l) r.a.h[l] = q.fma(u.a.g[l], u.a.h[l] * d1);
+            components(r.a.h,
+                       [&](auto k, int l) { return k.all(q).fma(k.at(u.a.g, l), k.at(u.a.h, l) * k.all(d1)); });
         } else {
             r.a.d1.s = fma_(d2, T(0), r.a.d1.s);
         }
