@@ -24,7 +24,7 @@ namespace {
 constexpr int kThreads = kFpThreads;
 
 // 4000 requests, n log-uniform in 2 .. 512, compensated FP32: dense 308 ms, here
-// 0.257 ms.  The FP64 FMAs of the residuals, nearly all of them in the
+// 0.258 ms.  The FP64 FMAs of the residuals, nearly all of them in the
 // Fletcher-Powell requests of n >= 128, need 0.106 ms; the rest is the latency
 // of the large requests' parts (one part alone takes 55 us, 16 of them FP64).
 

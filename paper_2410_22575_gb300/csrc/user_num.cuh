@@ -477,10 +477,11 @@ template <typename T, int C, bool A>
 __device__ __forceinline__ Num<T, C, A> pow(const Num<T, C, A> &u, double p)
 {
     // Three powers, so that each has pow()'s own accuracy (u^0 is 1 and the
-    // derivative of u^1 is 1).  A number outside the chunk uses phi'' only to notice that it is
-    // not finite; where u^(p-2) = u^(p-1) / u and its factor are far inside the
-    // range, that power is left out (the extended-operator test function, FP64,
-    // n = 64, 4096 points: 1.67 ms with three powers everywhere, 1.30 so).
+    // derivative of u^1 is 1).  A number outside the chunk uses phi'' only to
+    // notice that it is not finite; where u^(p-2) = u^(p-1) / u and its factor
+    // are far inside the range, that power is left out (the extended-operator
+    // test function, FP64, n = 64, 4096 points: 1.67 ms with three powers
+    // everywhere, 1.30 so).
     const T q = T(p), x = u.a.v, big = sizeof(T) == 8 ? T(1e75) : T(1e9);
     const T w0 = m_pow(x, q), w1 = m_pow(x, q - T(1));
     bool needed = !(x > T(1) / big && x < big && w1 < big && q < big && q > -big);
